@@ -11,34 +11,26 @@
 //   apply:  x' = M x for each row (bergson_precondition_rows, same GEMM as
 //           the on-the-fly scores).
 //
-// All products are "NT" GEMMs C = alpha A B^T + beta C + gamma I with A and B
-// row-major and the reduction index contiguous, run by the tcgen05 skinny
-// product of onthefly.cu (3xTF32: fp32 accuracy from tf32 tensor-core MMAs)
-// with 128-row tiles on both sides.  Products of the iteration are
-// symmetric in exact arithmetic, so B^T = B there; each update is
-// re-symmetrised so that rounding cannot build up an antisymmetric part.
+// All products are "NT" (C = A B^T, the reduction index contiguous in both
+// operands) on the pair kernel of square.cu, whose operands are fp16 hi + lo
+// planes with per-row scales: every matrix of the iteration is split once, by
+// the pass that also symmetrises or transposes it, and the product itself
+// takes the row and column maxima that pass scales by.  Products of the
+// iteration are symmetric in exact arithmetic; each update is re-symmetrised
+// so that rounding cannot build up an antisymmetric part.
+//
+// Measured (K = 3072, n = 1024, 12 updates, one GB300): 17.4 ms per fit and
+// power with tf32 parts on single CTAs, K slices through partial sums in
+// memory and separate transpose / symmetrise / norm passes; 5.55 ms as here (a product 119 us in ncu, its MMAs 76).
+
+#include <algorithm>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace bergson {
 
 namespace {
-
-// xt[k, i] = x[i, k] for i < n, zero for n <= i < n_pad.
-__global__ void transpose_kernel(const float* __restrict__ x, int n, int K, int64_t ldx,
-                                 float* __restrict__ xt, int n_pad) {
-  __shared__ float tile[32][33];
-  const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int i = i0 + r, k = k0 + threadIdx.x;
-    tile[r][threadIdx.x] = (i < n && k < K) ? x[i * ldx + k] : 0.0f;
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int k = k0 + r, i = i0 + threadIdx.x;
-    if (k < K && i < n_pad) xt[k * static_cast<int64_t>(n_pad) + i] = tile[threadIdx.x][r];
-  }
-}
 
 // scal[0] = sum_i (lam * R1[i,i] + (1 - lam) * R2[i,i])  (single CTA)
 __global__ void mixed_trace_kernel(const float* __restrict__ r1, const float* __restrict__ r2,
@@ -60,62 +52,97 @@ __global__ void mixed_trace_kernel(const float* __restrict__ r1, const float* __
   }
 }
 
-// out = lam R1 + (1 - lam) R2 + damping * trace / K * I   (R2 may be null: out = R1 + ...)
-__global__ void mix_kernel(const float* __restrict__ r1, const float* __restrict__ r2, int64_t ld,
-                           int K, float lam, float damping, const float* __restrict__ scal,
-                           float* __restrict__ out, int64_t ldo) {
+// Row i of out = lam R1 + (1 - lam) R2 + damping * trace / K * I (R2 may be
+// null: R1 + ...), its largest |entry| (float bits) and its compensated sum of
+// squares.  One CTA per row (grid stride).
+__global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
+                                                  const float* __restrict__ r2, int64_t ld, int K,
+                                                  float lam, float damping,
+                                                  const float* __restrict__ scal,
+                                                  float* __restrict__ out,
+                                                  uint32_t* __restrict__ rmax,
+                                                  float* __restrict__ part) {
+  __shared__ float red_s[8];
+  __shared__ uint32_t red_m[8];
   const float d = damping * scal[0] / static_cast<float>(K);
-  const int64_t n = static_cast<int64_t>(K) * K;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(e / K), j = static_cast<int>(e % K);
-    float v = r1[i * ld + j];
-    if (r2 != nullptr) v = lam * v + (1.0f - lam) * r2[i * ld + j];
-    if (i == j) v += d;
-    out[i * ldo + j] = v;
-  }
-}
-
-constexpr int kFrobBlocks = 512;
-
-// part[blockIdx] = compensated sum of squares of (R - shift I) over a
-// grid-stride slice of R.
-__global__ void frob_partial_kernel(const float* __restrict__ r, int64_t ld, int K, float shift,
-                                    float* __restrict__ part) {
-  __shared__ float red[32];
-  float s = 0.0f, comp = 0.0f;
-  const int64_t n = static_cast<int64_t>(K) * K;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t i = e / K, j = e % K;
-    const float x = r[i * ld + j] - (i == j ? shift : 0.0f);
-    const float y = x * x - comp;
-    const float t = s + y;
-    comp = (t - s) - y;
-    s = t;
-  }
+  for (int i = blockIdx.x; i < K; i += gridDim.x) {
+    const float4* a = reinterpret_cast<const float4*>(r1 + static_cast<int64_t>(i) * ld);
+    const float4* b =
+        r2 != nullptr ? reinterpret_cast<const float4*>(r2 + static_cast<int64_t>(i) * ld) : nullptr;
+    float4* o = reinterpret_cast<float4*>(out + static_cast<int64_t>(i) * K);
+    float s = 0.0f, comp = 0.0f;
+    uint32_t m = 0u;
+    for (int j = threadIdx.x; j < K / 4; j += 256) {
+      float4 v = a[j];
+      if (b != nullptr) {
+        const float4 w = b[j];
+        v.x = lam * v.x + (1.0f - lam) * w.x;
+        v.y = lam * v.y + (1.0f - lam) * w.y;
+        v.z = lam * v.z + (1.0f - lam) * w.z;
+        v.w = lam * v.w + (1.0f - lam) * w.w;
+      }
+      if (j == i / 4) {
+        if ((i & 3) == 0) v.x += d;
+        if ((i & 3) == 1) v.y += d;
+        if ((i & 3) == 2) v.z += d;
+        if ((i & 3) == 3) v.w += d;
+      }
+      o[j] = v;
+      m = max(max(m, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
+              max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+      const float y = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w - comp;
+      const float t = s + y;
+      comp = (t - s) - y;
+      s = t;
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.0f;
-    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t += red[w];
-    part[blockIdx.x] = t;
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+    m = __reduce_max_sync(0xffffffffu, m);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+      red_s[threadIdx.x >> 5] = s;
+      red_m[threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float t = 0.0f;
+      uint32_t mm = 0u;
+      for (int w = 0; w < 8; ++w) {
+        t += red_s[w];
+        mm = max(mm, red_m[w]);
+      }
+      part[i] = t;
+      rmax[i] = mm;
+    }
   }
 }
 
-// scal[1] = ||R||_F, scal[2] = 1/c, scal[3] = 1/sqrt(c), scal[4] = 1/c  (fixed-order sum)
-__global__ void frob_final_kernel(const float* __restrict__ part, int n_part,
-                                  float* __restrict__ scal) {
-  if (threadIdx.x != 0) return;
+// Fixed-order sum of part[0, n): compensated per thread, then a tree over the
+// threads of the single CTA.  Returned to thread 0.
+__device__ __forceinline__ float ordered_sum(const float* __restrict__ part, int n) {
+  __shared__ float red[32];
   float t = 0.0f, comp = 0.0f;
-  for (int i = 0; i < n_part; ++i) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const float y = part[i] - comp;
     const float u = t + y;
     comp = (u - t) - y;
     t = u;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  float s = 0.0f;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) s += red[w];
+  return s;
+}
+
+// scal[1] = ||R||_F = c, scal[2] = 1/c, scal[3] = 1/sqrt(c), scal[4] = 1/c
+__global__ void __launch_bounds__(1024) frob_final_kernel(const float* __restrict__ part,
+                                                          int n_part, float* __restrict__ scal) {
+  const float t = ordered_sum(part, n_part);
+  if (threadIdx.x != 0) return;
   const float c = sqrtf(t);
   scal[1] = c;
   scal[2] = 1.0f / c;
@@ -123,192 +150,232 @@ __global__ void frob_final_kernel(const float* __restrict__ part, int n_part,
   scal[4] = 1.0f / c;
 }
 
-// *out = scale * sqrt(fixed-order compensated sum of part[0, n_part))
-__global__ void frob_norm_kernel(const float* __restrict__ part, int n_part, float scale,
-                                 float* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  float t = 0.0f, comp = 0.0f;
-  for (int i = 0; i < n_part; ++i) {
-    const float y = part[i] - comp;
-    const float u = t + y;
-    comp = (u - t) - y;
-    t = u;
-  }
-  *out = scale * sqrtf(t);
+// *out = scale * sqrt(sum of part[0, n_part))
+__global__ void __launch_bounds__(1024) frob_norm_kernel(const float* __restrict__ part, int n_part,
+                                                         float scale, float* __restrict__ out) {
+  griddep_launch_dependents();
+  griddep_wait();
+  const float t = ordered_sum(part, n_part);
+  if (threadIdx.x == 0) *out = scale * sqrtf(t);
 }
 
-// y = r * scal[2] (R / c); z = I
-__global__ void ns_init_kernel(const float* __restrict__ r, int64_t ld, int K,
-                               const float* __restrict__ scal, float* __restrict__ y,
-                               float* __restrict__ z) {
+// The first iterate without products: Y0 = R / c (in place in y), its row
+// maxima rescaled the same way, and t = T0^T = 1.5 I - 0.5 Y0 (Z0 = I) with its
+// row and column maxima (cleared before) and, per tile, the sum of
+// (T0 - I)^2.  64 x 64 tiles.
+__global__ void __launch_bounds__(256) ns_first_kernel(float* __restrict__ y, int K,
+                                                       const float* __restrict__ scal,
+                                                       uint32_t* __restrict__ ymax,
+                                                       float* __restrict__ t,
+                                                       uint32_t* __restrict__ rmax,
+                                                       uint32_t* __restrict__ cmax,
+                                                       float* __restrict__ part) {
+  __shared__ uint32_t scol[64];
+  __shared__ float red[8];
+  griddep_launch_dependents();
+  griddep_wait();
   const float inv_c = scal[2];
-  const int64_t n = static_cast<int64_t>(K) * K;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(e / K), j = static_cast<int>(e % K);
-    y[e] = r[i * ld + j] * inv_c;
-    z[e] = i == j ? 1.0f : 0.0f;
-  }
-}
-
-// x <- (x + x^T) / 2 in place.  The iterates are symmetric in exact
-// arithmetic, but the products use B^T = B, which turns the rounding's
-// antisymmetric part into a growing error unless it is removed.  One CTA per
-// pair of 32 x 32 tiles (ti <= tj): both tiles are read row by row into shared
-// memory and written back row by row, so every global access is coalesced.
-__global__ void __launch_bounds__(256) symmetrize_kernel(float* __restrict__ x, int K) {
-  __shared__ float a[32][33], b[32][33];
-  const int ti = blockIdx.y, tj = blockIdx.x;
-  if (ti > tj) return;
-  const int i0 = ti * 32, j0 = tj * 32, c = threadIdx.x;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    a[r][c] = (i0 + r < K && j0 + c < K) ? x[static_cast<int64_t>(i0 + r) * K + j0 + c] : 0.0f;
-    b[r][c] = (j0 + r < K && i0 + c < K) ? x[static_cast<int64_t>(j0 + r) * K + i0 + c] : 0.0f;
-  }
+  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x < 64) scol[threadIdx.x] = 0u;
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    if (i0 + r < K && j0 + c < K)
-      x[static_cast<int64_t>(i0 + r) * K + j0 + c] = 0.5f * (a[r][c] + b[c][r]);
-    if (ti != tj && j0 + r < K && i0 + c < K)
-      x[static_cast<int64_t>(j0 + r) * K + i0 + c] = 0.5f * (b[r][c] + a[c][r]);
+  float s = 0.0f;
+  float v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i = i0 + w + 8 * (k >> 1), j = j0 + lane + 32 * (k & 1);
+    v[k] = (i < K && j < K) ? y[static_cast<int64_t>(i) * K + j] * inv_c : 0.0f;
   }
-}
-
-// x <- x^T in place (K x K, leading dimension K).  One CTA per pair of 32 x 32
-// tiles (ti <= tj), both read row by row into shared memory and written back
-// swapped, so every global access is coalesced.
-__global__ void __launch_bounds__(256) transpose_inplace_kernel(float* __restrict__ x, int K) {
-  __shared__ float a[32][33], b[32][33];
-  const int ti = blockIdx.y, tj = blockIdx.x;
-  if (ti > tj) return;
-  const int i0 = ti * 32, j0 = tj * 32, c = threadIdx.x;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    a[r][c] = (i0 + r < K && j0 + c < K) ? x[static_cast<int64_t>(i0 + r) * K + j0 + c] : 0.0f;
-    b[r][c] = (j0 + r < K && i0 + c < K) ? x[static_cast<int64_t>(j0 + r) * K + i0 + c] : 0.0f;
+  uint32_t cm[2] = {0u, 0u};
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int i = i0 + w + 8 * r;
+    uint32_t m = 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = j0 + lane + 32 * h;
+      if (i < K && j < K) {
+        const int64_t e = static_cast<int64_t>(i) * K + j;
+        y[e] = v[2 * r + h];
+        const float u = (i == j ? 1.5f : 0.0f) - 0.5f * v[2 * r + h];
+        t[e] = u;
+        const float d = u - (i == j ? 1.0f : 0.0f);
+        s += d * d;
+        const uint32_t b = __float_as_uint(u) & 0x7fffffffu;
+        m = max(m, b);
+        cm[h] = max(cm[h], b);
+      }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0 && i < K) {
+      atomicMax(&rmax[i], m);
+      if (j0 == 0) ymax[i] = __float_as_uint(__uint_as_float(ymax[i]) * inv_c);
+    }
   }
+  atomicMax(&scol[lane], cm[0]);
+  atomicMax(&scol[lane + 32], cm[1]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) red[w] = s;
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    if (i0 + r < K && j0 + c < K) x[static_cast<int64_t>(i0 + r) * K + j0 + c] = b[c][r];
-    if (ti != tj && j0 + r < K && i0 + c < K)
-      x[static_cast<int64_t>(j0 + r) * K + i0 + c] = a[c][r];
+  if (threadIdx.x < 64 && j0 + threadIdx.x < K) atomicMax(&cmax[j0 + threadIdx.x], scol[threadIdx.x]);
+  if (threadIdx.x == 0) {
+    float a = 0.0f;
+    for (int x = 0; x < 8; ++x) a += red[x];
+    part[blockIdx.y * gridDim.x + blockIdx.x] = a;
   }
 }
 
-// dst[i, j] = src[i * K + j] * (*scale)
-__global__ void scale_copy_kernel(const float* __restrict__ src, int K,
-                                  const float* __restrict__ scale, float* __restrict__ dst,
-                                  int64_t ldd) {
+// m = *scale * I
+__global__ void scaled_identity_kernel(int K, const float* __restrict__ scale,
+                                       float* __restrict__ m, int64_t ldm) {
   const float sc = *scale;
-  const int64_t n = static_cast<int64_t>(K) * K;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    dst[(e / K) * ldd + e % K] = src[e] * sc;
-}
-
-// C[m, n] = alpha' sum_k A[m, k] B[n, k] + beta C[m, n] + gamma [m == n] for
-// M x K A and N x K B (alpha' = alpha * (*alpha_s) when alpha_s is given);
-// `ws` holds xgemm_plan(M, N, K).
-cudaError_t gemm_nt(const float* A, int64_t lda, const float* B, int64_t ldb, float* C,
-                    int64_t ldc, int M, int N, int K, float alpha, float beta, float gamma,
-                    const float* alpha_s, uint8_t* ws, int* status, int sms, cudaStream_t s) {
-  XGemmArgs a;
-  a.x = A;
-  a.ldx = lda;
-  a.y = B;
-  a.ldy = ldb;
-  a.B = M;
-  a.Q = N;
-  a.K = K;
-  a.unit = 0;
-  a.alpha = alpha;
-  a.alpha_s = alpha_s;
-  a.beta = beta;
-  a.gamma = gamma;
-  a.scores = C;
-  a.ld_scores = ldc;
-  a.ws = ws;
-  a.status = status;
-  a.timeout_ns = kWaitTimeoutNs;
-  return xgemm_run(a, sms, s);
+  for (int i = blockIdx.x; i < K; i += gridDim.x)
+    for (int j = threadIdx.x; j < K; j += blockDim.x)
+      m[static_cast<int64_t>(i) * ldm + j] = i == j ? sc : 0.0f;
 }
 
 size_t round_up256(size_t x) { return (x + 255) / 256 * 256; }
 
-unsigned elementwise_blocks(int64_t n) {
-  const int64_t b = (n + 255) / 256;
-  return static_cast<unsigned>(b < 8192 ? b : 8192);
+int64_t split_ld(int64_t K) { return (K + 7) / 8 * 8; }
+
+// Carves a split operand of `rows` rows of K entries out of ws at *off.
+size_t split_bytes(int64_t rows, int64_t K) {
+  return round_up256(2 * static_cast<size_t>(rows) * split_ld(K) * sizeof(__half)) +
+         round_up256(static_cast<size_t>(rows) * sizeof(int));
+}
+SplitOperand take_split(uint8_t* ws, size_t* off, int rows, int K) {
+  SplitOperand o;
+  o.rows = rows;
+  o.K = K;
+  o.ld = split_ld(K);
+  o.planes = reinterpret_cast<__half*>(ws + *off);
+  o.exps = reinterpret_cast<int*>(
+      ws + *off + round_up256(2 * static_cast<size_t>(rows) * o.ld * sizeof(__half)));
+  *off += split_bytes(rows, K);
+  return o;
+}
+
+constexpr int kMaxSlots = 4;   // row / column maxima of the products in flight (see launch_fisher_power)
+
+size_t part_floats(int64_t K) {
+  const int64_t t = (K + 63) / 64;
+  return static_cast<size_t>(std::max<int64_t>(
+      K, std::max<int64_t>(t * t, square_part_floats(static_cast<int>(K), static_cast<int>(K)))));
 }
 
 }  // namespace
 
 size_t fisher_fit_workspace(int64_t n, int64_t K) {
-  const int64_t n_pad = (n + 3) / 4 * 4;
-  return round_up256(static_cast<size_t>(K) * n_pad * sizeof(float)) +
-         xgemm_plan(K, K, n_pad).total;
+  return split_bytes(K, n) + round_up256(static_cast<size_t>(K) * sizeof(uint32_t));
 }
 
 cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* r, int64_t ldr,
                               float* ws, int* status, int sms, cudaStream_t s) {
-  const int n_pad = (n + 3) / 4 * 4;
-  dim3 grid((n_pad + 31) / 32, (K + 31) / 32);
-  transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(x, n, K, ldx, ws, n_pad);
-  cudaError_t e = cudaGetLastError();
+  uint8_t* base = reinterpret_cast<uint8_t*>(ws);
+  size_t off = 0;
+  const SplitOperand xt = take_split(base, &off, K, n);
+  uint32_t* cmax = reinterpret_cast<uint32_t*>(base + off);
+  const cudaError_t e = launch_transpose_split(x, n, K, ldx, cmax, xt, s);
   if (e != cudaSuccess) return e;
-  uint8_t* gws = reinterpret_cast<uint8_t*>(ws) +
-                 round_up256(static_cast<size_t>(K) * n_pad * sizeof(float));
-  return gemm_nt(ws, n_pad, ws, n_pad, r, ldr, K, K, n_pad, 1.0f / static_cast<float>(n), 0.0f,
-                 0.0f, nullptr, gws, status, sms, s);
+  SquareArgs a;
+  a.x = xt;
+  a.y = xt;
+  a.symmetric = true;
+  a.alpha = 1.0f / static_cast<float>(n);
+  a.c = r;
+  a.ldc = ldr;
+  a.status = status;
+  return launch_square(a, sms, s);
 }
 
 size_t fisher_power_workspace(int64_t K) {
-  return round_up256((4 * static_cast<size_t>(K) * K + 64 + kFrobBlocks) * sizeof(float)) +
-         xgemm_plan(K, K, K).total;
+  const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
+  return 2 * kk + 4 * split_bytes(K, K) +
+         round_up256((2 * kMaxSlots + 1) * static_cast<size_t>(K) * sizeof(uint32_t)) +
+         round_up256(part_floats(K) * sizeof(float)) + 256;
 }
 
 cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t ldr, float lam,
                                 float damping, int inverse, int iterations, float tol,
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
                                 float* ws, int* status, int sms, cudaStream_t s) {
-  const int64_t kk = static_cast<int64_t>(K) * K;
-  uint8_t* gws = reinterpret_cast<uint8_t*>(ws) +
-                 round_up256((4 * static_cast<size_t>(K) * K + 64 + kFrobBlocks) * sizeof(float));
-  float* a = ws;            // mixed, damped R
-  float* y = a + kk;
-  float* z = y + kk;
-  float* t = z + kk;
-  float* scal = t + kk;     // trace, ||R||_F, 1/c, 1/sqrt(c), 1/c, residual;
-                            // [64, 64 + 512): partial sums
+  // Two fp32 matrices (the last Z product; the Y product, then T) and the
+  // splits of Z, Y, T and T^T.
+  uint8_t* base = reinterpret_cast<uint8_t*>(ws);
+  const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
+  float* yt = reinterpret_cast<float*>(base);          // Y product, then T
+  float* zf = reinterpret_cast<float*>(base + kk);     // Z product
+  size_t off = 2 * kk;
+  const SplitOperand zs = take_split(base, &off, K, K);
+  const SplitOperand ys = take_split(base, &off, K, K);
+  const SplitOperand ts = take_split(base, &off, K, K);
+  const SplitOperand tts = take_split(base, &off, K, K);
+  // Maxima: slot i holds a product's row maxima, then its column maxima.  Each
+  // product clears the slot of the next one, whose last reader (a pass three
+  // products back) has ended by then.
+  uint32_t* maxima = reinterpret_cast<uint32_t*>(base + off);
+  uint32_t* ymax = maxima + 2 * static_cast<int64_t>(kMaxSlots) * K;
+  const size_t max_bytes = (2 * kMaxSlots + 1) * static_cast<size_t>(K) * sizeof(uint32_t);
+  off += round_up256(max_bytes);
+  float* part = reinterpret_cast<float*>(base + off);
+  off += round_up256(part_floats(K) * sizeof(float));
+  float* scal = reinterpret_cast<float*>(base + off);  // trace, c, 1/c, 1/sqrt(c), 1/c, residual
+  int slot = 0;
+  auto rows_of = [&](int i) { return maxima + 2 * static_cast<int64_t>(i % kMaxSlots) * K; };
+  auto product = [&](const SplitOperand& x, const SplitOperand& y, float alpha, float gamma,
+                     float* c, float* sums) {
+    SquareArgs a;
+    a.x = x;
+    a.y = y;
+    a.alpha = alpha;
+    a.gamma = gamma;
+    a.c = c;
+    a.ldc = K;
+    a.row_max = rows_of(slot);
+    a.col_max = rows_of(slot) + K;
+    a.zero_next = rows_of(slot + 1);
+    a.part = sums;
+    a.status = status;
+    ++slot;
+    return launch_square(a, sms, s);
+  };
   const bool track = residuals != nullptr || tol > 0.0f;
   if (iterations_done != nullptr) *iterations_done = 0;
-  mixed_trace_kernel<<<1, 1024, 0, s>>>(r1, r2, ldr, K, lam, scal);
-  mix_kernel<<<elementwise_blocks(kk), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, a, K);
-  frob_partial_kernel<<<kFrobBlocks, 256, 0, s>>>(a, K, K, 0.0f, scal + 64);
-  frob_final_kernel<<<1, 32, 0, s>>>(scal + 64, kFrobBlocks, scal);
-  ns_init_kernel<<<elementwise_blocks(kk), 256, 0, s>>>(a, K, K, scal, y, z);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaMemsetAsync(maxima, 0, max_bytes, s);
   if (e != cudaSuccess) return e;
-  const dim3 tiles((K + 31) / 32, (K + 31) / 32);
+  mixed_trace_kernel<<<1, 1024, 0, s>>>(r1, r2, ldr, K, lam, scal);
+  mix_kernel<<<std::min(K, 4096), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, yt, ymax, part);
+  frob_final_kernel<<<1, 1024, 0, s>>>(part, K, scal);
+  const int t64 = (K + 63) / 64;
+  ns_first_kernel<<<dim3(t64, t64), 256, 0, s>>>(yt, K, scal, ymax, zf, rows_of(0), rows_of(0) + K,
+                                                 part);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  ++slot;
+  bool identity = true;          // Z is still I
+  const int n_part = square_part_count(K, K, sms);
   for (int it = 0;; ++it) {
     if (!track && it == iterations) break;
     // T = 1.5 I - 0.5 Z Y;  Z <- T Z;  Y <- Y T.
     // Z Y is not symmetric in floating point, so T != T^T: the Y update must
     // use T itself.  The products are NT (C = A B^T), so T Z = nt(T, Z) (Z is
-    // symmetric) and Y T = nt(Y, T^T): T is transposed in place between them.
+    // symmetric) and Y T = nt(Y, T^T): T is split both ways.
     // (Taking Y T^T instead is unstable: to first order, a symmetric
     // perturbation of the iterates along eigenvectors i, j of R grows by
     // (rho - 1) / 2 per step, rho = (s_i / s_j + s_j / s_i) / 2 with s the
     // eigenvalues of R^1/2, so once R's condition number exceeds ~34
     // (s_i / s_j > 3 + sqrt(8)) the converged iterates drift away again.
     // With Y T the same perturbation maps to a fixed point: stable.)
-    if ((e = gemm_nt(z, K, y, K, t, K, K, K, K, -0.5f, 0.0f, 1.5f, nullptr, gws, status, sms,
-                     s)) != cudaSuccess)
+    const int t_slot = it == 0 ? 0 : slot;
+    if (it > 0 && (e = product(zs, ys, -0.5f, 1.5f, yt, track ? part : nullptr)) != cudaSuccess)
       return e;
     if (track) {
       // ||I - Z Y||_F / sqrt(K) = 2 ||T - I||_F / sqrt(K): the current iterate's
       // residual (Z Y = Z (R/c) Z = M R M while the iteration keeps Y = (R/c) Z).
-      frob_partial_kernel<<<kFrobBlocks, 256, 0, s>>>(t, K, K, 1.0f, scal + 64);
-      frob_norm_kernel<<<1, 32, 0, s>>>(scal + 64, kFrobBlocks,
-                                        2.0f / sqrtf(static_cast<float>(K)), scal + 5);
+      e = launch_dependent(frob_norm_kernel, dim3(1), dim3(1024), 0, s,
+                           static_cast<const float*>(part), it == 0 ? t64 * t64 : n_part,
+                           2.0f / sqrtf(static_cast<float>(K)), scal + 5);
+      if (e != cudaSuccess) return e;
       float res = 0.0f;
       if ((e = cudaMemcpyAsync(&res, scal + 5, sizeof(float), cudaMemcpyDeviceToHost, s)) !=
               cudaSuccess ||
@@ -318,26 +385,47 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
       if (res <= tol) break;
     }
     if (it == iterations) break;
-    if ((e = gemm_nt(t, K, z, K, a, K, K, K, K, 1.0f, 0.0f, 0.0f, nullptr, gws, status, sms,
-                     s)) != cudaSuccess)            // a = T Z (new Z)
+    const uint32_t* tmax = rows_of(t_slot);
+    if (it == 0) {
+      // zf holds T0^T, and Z1 = T0: no product; Y1 = Y0 T0
+      if ((e = launch_square_pass(zf, K, K, tmax, tmax + K, &tts, nullptr, &zs, s)) !=
+              cudaSuccess ||
+          (e = launch_square_pass(yt, K, K, ymax, ymax, &ys, nullptr, nullptr, s)) != cudaSuccess ||
+          (e = product(ys, tts, 1.0f, 0.0f, yt, nullptr)) != cudaSuccess)
+        return e;
+    } else {
+      if ((e = launch_square_pass(yt, K, K, tmax, tmax + K, &ts, &tts, nullptr, s)) != cudaSuccess ||
+          (e = product(ts, zs, 1.0f, 0.0f, zf, nullptr)) != cudaSuccess)
+        return e;
+      const uint32_t* zmax = rows_of(slot - 1);
+      if ((e = product(ys, tts, 1.0f, 0.0f, yt, nullptr)) != cudaSuccess ||
+          (e = launch_square_pass(zf, K, K, zmax, zmax + K, nullptr, nullptr, &zs, s)) !=
+              cudaSuccess)
+        return e;
+    }
+    const uint32_t* y_rows = rows_of(slot - 1);
+    if ((e = launch_square_pass(yt, K, K, y_rows, y_rows + K, nullptr, nullptr, &ys, s)) !=
+        cudaSuccess)
       return e;
-    transpose_inplace_kernel<<<tiles, dim3(32, 8), 0, s>>>(t, K);     // t = T^T
-    if ((e = gemm_nt(y, K, t, K, z, K, K, K, K, 1.0f, 0.0f, 0.0f, nullptr, gws, status, sms,
-                     s)) != cudaSuccess)            // old Z buffer = Y T (new Y)
-      return e;
-    float* old_y = y;
-    y = z;
-    z = a;
-    a = old_y;
-    symmetrize_kernel<<<tiles, dim3(32, 8), 0, s>>>(y, K);
-    symmetrize_kernel<<<tiles, dim3(32, 8), 0, s>>>(z, K);
+    identity = false;
     if (iterations_done != nullptr) *iterations_done = it + 1;
   }
   // Z ~ (R/c)^-1/2:  R^-1/2 = Z / sqrt(c);  R^-1 = Z Z / c
-  if (inverse)
-    return gemm_nt(z, K, z, K, m, ldm, K, K, K, 1.0f, 0.0f, 0.0f, scal + 4, gws, status, sms, s);
-  scale_copy_kernel<<<elementwise_blocks(kk), 256, 0, s>>>(z, K, scal + 3, m, ldm);
-  return cudaGetLastError();
+  if (identity) {
+    scaled_identity_kernel<<<std::min(K, 4096), 256, 0, s>>>(K, inverse ? scal + 4 : scal + 3, m,
+                                                             ldm);
+    return cudaGetLastError();
+  }
+  if (!inverse) return launch_symmetric_scale(zf, K, K, scal + 3, m, ldm, s);
+  SquareArgs a;
+  a.x = zs;
+  a.y = zs;
+  a.symmetric = true;
+  a.alpha_s = scal + 4;
+  a.c = m;
+  a.ldc = ldm;
+  a.status = status;
+  return launch_square(a, sms, s);
 }
 
 }  // namespace bergson

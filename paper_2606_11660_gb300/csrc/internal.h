@@ -243,6 +243,46 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
                                 float* ws, int* status, int sms, cudaStream_t s);
 
+// Square fp32-accurate products (square.cu).  An operand of `rows` rows of K
+// entries, split into two fp16 planes (hi rows, then lo rows; leading
+// dimension ld, a multiple of 8) with a power-of-two scale per row:
+// entry = 2^-exps[row] (hi + lo).
+struct SplitOperand {
+  __half* planes = nullptr;
+  int* exps = nullptr;
+  int rows = 0;
+  int K = 0;
+  int64_t ld = 0;
+};
+struct SquareArgs {
+  SplitOperand x, y;               // C[b, q] = alpha' <x_b, y_q> + gamma [b == q]
+  bool symmetric = false;          // x == y: half the tiles, mirrored
+  float alpha = 1.0f;
+  const float* alpha_s = nullptr;  // alpha' = alpha * (*alpha_s) when given
+  float gamma = 0.0f;
+  float* c = nullptr;              // [x.rows, ldc]
+  int64_t ldc = 0;
+  uint32_t* row_max = nullptr;     // max |C[b, :]| and max |C[:, q]| as float bits (cleared
+  uint32_t* col_max = nullptr;     //   before the launch), or both nullptr
+  uint32_t* zero_next = nullptr;   // x.rows + y.rows words to clear for a later product
+  float* part = nullptr;           // square_part_floats() sums of (C - I)^2, or nullptr
+  int* status = nullptr;
+};
+cudaError_t launch_square(const SquareArgs& a, int sms, cudaStream_t s);
+int64_t square_part_floats(int M, int N);         // the most sums `part` may receive
+int square_part_count(int M, int N, int sms);     // the sums a plain product writes there
+// Splits of c's rows, columns and symmetric part (K x K; each may be nullptr)
+// scaled by its row and column maxima.
+cudaError_t launch_square_pass(const float* c, int64_t ldc, int K, const uint32_t* rmax,
+                               const uint32_t* cmax, const SplitOperand* row,
+                               const SplitOperand* col, const SplitOperand* sym, cudaStream_t s);
+// m = (c + c^T) / 2 * (*scale)
+cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
+                                   int64_t ldm, cudaStream_t s);
+// The split of x^T from x [n, ldx]; cmax: K words of scratch.
+cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx, uint32_t* cmax,
+                                   const SplitOperand& o, cudaStream_t s);
+
 // Skinny fp32 product C[b, q] = <x_b, y_q> on the tensor cores (on-the-fly
 // scores, preconditioner application): plan and workspace layout.
 struct XGemmPlan {
@@ -272,11 +312,7 @@ struct XGemmArgs {
   const float* y;          // [Q, ldy] fp32, 16-byte aligned rows
   int64_t ldy;
   int B, Q, K;
-  int unit;                // 1: cosine (scale by both norms), 0: affine (below)
-  float alpha = 1.0f;      // unit == 0: out = alpha' <x_b, y_q> + beta out + gamma [b == q],
-  const float* alpha_s = nullptr;   //   alpha' = alpha * (*alpha_s) when alpha_s is given
-  float beta = 0.0f;
-  float gamma = 0.0f;
+  int unit;                // 1: cosine (scale by both norms), 0: plain
   float* scores;           // out [B, ld_scores]
   int64_t ld_scores;
   uint8_t* ws;             // workspace laid out by xgemm_plan(B, Q, K)
@@ -290,5 +326,10 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s);
 // 2-D tiled tensor map with the 128-byte swizzle (host; defined with the C ABI).
 CUresult encode_tmap_2d(CUtensorMap* tm, CUtensorMapDataType dt, const void* ptr, int64_t inner,
                         int64_t outer, int64_t row_bytes, int box_inner, int box_outer);
+
+// 3-D tiled tensor map of a split operand's two fp16 planes, box {box_inner,
+// box_outer, 2}, 128-byte swizzle.
+CUresult encode_tmap_planes(CUtensorMap* tm, const void* ptr, int64_t inner, int64_t outer,
+                            int64_t ld, int box_inner, int box_outer);
 
 }  // namespace bergson

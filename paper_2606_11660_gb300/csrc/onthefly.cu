@@ -856,16 +856,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // of q's y tile, its segments in K order).  Cosine (xnorm given): scores[b, q]
 // = s / sqrt(nx_b) / sqrt(ny_q), nx_b the sum over the row's chunks (in
 // order) of xnorm[b, c], ny_q the sum over the same planes of ynorm[z, q] (0
-// when either row is zero).  Otherwise scores[b, q] = alpha' s + beta scores[b, q] +
-// gamma [b == q], alpha' = alpha * (*alpha_s) when alpha_s is given.
+// when either row is zero).  Otherwise scores[b, q] = s.
 __global__ void finish_kernel(const float* __restrict__ partial, int S, int B, int Q,
                               const float* __restrict__ xnorm, int n_chunks,
                               const float* __restrict__ ynorm, int seg_clusters, int steps,
-                              int y_rows, float alpha, const float* __restrict__ alpha_s,
-                              float beta, float gamma, float* scores, int64_t ld) {
-  griddep_wait();                 // partials, norms and alpha_s come from earlier grids
+                              int y_rows, float* scores, int64_t ld) {
+  griddep_wait();                 // partials and norms come from earlier grids
   const int64_t n = static_cast<int64_t>(B) * Q;
-  const float al = alpha_s != nullptr ? alpha * *alpha_s : alpha;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;     // grid: (Q / 256, rows of b)
   if (q >= Q) return;
   // planes of this row's y tile: all S, or on pairs the tile's segments
@@ -885,10 +882,7 @@ __global__ void finish_kernel(const float* __restrict__ partial, int S, int B, i
       for (int z = 0; z < planes; ++z) ny += ynorm[static_cast<int64_t>(z) * Q + q];
       *dst = nx > 0.0f && ny > 0.0f ? s * (1.0f / sqrtf(nx)) * (1.0f / sqrtf(ny)) : 0.0f;
     } else {
-      float v = al * s;
-      if (beta != 0.0f) v = fmaf(beta, *dst, v);
-      if (b == q) v += gamma;
-      *dst = v;
+      *dst = s;
     }
   }
 }
@@ -1066,7 +1060,7 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s) {
   const float* xn = a.unit ? xnorm : nullptr;
   return launch_dependent(finish_kernel, fgrid, dim3(256), 0, s, p.partial, pl.S, a.B, a.Q, xn,
                           pl.n_chunks, p.ynorm, pl.pair ? pl.n_clusters : 0, pl.steps, pl.y_rows,
-                          a.alpha, a.alpha_s, a.beta, a.gamma, a.scores, a.ld_scores);
+                          a.scores, a.ld_scores);
 }
 
 }  // namespace bergson

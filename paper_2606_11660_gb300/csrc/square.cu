@@ -1,0 +1,710 @@
+// Square products of the Fisher preconditioner (C[b, q] = <x_b, y_q> for two
+// operands of thousands of rows, fp32 accuracy) on the tensor cores.
+//
+// Operands are split once, by the pass that writes them, into two fp16 planes
+// with a power-of-two scale per row:
+//   x_b = 2^-e_b (hi + lo),  e_b such that max |x_b| 2^e_b lies in [2^14, 2^15),
+//   hi = fp16(x 2^e), lo = fp16(x 2^e - hi)        (both rounded to nearest),
+// which leaves |x - hi - lo| <= 2^-23 |x|, or 2^-40 of the row's largest entry
+// where lo becomes subnormal, and the product is taken as
+//   <x, y> ~= <x_lo, y_hi> + <x_hi, y_lo> + <x_hi, y_hi>,
+// the three-product scheme of Ootomo and Yokota (2022) with fp16 parts.  fp16
+// parts hold the same 11 + 11 bits as tf32 parts, at twice the MMA rate, half
+// the operand bytes (4 per entry for both planes) and half as many truncating
+// accumulations per column.
+//
+// Bound: the tensor pipe.  CTA pairs take 256 x 256 output tiles (M = 256 rows
+// of y over the pair, N = 256 rows of x, K = 16 per MMA): a 64-column stage is
+// 64 KB per CTA for 12 MMAs of 128 cycles, 43 bytes of L2 reads per SM and
+// cycle, and 104 of the 128 bytes of shared-memory bandwidth (operand reads 64,
+// TMA writes 40), which a single-CTA 128 x 256 tile (160 with its reads) would
+// not fit.
+//
+// The tensor cores' fp32 accumulation rounds toward zero, so an accumulation
+// chain covers at most kChainStages 64-column stages (48 MMAs, the small lo
+// terms of each 16 columns first); the epilogue adds the chains in registers
+// with IEEE adds, in order, while the next chain runs in the other half of
+// TMEM.  No partial sums go to memory.
+
+#include <algorithm>
+
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace bergson {
+
+namespace {
+
+constexpr int kSqM = 256;                 // rows of y per tile (128 per CTA)
+constexpr int kSqK = 64;                  // fp16 columns per stage: one 128-byte row
+constexpr int kChainStages = 4;           // stages per accumulation chain
+constexpr int kSqThreads = 64 + 256;      // producer, MMA, 8 epilogue warps
+constexpr int kSqBarBytes = 256;
+constexpr int kSqSmemBudget = 232448;
+constexpr int kOutTile = 32 * 33;         // floats of an epilogue warp's output tile
+constexpr int kOutBytes = 8 * kOutTile * 4;
+constexpr uint64_t kSqDrainTimeoutNs = 2000000000ull;
+
+template <int TN_>
+struct SqCfg {
+  static constexpr int TN = TN_;                           // rows of x per tile
+  static constexpr int kABytes = 2 * 128 * 128;            // y: hi and lo planes, 128 rows
+  static constexpr int kBBytes = 2 * (TN / 2) * 128;       // x: this CTA's half of the N side
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kStages = (kSqSmemBudget - 1024 - kSqBarBytes - kOutBytes) / kStageBytes;
+  static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kSqBarBytes + kOutBytes;
+  static constexpr int kTmemCols = 2 * TN;                 // two accumulators
+  static constexpr int kCols = TN / 2;                     // accumulator columns per epilogue warp
+};
+
+struct SqParams {
+  int M, N, K;               // rows of y (q), rows of x (b), columns
+  int n_mt, n_nt;            // tiles
+  int n_tiles;
+  int symmetric;             // x == y: tiles with some b <= q, mirrored into C[q, b]
+  const int* ey;             // [M] scale exponents of y's rows
+  const int* ex;             // [N] scale exponents of x's rows
+  float alpha;
+  const float* alpha_s;      // or nullptr
+  float gamma;               // added on the diagonal
+  float* c;                  // [N, ldc]
+  int64_t ldc;
+  uint32_t* row_max;         // [N] / [M] maxima of |C| over each b / each q (float bits), or
+  uint32_t* col_max;         //   nullptr
+  uint32_t* zero_next;       // [N + M] words cleared for a later product, or nullptr
+  float* part;               // [n_tiles, 16] sums of (C - I)^2 per tile and epilogue warp, or nullptr
+  int* status;
+  uint64_t timeout_ns;
+};
+
+// Tile i of the launch.  Symmetric products enumerate the tiles with some b <=
+// q row by row (row mt has TN == 256 ? mt + 1 : 2 mt + 2 of them, the last row
+// maybe one fewer); others go in groups of kGroup tile rows, so that the tiles
+// in flight form a near-square block and share operand panels in L2.
+constexpr int kGroup = 8;
+template <int TN>
+__device__ __forceinline__ void tile_of(const SqParams& p, int i, int* mt, int* nt) {
+  if (p.symmetric) {
+    constexpr int w = kSqM / TN;                     // row mt starts at w mt (mt + 1) / 2
+    int m = static_cast<int>((sqrtf(8.0f * static_cast<float>(i / w) + 1.0f) - 1.0f) * 0.5f);
+    while (w * (m + 1) * (m + 2) / 2 <= i) ++m;
+    while (w * m * (m + 1) / 2 > i) --m;
+    *mt = m;
+    *nt = i - w * m * (m + 1) / 2;
+    return;
+  }
+  const int per = kGroup * p.n_nt;
+  const int g = i / per, r = i % per;
+  const int m0 = g * kGroup;
+  const int gm = min(kGroup, p.n_mt - m0);
+  *mt = m0 + r % gm;
+  *nt = r / gm;
+}
+
+// TMA load of a {64 columns, rows, 2 planes} box for a CTA pair's barrier.
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap, uint32_t bar,
+                                                 int c0, int c1, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      ".L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
+      "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(0), "l"(policy)
+      : "memory");
+}
+
+__device__ __forceinline__ float pow2f(int e) {     // -126 <= e <= 127
+  return __uint_as_float(static_cast<uint32_t>(e + 127) << 23);
+}
+// v 2^e for |e| <= 252, in two exact factors (results below the normal range
+// round as fp32 does).
+__device__ __forceinline__ float scale2(float v, int e) {
+  const int h = e >> 1;
+  return v * pow2f(h) * pow2f(e - h);
+}
+
+// Scale exponent of a row whose largest |entry| has the float bits `m`: the
+// scaled maximum lies in [2^14, 2^15).  Zero rows and rows with an infinity or
+// NaN keep 0 (their products are what the entries make them).
+__device__ __forceinline__ int row_exponent(uint32_t m) {
+  if (m == 0u || m >= 0x7f800000u) return 0;
+  const int ex = max(static_cast<int>(m >> 23), 1) - 127;
+  return min(14 - ex, 120);
+}
+
+__device__ __forceinline__ bool sq_warp_wait(uint32_t bar, uint32_t parity, uint64_t tmo,
+                                             const volatile int* abort_flag) {
+  bool ok = true;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait_inline(bar, parity, tmo, abort_flag);
+  return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+}
+
+// C[b, q] = alpha' <x_b, y_q> + gamma [b == q] over persistent CTA pairs.
+// Synchronisation as in the pair scorer: the odd CTA's loads complete on the
+// even CTA's `full`, the even CTA's MMA thread frees a stage in both CTAs and
+// hands accumulators to both epilogues by multicast commits, and every
+// epilogue warp of both CTAs releases an accumulator on the even CTA's
+// `tempty`.  Every wait is bounded.
+template <int TN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
+    square_kernel(const __grid_constant__ CUtensorMap tm_y,
+                  const __grid_constant__ CUtensorMap tm_x, const SqParams p) {
+  using C = SqCfg<TN>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  const uint32_t sbase = smem_u32(smem);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);
+  uint64_t* empty = full + C::kStages;
+  uint64_t* tfull = empty + C::kStages;
+  uint64_t* tempty = tfull + 2;
+  uint64_t* drain = tempty + 2;
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(drain + 1);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
+
+  const uint32_t rank = cluster_ctarank();
+  const int cid = blockIdx.x >> 1;
+  const int n_cl = gridDim.x >> 1;
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int nK = (p.K + kSqK - 1) / kSqK;
+  griddep_launch_dependents();   // the next grid sets itself up and waits for this one to end
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::kStages; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&tfull[i]), 1);
+      mbar_init(smem_u32(&tempty[i]), 16);           // 8 epilogue warps of each CTA
+    }
+    mbar_init(smem_u32(drain), 1);
+    *s_abort = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(s_tmem), C::kTmemCols);
+    tmem_relinquish_pair();
+  }
+  griddep_wait();                // operands, exponents and maxima come from earlier grids
+  tc_fence_before();
+  cluster_sync();
+  tc_fence_after();
+  const uint32_t tmem = *s_tmem;
+  const uint64_t tmo = p.timeout_ns;
+  if (p.zero_next != nullptr)
+    for (int i = blockIdx.x * kSqThreads + threadIdx.x; i < p.N + p.M; i += gridDim.x * kSqThreads)
+      p.zero_next[i] = 0u;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    if (lane == 0) {
+      prefetch_tmap(&tm_y);
+      prefetch_tmap(&tm_x);
+      const uint64_t pol = policy_evict_normal();
+      int stage = 0;
+      uint32_t ph = 0;
+      uint32_t issued = 0, issued_par = 0;
+      bool ok = true;
+      for (int t = cid; t < p.n_tiles && ok; t += n_cl) {
+        int mt, nt;
+        tile_of<TN>(p, t, &mt, &nt);
+        for (int kc = 0; kc < nK; ++kc) {
+          if (!mbar_wait(smem_u32(&empty[stage]), ph ^ 1, tmo, s_abort)) { ok = false; break; }
+          const uint32_t fb_local = smem_u32(&full[stage]);
+          const uint32_t fb = mapa_shared(fb_local, 0);
+          if (rank == 0) mbar_arrive_expect_tx(fb_local, 2 * C::kStageBytes);
+          const uint32_t dst = sbase + stage * C::kStageBytes;
+          tma_load_3d_pair(dst, &tm_y, fb, kc * kSqK, mt * kSqM + static_cast<int>(rank) * 128,
+                           pol);
+          tma_load_3d_pair(dst + C::kABytes, &tm_x, fb, kc * kSqK,
+                           nt * TN + static_cast<int>(rank) * (TN / 2), pol);
+          issued |= 1u << stage;
+          issued_par = (issued_par & ~(1u << stage)) | (ph << stage);
+          if (++stage == C::kStages) { stage = 0; ph ^= 1; }
+        }
+      }
+      if (!ok) {
+        raise_device_error(p.status, s_abort, kStatusTimeout);
+        if (rank == 0) {
+          for (int s = 0; s < C::kStages; ++s)
+            if (issued >> s & 1)
+              mbar_wait(smem_u32(&full[s]), (issued_par >> s) & 1, kSqDrainTimeoutNs, nullptr);
+        } else {
+          const uint64_t t0 = global_timer_ns();      // its loads complete on the other CTA's barrier
+          while (global_timer_ns() - t0 < 1000000ull) {
+          }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer (even CTA)
+    if (rank == 0 && lane == 0) {
+      const uint32_t idesc = make_idesc_f16(kSqM, TN, false);
+      int stage = 0;
+      uint32_t ph = 0;
+      int ab = 0;
+      uint32_t aph = 0;
+      bool ok = true;
+      for (int t = cid; t < p.n_tiles && ok; t += n_cl) {
+        int mt, nt;
+        tile_of<TN>(p, t, &mt, &nt);
+        for (int c0 = 0; c0 < nK && ok; c0 += kChainStages) {
+          const int c1 = min(nK, c0 + kChainStages);
+          if (!mbar_wait(smem_u32(&tempty[ab]), aph ^ 1, tmo, s_abort)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d = tmem + ab * TN;
+          for (int kc = c0; kc < c1; ++kc) {
+            if (!mbar_wait(smem_u32(&full[stage]), ph, tmo, s_abort)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t sa = sbase + stage * C::kStageBytes;
+            const uint64_t yh = sw128_desc(sa), yl = sw128_desc(sa + C::kABytes / 2);
+            const uint64_t xh = sw128_desc(sa + C::kABytes);
+            const uint64_t xl = sw128_desc(sa + C::kABytes + C::kBBytes / 2);
+#pragma unroll
+            for (int kk = 0; kk < kSqK / 16; ++kk) {   // 16 fp16 = 32 bytes: +2 in the address field
+              const uint64_t o = 2 * kk;
+              umma_f16_pair(d, yl + o, xh + o, idesc, kc != c0 || kk != 0);
+              umma_f16_pair(d, yh + o, xl + o, idesc, 1u);
+              umma_f16_pair(d, yh + o, xh + o, idesc, 1u);
+            }
+            umma_commit_pair(smem_u32(&empty[stage]), 0x3);
+            if (++stage == C::kStages) { stage = 0; ph ^= 1; }
+          }
+          if (!ok) break;
+          umma_commit_pair(smem_u32(&tfull[ab]), 0x3);
+          if (++ab == 2) { ab = 0; aph ^= 1; }
+        }
+      }
+      if (!ok) raise_device_error(p.status, s_abort, kStatusTimeout);
+      umma_commit_pair(smem_u32(drain), 0x1);
+      mbar_wait(smem_u32(drain), 0, kSqDrainTimeoutNs, nullptr);
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ epilogue
+    // Thread = row q of this CTA's half (TMEM lane) and kCols columns b.
+    const int ew = warp - 2;
+    const int quarter = warp & 3;
+    const int half = ew >> 2;
+    float* tile = reinterpret_cast<float*>(smem + C::kStages * C::kStageBytes + kSqBarBytes) +
+                  ew * kOutTile;
+    const float al = p.alpha_s != nullptr ? p.alpha * *p.alpha_s : p.alpha;
+    int ab = 0;
+    uint32_t aph = 0;
+    bool aborted = false;
+    for (int t = cid; t < p.n_tiles && !aborted; t += n_cl) {
+      int mt, nt;
+      tile_of<TN>(p, t, &mt, &nt);
+      float acc[C::kCols];               // 0 + v = v: the first chain lands unchanged
+#pragma unroll
+      for (int j = 0; j < C::kCols; ++j) acc[j] = 0.0f;
+      for (int c0 = 0; c0 < nK; c0 += kChainStages) {
+        if (!sq_warp_wait(smem_u32(&tfull[ab]), aph, tmo, s_abort)) {
+          raise_device_error(p.status, s_abort, kStatusTimeout);
+          aborted = true;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t tb = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + ab * TN +
+                            half * C::kCols;
+#pragma unroll
+        for (int c = 0; c < C::kCols; c += 16) {
+          float v[16];
+          tmem_ld16(tb + c, v);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(mapa_shared(smem_u32(&tempty[ab]), 0));
+        if (++ab == 2) { ab = 0; aph ^= 1; }
+      }
+      if (aborted) break;
+      // Out through a 32 x 32 tile of shared memory per warp, in rolled loops
+      // (unrolled over the registers, the same code is 80 KB of instructions
+      // fetched once per tile: 15 us of a 23 us launch at K = 256).
+      const int q0 = mt * kSqM + static_cast<int>(rank) * 128 + 32 * quarter;
+      const int q = q0 + lane;
+      const bool qin = q < p.M;
+      const int b0 = nt * TN + half * C::kCols;
+      const int eq = qin ? p.ey[q] : 0;
+      const float uq1 = pow2f(-(eq >> 1)), uq2 = pow2f(-(eq - (eq >> 1)));
+      uint32_t cmax = 0u;
+      float ssq = 0.0f, comp = 0.0f;
+#pragma unroll
+      for (int c = 0; c < C::kCols; c += 32) {
+        const int bc = b0 + c;
+        const int nb = min(32, p.N - bc);
+        const int eb = lane < nb ? p.ex[bc + lane] : 0;
+        const float ub1 = pow2f(-(eb >> 1)), ub2 = pow2f(-(eb - (eb >> 1)));
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) tile[j * 33 + lane] = acc[c + j];
+        __syncwarp();
+        float* dst = p.c + static_cast<int64_t>(bc) * p.ldc + q;
+#pragma unroll 4
+        for (int j = 0; j < 32; ++j, dst += p.ldc) {
+          // acc 2^-(eq + eb): both factors stay within 2^+-120, and so do the halves
+          const float f1 = uq1 * __shfl_sync(0xffffffffu, ub1, j);
+          const float f2 = uq2 * __shfl_sync(0xffffffffu, ub2, j);
+          const int b = bc + j;
+          float v = al * (tile[j * 33 + lane] * f1 * f2);
+          if (b == q) v += p.gamma;
+          const bool in = qin && j < nb;
+          if (in && (!p.symmetric || b <= q)) *dst = v;
+          tile[j * 33 + lane] = in ? v : 0.0f;
+          cmax = max(cmax, in ? __float_as_uint(v) & 0x7fffffffu : 0u);
+          const float r = in ? v - (b == q ? 1.0f : 0.0f) : 0.0f;
+          const float y = r * r - comp;
+          const float u = ssq + y;
+          comp = (u - ssq) - y;
+          ssq = u;
+        }
+        __syncwarp();
+        if (p.row_max != nullptr) {
+          uint32_t m = 0u;
+#pragma unroll 8
+          for (int i = 0; i < 32; ++i)
+            m = max(m, __float_as_uint(tile[lane * 33 + i]) & 0x7fffffffu);
+          if (lane < nb) atomicMax(&p.row_max[bc + lane], m);
+        }
+        if (p.symmetric && lane < nb) {                 // the mirror image C[q, b], b < q
+          float* mir = p.c + static_cast<int64_t>(q0) * p.ldc + bc + lane;
+          const int nq = min(32, p.M - q0);
+#pragma unroll 4
+          for (int i = 0; i < nq; ++i, mir += p.ldc)
+            if (bc + lane < q0 + i) *mir = tile[lane * 33 + i];
+        }
+      }
+      if (p.col_max != nullptr && qin) atomicMax(&p.col_max[q], cmax);
+      if (p.part != nullptr) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
+        if (lane == 0) p.part[static_cast<int64_t>(t) * 16 + rank * 8 + ew] = ssq;
+      }
+    }
+  }
+
+  tc_fence_before();
+  cluster_sync();              // no MMA, commit or remote arrival is still in flight
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, C::kTmemCols);
+  }
+}
+
+// ------------------------------------------------------------ operand passes
+
+// (hi, lo) of the scaled value: hi + lo = v up to 2^-23 |v|.
+__device__ __forceinline__ void split_half(float v, __half* hi, __half* lo) {
+  *hi = __float2half_rn(v);
+  *lo = __float2half_rn(v - __half2float(*hi));
+}
+
+constexpr int kPassTile = 64;
+
+// Writes 64 values of one row of a split operand, two per lane.
+__device__ __forceinline__ void put_row(const SplitOperand& o, int row, int col0, int lane, float a,
+                                        float b, int e) {
+  const int c = col0 + 2 * lane;
+  if (row >= o.rows || c >= o.K) return;
+  __half2 h, l;
+  __half t;
+  split_half(scale2(a, e), &h.x, &t);
+  l.x = t;
+  split_half(scale2(b, e), &h.y, &t);
+  l.y = t;
+  __half* hp = o.planes + static_cast<int64_t>(row) * o.ld + c;
+  __half* lp = hp + static_cast<int64_t>(o.rows) * o.ld;
+  if (c + 1 < o.K) {
+    *reinterpret_cast<__half2*>(hp) = h;
+    *reinterpret_cast<__half2*>(lp) = l;
+  } else {
+    *hp = h.x;
+    *lp = l.x;
+  }
+}
+
+// One pass over a K x K matrix c (row maxima rmax, column maxima cmax, float
+// bits) that writes any of: the split of its rows (o.row), of its columns
+// (o.col: the rows of c^T) and of the rows of its symmetric part
+// (c + c^T) / 2 (o.sym; scaled by the larger of the row's and the column's
+// maximum, a bound of that part's maximum).  One CTA per pair of 64 x 64
+// tiles (ti <= tj): each tile is read once, row by row, and everything is
+// written row by row.  Memory bound: 4 bytes read and 4 written per entry
+// and operand.
+struct SquarePass {
+  const float* c;
+  int64_t ldc;
+  int K;
+  const uint32_t* rmax;
+  const uint32_t* cmax;
+  SplitOperand row, col, sym;    // planes == nullptr: not written
+};
+
+__global__ void __launch_bounds__(256) square_pass_kernel(const SquarePass p) {
+  __shared__ float sa[kPassTile][kPassTile + 1], sb[kPassTile][kPassTile + 1];
+  __shared__ int sexp[3][2][kPassTile];         // row, col, sym exponents of both tiles' rows
+  const int ti = blockIdx.y, tj = blockIdx.x;
+  if (ti > tj) return;
+  griddep_launch_dependents();
+  griddep_wait();
+  const int i0 = ti * kPassTile, j0 = tj * kPassTile;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // every load of both tiles in flight before the first is used
+  float va[16], vb[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int r = w + 8 * (u >> 1), cc = lane + 32 * (u & 1);
+    va[u] = (i0 + r < p.K && j0 + cc < p.K)
+                ? p.c[static_cast<int64_t>(i0 + r) * p.ldc + j0 + cc] : 0.0f;
+    vb[u] = (ti != tj && j0 + r < p.K && i0 + cc < p.K)
+                ? p.c[static_cast<int64_t>(j0 + r) * p.ldc + i0 + cc] : 0.0f;
+  }
+  if (threadIdx.x < 2 * kPassTile) {
+    const int side = threadIdx.x / kPassTile, r = threadIdx.x % kPassTile;
+    const int row = (side ? j0 : i0) + r;
+    const uint32_t rm = row < p.K ? p.rmax[row] : 0u, cm = row < p.K ? p.cmax[row] : 0u;
+    sexp[0][side][r] = row_exponent(rm);
+    sexp[1][side][r] = row_exponent(cm);
+    sexp[2][side][r] = row_exponent(max(rm, cm));
+    if (row < p.K && (side ? i0 : j0) == 0) {   // the tile at column 0 records its rows' exponents
+      if (p.row.planes != nullptr) p.row.exps[row] = sexp[0][side][r];
+      if (p.col.planes != nullptr) p.col.exps[row] = sexp[1][side][r];
+      if (p.sym.planes != nullptr) p.sym.exps[row] = sexp[2][side][r];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int r = w + 8 * (u >> 1), cc = lane + 32 * (u & 1);
+    sa[r][cc] = va[u];
+    sb[r][cc] = ti == tj ? va[u] : vb[u];
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int r = w; r < kPassTile; r += 8) {
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      if (side == 1 && ti == tj) break;
+      const int row = (side ? j0 : i0) + r, col0 = side ? i0 : j0;
+      if (row >= p.K) continue;
+      const float a0 = side ? sb[r][2 * lane] : sa[r][2 * lane];
+      const float a1 = side ? sb[r][2 * lane + 1] : sa[r][2 * lane + 1];
+      const float t0 = side ? sa[2 * lane][r] : sb[2 * lane][r];        // the transposed entries
+      const float t1 = side ? sa[2 * lane + 1][r] : sb[2 * lane + 1][r];
+      if (p.row.planes != nullptr) put_row(p.row, row, col0, lane, a0, a1, sexp[0][side][r]);
+      if (p.col.planes != nullptr) put_row(p.col, row, col0, lane, t0, t1, sexp[1][side][r]);
+      if (p.sym.planes != nullptr)
+        put_row(p.sym, row, col0, lane, 0.5f * (a0 + t0), 0.5f * (a1 + t1), sexp[2][side][r]);
+    }
+  }
+}
+
+// m = (c + c^T) / 2 * (*scale)
+__global__ void __launch_bounds__(256) symmetric_scale_kernel(const float* __restrict__ c, int K,
+                                                              int64_t ldc,
+                                                              const float* __restrict__ scale,
+                                                              float* __restrict__ m, int64_t ldm) {
+  __shared__ float sa[32][33], sb[32][33];
+  const int ti = blockIdx.y, tj = blockIdx.x;
+  if (ti > tj) return;
+  griddep_wait();
+  const int i0 = ti * 32, j0 = tj * 32, x = threadIdx.x;
+  for (int r = threadIdx.y; r < 32; r += 8) {
+    sa[r][x] = (i0 + r < K && j0 + x < K) ? c[static_cast<int64_t>(i0 + r) * ldc + j0 + x] : 0.0f;
+    sb[r][x] = (j0 + r < K && i0 + x < K) ? c[static_cast<int64_t>(j0 + r) * ldc + i0 + x] : 0.0f;
+  }
+  __syncthreads();
+  const float s = *scale;
+  for (int r = threadIdx.y; r < 32; r += 8) {
+    if (i0 + r < K && j0 + x < K)
+      m[static_cast<int64_t>(i0 + r) * ldm + j0 + x] = 0.5f * (sa[r][x] + sb[x][r]) * s;
+    if (ti != tj && j0 + r < K && i0 + x < K)
+      m[static_cast<int64_t>(j0 + r) * ldm + i0 + x] = 0.5f * (sb[r][x] + sa[x][r]) * s;
+  }
+}
+
+// cmax[k] = max over i of |x[i, k]| (float bits; cleared before).  Grid:
+// (columns / 1024, slabs of kMaxRows rows); four columns per thread (K % 4 ==
+// 0 and 16-byte aligned rows, or one column at a time).
+constexpr int kMaxRows = 16;
+__global__ void __launch_bounds__(256) column_max_kernel(const float* __restrict__ x, int n, int K,
+                                                         int64_t ldx, int vec,
+                                                         uint32_t* __restrict__ cmax) {
+  const int i0 = blockIdx.y * kMaxRows, i1 = min(n, i0 + kMaxRows);
+  if (vec) {
+    const int k = (blockIdx.x * 256 + threadIdx.x) * 4;
+    if (k >= K) return;
+    uint4 m = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int u = 0; u < kMaxRows; ++u) {
+      if (i0 + u >= i1) break;
+      const uint4 v = *reinterpret_cast<const uint4*>(x + static_cast<int64_t>(i0 + u) * ldx + k);
+      m.x = max(m.x, v.x & 0x7fffffffu);
+      m.y = max(m.y, v.y & 0x7fffffffu);
+      m.z = max(m.z, v.z & 0x7fffffffu);
+      m.w = max(m.w, v.w & 0x7fffffffu);
+    }
+    atomicMax(&cmax[k], m.x);
+    atomicMax(&cmax[k + 1], m.y);
+    atomicMax(&cmax[k + 2], m.z);
+    atomicMax(&cmax[k + 3], m.w);
+    return;
+  }
+  for (int h = 0; h < 4; ++h) {
+    const int k = blockIdx.x * 1024 + h * 256 + threadIdx.x;
+    if (k >= K) return;
+    uint32_t m = 0u;
+    for (int i = i0; i < i1; ++i)
+      m = max(m, __float_as_uint(x[static_cast<int64_t>(i) * ldx + k]) & 0x7fffffffu);
+    atomicMax(&cmax[k], m);
+  }
+}
+
+// The split of x^T (K rows of n entries) from x [n, ldx].
+__global__ void __launch_bounds__(256) transpose_split_kernel(const float* __restrict__ x, int n,
+                                                              int K, int64_t ldx,
+                                                              const uint32_t* __restrict__ cmax,
+                                                              const SplitOperand o) {
+  __shared__ float s[kPassTile][kPassTile + 1];
+  __shared__ int sexp[kPassTile];
+  griddep_launch_dependents();
+  griddep_wait();
+  const int i0 = blockIdx.x * kPassTile, k0 = blockIdx.y * kPassTile;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float v[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int r = w + 8 * (u >> 1), cc = lane + 32 * (u & 1);
+    v[u] = (i0 + r < n && k0 + cc < K) ? x[static_cast<int64_t>(i0 + r) * ldx + k0 + cc] : 0.0f;
+  }
+  if (threadIdx.x < kPassTile) {
+    const int k = k0 + threadIdx.x;
+    sexp[threadIdx.x] = row_exponent(k < K ? cmax[k] : 0u);
+    if (i0 == 0 && k < K) o.exps[k] = sexp[threadIdx.x];
+  }
+#pragma unroll
+  for (int u = 0; u < 16; ++u) s[w + 8 * (u >> 1)][lane + 32 * (u & 1)] = v[u];
+  __syncthreads();
+#pragma unroll 4
+  for (int r = w; r < kPassTile; r += 8)
+    put_row(o, k0 + r, i0, lane, s[2 * lane][r], s[2 * lane + 1][r], sexp[r]);
+}
+
+int64_t square_tiles(int M, int N, int tn, bool symmetric) {
+  const int64_t mt = (M + kSqM - 1) / kSqM, nt = (N + tn - 1) / tn;
+  // symmetric: rows of (mt + 1) 256 / tn tiles, the last clipped to nt
+  return symmetric ? (kSqM / tn) * mt * (mt - 1) / 2 + nt : mt * nt;
+}
+
+// Tile width: the one whose rounds over the clusters cost least.  A 128-wide
+// tile is half the products of a 256-wide one but keeps shared memory busier
+// than the tensor pipe (158 bytes per cycle wanted of 128) and pays the same
+// fill and epilogue, so it counts 0.65.
+int square_tile_width(int M, int N, int clusters, bool symmetric) {
+  const int64_t r256 = (square_tiles(M, N, 256, symmetric) + clusters - 1) / clusters;
+  const int64_t r128 = (square_tiles(M, N, 128, symmetric) + clusters - 1) / clusters;
+  return static_cast<double>(r128) * 0.65 < static_cast<double>(r256) ? 128 : 256;
+}
+
+template <int TN>
+cudaError_t launch_square_t(const SplitOperand& y, const SplitOperand& x, SqParams p, int clusters,
+                            cudaStream_t s) {
+  using C = SqCfg<TN>;
+  CUtensorMap tm_y, tm_x;
+  if (encode_tmap_planes(&tm_y, y.planes, y.K, y.rows, y.ld, kSqK, 128) != CUDA_SUCCESS ||
+      encode_tmap_planes(&tm_x, x.planes, x.K, x.rows, x.ld, kSqK, TN / 2) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  static PerDeviceOnce attr;
+  const cudaError_t e = smem_attr_once(attr, square_kernel<TN>, C::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  p.n_mt = (p.M + kSqM - 1) / kSqM;
+  p.n_nt = (p.N + TN - 1) / TN;
+  p.n_tiles = static_cast<int>(square_tiles(p.M, p.N, TN, p.symmetric != 0));
+  const int grid = 2 * std::max(1, std::min(clusters, p.n_tiles));
+  return launch_dependent(square_kernel<TN>, dim3(grid), dim3(kSqThreads), C::kSmemBytes, s, tm_y,
+                          tm_x, p);
+}
+
+}  // namespace
+
+// Most sums a product writes to `part`, and how many it does.
+int64_t square_part_floats(int M, int N) {
+  return 16 * static_cast<int64_t>((M + kSqM - 1) / kSqM) * ((N + 127) / 128);
+}
+
+int square_part_count(int M, int N, int sms) {
+  const int clusters = std::max(1, sms / 2);
+  return static_cast<int>(
+      16 * square_tiles(M, N, square_tile_width(M, N, clusters, false), false));
+}
+
+cudaError_t launch_square(const SquareArgs& a, int sms, cudaStream_t s) {
+  SqParams p = {};
+  p.M = a.y.rows;
+  p.N = a.x.rows;
+  p.K = a.y.K;
+  p.symmetric = a.symmetric ? 1 : 0;
+  p.ey = a.y.exps;
+  p.ex = a.x.exps;
+  p.alpha = a.alpha;
+  p.alpha_s = a.alpha_s;
+  p.gamma = a.gamma;
+  p.c = a.c;
+  p.ldc = a.ldc;
+  p.row_max = a.row_max;
+  p.col_max = a.col_max;
+  p.zero_next = a.zero_next;
+  p.part = a.part;
+  p.status = a.status;
+  p.timeout_ns = kWaitTimeoutNs;
+  const int clusters = std::max(1, sms / 2);
+  return square_tile_width(p.M, p.N, clusters, a.symmetric) == 256
+             ? launch_square_t<256>(a.y, a.x, p, clusters, s)
+             : launch_square_t<128>(a.y, a.x, p, clusters, s);
+}
+
+cudaError_t launch_square_pass(const float* c, int64_t ldc, int K, const uint32_t* rmax,
+                               const uint32_t* cmax, const SplitOperand* row,
+                               const SplitOperand* col, const SplitOperand* sym, cudaStream_t s) {
+  SquarePass p = {};
+  p.c = c;
+  p.ldc = ldc;
+  p.K = K;
+  p.rmax = rmax;
+  p.cmax = cmax;
+  if (row != nullptr) p.row = *row;
+  if (col != nullptr) p.col = *col;
+  if (sym != nullptr) p.sym = *sym;
+  const int t = (K + kPassTile - 1) / kPassTile;
+  return launch_dependent(square_pass_kernel, dim3(t, t), dim3(256), 0, s, p);
+}
+
+cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
+                                   int64_t ldm, cudaStream_t s) {
+  const int t = (K + 31) / 32;
+  return launch_dependent(symmetric_scale_kernel, dim3(t, t), dim3(32, 8), 0, s, c, K, ldc, scale,
+                          m, ldm);
+}
+
+cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx, uint32_t* cmax,
+                                   const SplitOperand& o, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(cmax, 0, static_cast<size_t>(K) * sizeof(uint32_t), s);
+  if (e != cudaSuccess) return e;
+  const int vec = ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 ? 1 : 0;
+  // n <= 2^24: at most 2^20 slabs, more than a grid's y dimension holds
+  const int slabs = (n + kMaxRows - 1) / kMaxRows;
+  for (int s0 = 0; s0 < slabs; s0 += 65535) {
+    const int cnt = std::min(65535, slabs - s0);
+    const int64_t row0 = static_cast<int64_t>(s0) * kMaxRows;
+    column_max_kernel<<<dim3((K + 1023) / 1024, cnt), 256, 0, s>>>(
+        x + row0 * ldx, static_cast<int>(n - row0), K, ldx, vec, cmax);
+  }
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const dim3 grid((n + kPassTile - 1) / kPassTile, (K + kPassTile - 1) / kPassTile);
+  return launch_dependent(transpose_split_kernel, grid, dim3(256), 0, s, x, n, K, ldx,
+                          static_cast<const uint32_t*>(cmax), o);
+}
+
+}  // namespace bergson

@@ -1,0 +1,89 @@
+"""Square fp32-accurate products (Fisher fit, Newton-Schulz) at tile edges.
+
+Sizes straddle the 128- and 256-row tiles, the 64-column stages and the
+256-column accumulation chains, with columns of very different scale, zero
+columns and an outlying example, against fp64.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2606_11660_gb300 as bg
+from oracle import bergson_oracle as orc
+from paper_2606_11660_gb300 import workloads as wl
+from tests._util import np32
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _fit(x, pad=0):
+    n, K = x.shape
+    buf = torch.zeros((n, K + pad), device=DEV)
+    buf[:, :K] = x.to(DEV)
+    R = torch.full((K, K + pad), float("nan"), device=DEV)
+    ws = bg.workspace_tensor(bg.bergson_fisher_fit_workspace(n, K), DEV)
+    bg.bergson_fisher_fit(buf, n, K, R, ws)
+    assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+    return R[:, :K]
+
+
+@pytest.mark.parametrize("n,K,pad", [(1, 4, 0), (7, 12, 4), (64, 128, 0), (65, 132, 8),
+                                     (300, 252, 0), (257, 260, 0), (130, 516, 4), (1025, 1028, 0)])
+def test_fit_at_tile_edges(n, K, pad):
+    g = wl.generator(n + K, "cpu")
+    x = torch.randn((n, K), generator=g) * torch.logspace(-4, 4, K)
+    x[n // 2] *= 2.0 ** 12                    # one example far above the rest
+    x[:, K // 2] = 0.0
+    R = np32(_fit(x, pad)).astype(np.float64)
+    assert np.array_equal(R, R.T)
+    want = orc.fisher_fit(x.numpy())
+    # per entry, against the Cauchy-Schwarz scale: both operands' 2^-23, a chain of at most 48
+    # truncating sums of 2^-23, and n / 256 fp32 sums of chains
+    d = np.sqrt(np.diag(want))
+    err = np.abs(R - want) / np.maximum(np.outer(d, d), 1e-300)
+    assert err.max() <= (2 + 48 + (n // 256 + 2)) * 2.0 ** -23, err.max()
+
+
+def test_fit_keeps_infinities_and_nan_in_their_rows():
+    g = wl.generator(3, "cpu")
+    x = torch.randn((70, 136), generator=g)
+    x[5, 7] = float("inf")
+    x[9, 100] = float("nan")
+    R = np32(_fit(x))
+    bad = np.zeros(136, bool)
+    bad[[7, 100]] = True
+    assert np.isfinite(R[~bad][:, ~bad]).all()
+    assert not np.isfinite(R[bad]).any() and not np.isfinite(R[:, bad]).any()
+
+
+@pytest.mark.parametrize("K", [4, 60, 132, 260, 516])
+@pytest.mark.parametrize("power", [bg.BERGSON_FISHER_INV_SQRT, bg.BERGSON_FISHER_INV])
+def test_power_at_tile_edges(K, power):
+    g = wl.generator(K, "cpu")
+    x1 = torch.randn((2 * K, K), generator=g) * torch.linspace(0.5, 2.0, K)
+    x2 = torch.randn((K + 3, K), generator=g)
+    R1, R2 = orc.fisher_fit(x1.numpy()), orc.fisher_fit(x2.numpy())
+    M = torch.full((K, K + 4), float("nan"), device=DEV)
+    ws = bg.workspace_tensor(bg.bergson_fisher_preconditioner_workspace(K), DEV)
+    t1, t2 = (torch.tensor(r, dtype=torch.float32, device=DEV) for r in (R1, R2))
+    done, res = bg.bergson_fisher_preconditioner_tol(t1, t2, K, 0.25, 0.1, power, 40, 2e-5, M, ws)
+    assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+    assert done < 40 and res[-1] <= 2e-5
+    p = -0.5 if power == bg.BERGSON_FISHER_INV_SQRT else -1.0
+    want = orc.fisher_power(orc.fisher_mix(R1, R2, 0.25, 0.1), p)
+    got = np32(M)[:, :K].astype(np.float64)
+    # the residual bounds ||M R M - I||; the inverse doubles it, the condition number is below 100
+    assert np.linalg.norm(got - want) / np.linalg.norm(want) < 1e-3
+
+
+@pytest.mark.parametrize("power", [bg.BERGSON_FISHER_INV_SQRT, bg.BERGSON_FISHER_INV])
+def test_power_that_starts_converged(power):
+    # R = I at K = 4 has c = 2: a tolerance above the first residual stops at Z = I
+    R = torch.eye(4, device=DEV)
+    M = torch.full((4, 4), float("nan"), device=DEV)
+    ws = bg.workspace_tensor(bg.bergson_fisher_preconditioner_workspace(4), DEV)
+    done, res = bg.bergson_fisher_preconditioner_tol(R, None, 4, 1.0, 0.0, power, 10, 0.9, M, ws)
+    assert done == 0 and len(res) == 1 and abs(res[0] - 0.5) < 1e-6
+    want = 2.0 ** (-0.5 if power == bg.BERGSON_FISHER_INV_SQRT else -1.0)
+    np.testing.assert_allclose(np32(M), np.eye(4) * want, rtol=1e-6)
