@@ -412,13 +412,13 @@ BERGSON_API int bergson_fisher_preconditioner(const float* R1, const float* R2, 
  *   res_i = ||I - Z_i Y_i||_F / sqrt(K)     (= ||M_i R M_i - I||_F / sqrt(K)
  *                                            while the iteration keeps Y = R Z / c),
  *
- * is read back to the host; the iteration stops at the first i with
+ * is taken on the device; the iteration stops at the first i with
  * res_i <= tol, or after max_iterations updates.  M is formed from that iterate.
  *   residuals   host fp32 [max_iterations + 1] or NULL: res_0, res_1, ... up to
  *               the last iterate computed.
  *   iterations  host int or NULL: the number of updates applied.
- * Unlike the other calls this one synchronises `stream` once per iterate
- * (one 4-byte read each; the call is a one-time setup cost).  tol = 0 runs
+ * Unlike the other calls this one synchronises `stream` every few iterates
+ * to read the residuals back (the call is a one-time setup cost).  tol = 0 runs
  * all max_iterations updates and still records every residual.
  * Errors: those of bergson_fisher_preconditioner, and EINVAL for tol < 0.
  */

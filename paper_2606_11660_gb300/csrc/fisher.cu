@@ -14,14 +14,16 @@
 // All products are "NT" (C = A B^T, the reduction index contiguous in both
 // operands) on the pair kernel of square.cu, whose operands are fp16 hi + lo
 // planes with per-row scales: every matrix of the iteration is split once, by
-// the pass that also symmetrises or transposes it, and the product itself
-// takes the row and column maxima that pass scales by.  Products of the
+// the pass that also symmetrises it (the product takes the row and column
+// maxima that pass scales by), or by the product itself (T).  Products of the
 // iteration are symmetric in exact arithmetic; each update is re-symmetrised
 // so that rounding cannot build up an antisymmetric part.
 //
-// Measured (K = 3072, n = 1024, 12 updates, one GB300): 17.4 ms per fit and
+// Measured (one GB300, n = 1024, 12 updates at K = 3072): 17.4 ms per fit and
 // power with tf32 parts on single CTAs, K slices through partial sums in
-// memory and separate transpose / symmetrise / norm passes; 5.55 ms as here (a product 119 us in ncu, its MMAs 76).
+// memory and separate transpose / symmetrise / norm passes; 5.6 ms as here.
+// Per update: 42 / 63 / 420 us at K = 256 / 1024 / 3072 (58 / 97 / 425 us with a
+// launch for every product and pass and T split by a pass of its own).
 
 #include <algorithm>
 
@@ -140,9 +142,11 @@ __device__ __forceinline__ float ordered_sum(const float* __restrict__ part, int
 
 // scal[1] = ||R||_F = c, scal[2] = 1/c, scal[3] = 1/sqrt(c), scal[4] = 1/c
 __global__ void __launch_bounds__(1024) frob_final_kernel(const float* __restrict__ part,
-                                                          int n_part, float* __restrict__ scal) {
+                                                          int n_part, float* __restrict__ scal,
+                                                          int* stop) {
   const float t = ordered_sum(part, n_part);
   if (threadIdx.x != 0) return;
+  *stop = 0;
   const float c = sqrtf(t);
   scal[1] = c;
   scal[2] = 1.0f / c;
@@ -150,13 +154,19 @@ __global__ void __launch_bounds__(1024) frob_final_kernel(const float* __restric
   scal[4] = 1.0f / c;
 }
 
-// *out = scale * sqrt(sum of part[0, n_part))
+// *out = scale * sqrt(sum of part[0, n_part)); *stop is set once that is <= tol.
 __global__ void __launch_bounds__(1024) frob_norm_kernel(const float* __restrict__ part, int n_part,
-                                                         float scale, float* __restrict__ out) {
+                                                         float scale, float tol,
+                                                         float* __restrict__ out, int* stop) {
   griddep_launch_dependents();
   griddep_wait();
+  if (*stop != 0) return;
   const float t = ordered_sum(part, n_part);
-  if (threadIdx.x == 0) *out = scale * sqrtf(t);
+  if (threadIdx.x == 0) {
+    const float r = scale * sqrtf(t);
+    *out = r;
+    if (r <= tol) *stop = 1;
+  }
 }
 
 // The first iterate without products: Y0 = R / c (in place in y), its row
@@ -256,7 +266,20 @@ SplitOperand take_split(uint8_t* ws, size_t* off, int rows, int K) {
   return o;
 }
 
-constexpr int kMaxSlots = 4;   // row / column maxima of the products in flight (see launch_fisher_power)
+// T = 1.5 I - 0.5 Z Y has its spectrum in [1, 1.5] (in [1.5 - cond/2, 1.5] at
+// worst before an iteration diverges), so its rows' maxima are known without
+// looking: entries up to 127 fit in fp16 at this exponent, and an entry's lo
+// part is exact to 2^-34, far below the 2^-24 of T's diagonal.  So the product
+// itself writes the splits of T and T^T, with no fp32 T and no pass over it.
+constexpr int kTExp = 9;
+
+// Iterates enqueued between two read-backs of their residuals.  Everything after
+// the first one within the tolerance finds the stop flag set and does nothing,
+// so the device need not wait for the host after every residual (25 us a time).
+constexpr int kItersPerSync = 4;
+constexpr int kMaxIterations = 100;
+constexpr int kScalBytes = 512;      // scalars [0, 8), residuals [8, 8 + kMaxIterations]
+static_assert((8 + kMaxIterations + 1) * sizeof(float) <= kScalBytes, "residual slots");
 
 size_t part_floats(int64_t K) {
   const int64_t t = (K + 63) / 64;
@@ -286,76 +309,80 @@ cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* 
   a.c = r;
   a.ldc = ldr;
   a.status = status;
-  return launch_square(a, sms, s);
+  return launch_square(&a, 1, sms, s);
 }
 
 size_t fisher_power_workspace(int64_t K) {
   const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
-  return 2 * kk + 4 * split_bytes(K, K) +
-         round_up256((2 * kMaxSlots + 1) * static_cast<size_t>(K) * sizeof(uint32_t)) +
-         round_up256(part_floats(K) * sizeof(float)) + 256;
+  return 2 * kk + 4 * split_bytes(K, K) + round_up256(9 * static_cast<size_t>(K) * sizeof(uint32_t)) +
+         round_up256(part_floats(K) * sizeof(float)) + kScalBytes;
 }
 
 cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t ldr, float lam,
                                 float damping, int inverse, int iterations, float tol,
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
                                 float* ws, int* status, int sms, cudaStream_t s) {
-  // Two fp32 matrices (the last Z product; the Y product, then T) and the
-  // splits of Z, Y, T and T^T.
+  // Two fp32 matrices (the Z and Y products) and the splits of Z, Y, T and T^T.
   uint8_t* base = reinterpret_cast<uint8_t*>(ws);
   const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
-  float* yt = reinterpret_cast<float*>(base);          // Y product, then T
-  float* zf = reinterpret_cast<float*>(base + kk);     // Z product
+  float* yf = reinterpret_cast<float*>(base);
+  float* zf = reinterpret_cast<float*>(base + kk);
   size_t off = 2 * kk;
   const SplitOperand zs = take_split(base, &off, K, K);
   const SplitOperand ys = take_split(base, &off, K, K);
-  const SplitOperand ts = take_split(base, &off, K, K);
-  const SplitOperand tts = take_split(base, &off, K, K);
-  // Maxima: slot i holds a product's row maxima, then its column maxima.  Each
-  // product clears the slot of the next one, whose last reader (a pass three
-  // products back) has ended by then.
+  SplitOperand ts = take_split(base, &off, K, K);
+  SplitOperand tts = take_split(base, &off, K, K);
+  ts.exps = tts.exps = nullptr;
+  ts.exp0 = tts.exp0 = kTExp;
+  // Maxima in two slots: rows and columns of the Z product, then of the Y
+  // product (K words each).  The T product between two uses of a slot clears it.
   uint32_t* maxima = reinterpret_cast<uint32_t*>(base + off);
-  uint32_t* ymax = maxima + 2 * static_cast<int64_t>(kMaxSlots) * K;
-  const size_t max_bytes = (2 * kMaxSlots + 1) * static_cast<size_t>(K) * sizeof(uint32_t);
+  uint32_t* ymax = maxima + 8 * static_cast<int64_t>(K);      // row maxima of R, then of Y0
+  const size_t max_bytes = 9 * static_cast<size_t>(K) * sizeof(uint32_t);
   off += round_up256(max_bytes);
   float* part = reinterpret_cast<float*>(base + off);
   off += round_up256(part_floats(K) * sizeof(float));
-  float* scal = reinterpret_cast<float*>(base + off);  // trace, c, 1/c, 1/sqrt(c), 1/c, residual
-  int slot = 0;
-  auto rows_of = [&](int i) { return maxima + 2 * static_cast<int64_t>(i % kMaxSlots) * K; };
-  auto product = [&](const SplitOperand& x, const SplitOperand& y, float alpha, float gamma,
-                     float* c, float* sums) {
+  float* scal = reinterpret_cast<float*>(base + off);  // trace, c, 1/c, 1/sqrt(c), 1/c, -, stop
+  int* stop = reinterpret_cast<int*>(scal + 6);
+  auto slot = [&](int it) { return maxima + 4 * static_cast<int64_t>(it & 1) * K; };
+  auto product = [&](const SplitOperand& x, const SplitOperand& y, float* c, uint32_t* max) {
     SquareArgs a;
     a.x = x;
     a.y = y;
-    a.alpha = alpha;
-    a.gamma = gamma;
     a.c = c;
     a.ldc = K;
-    a.row_max = rows_of(slot);
-    a.col_max = rows_of(slot) + K;
-    a.zero_next = rows_of(slot + 1);
-    a.part = sums;
+    a.row_max = max;
+    a.col_max = max + K;
+    a.stop = stop;
     a.status = status;
-    ++slot;
-    return launch_square(a, sms, s);
+    return a;
+  };
+  auto sym_pass = [&](const float* c, const uint32_t* max, const SplitOperand& o) {
+    SquarePassArgs a;
+    a.c = c;
+    a.rmax = max;
+    a.cmax = max + K;
+    a.sym = o;
+    return a;
   };
   const bool track = residuals != nullptr || tol > 0.0f;
   if (iterations_done != nullptr) *iterations_done = 0;
   cudaError_t e = cudaMemsetAsync(maxima, 0, max_bytes, s);
   if (e != cudaSuccess) return e;
   mixed_trace_kernel<<<1, 1024, 0, s>>>(r1, r2, ldr, K, lam, scal);
-  mix_kernel<<<std::min(K, 4096), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, yt, ymax, part);
-  frob_final_kernel<<<1, 1024, 0, s>>>(part, K, scal);
+  mix_kernel<<<std::min(K, 4096), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, yf, ymax, part);
+  frob_final_kernel<<<1, 1024, 0, s>>>(part, K, scal, stop);
   const int t64 = (K + 63) / 64;
-  ns_first_kernel<<<dim3(t64, t64), 256, 0, s>>>(yt, K, scal, ymax, zf, rows_of(0), rows_of(0) + K,
-                                                 part);
+  ns_first_kernel<<<dim3(t64, t64), 256, 0, s>>>(yf, K, scal, ymax, zf, slot(0), slot(0) + K, part);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  ++slot;
-  bool identity = true;          // Z is still I
   const int n_part = square_part_count(K, K, sms);
+  int updates = 0;               // updates applied (Z is still I at 0)
+  int read = 0;                  // residuals read back
   for (int it = 0;; ++it) {
-    if (!track && it == iterations) break;
+    if (!track && it == iterations) {
+      updates = it;
+      break;
+    }
     // T = 1.5 I - 0.5 Z Y;  Z <- T Z;  Y <- Y T.
     // Z Y is not symmetric in floating point, so T != T^T: the Y update must
     // use T itself.  The products are NT (C = A B^T), so T Z = nt(T, Z) (Z is
@@ -366,52 +393,75 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
     // eigenvalues of R^1/2, so once R's condition number exceeds ~34
     // (s_i / s_j > 3 + sqrt(8)) the converged iterates drift away again.
     // With Y T the same perturbation maps to a fixed point: stable.)
-    const int t_slot = it == 0 ? 0 : slot;
-    if (it > 0 && (e = product(zs, ys, -0.5f, 1.5f, yt, track ? part : nullptr)) != cudaSuccess)
-      return e;
+    if (it > 0) {
+      SquareArgs t;
+      t.x = zs;
+      t.y = ys;
+      t.alpha = -0.5f;
+      t.gamma = 1.5f;
+      t.row_out = ts;
+      t.col_out = tts;
+      t.zero_next = slot(it);              // read last by the passes of update it - 2
+      t.n_zero = 4 * K;
+      t.part = track ? part : nullptr;
+      t.stop = stop;
+      t.status = status;
+      if ((e = launch_square(&t, 1, sms, s)) != cudaSuccess) return e;
+    }
     if (track) {
       // ||I - Z Y||_F / sqrt(K) = 2 ||T - I||_F / sqrt(K): the current iterate's
       // residual (Z Y = Z (R/c) Z = M R M while the iteration keeps Y = (R/c) Z).
       e = launch_dependent(frob_norm_kernel, dim3(1), dim3(1024), 0, s,
                            static_cast<const float*>(part), it == 0 ? t64 * t64 : n_part,
-                           2.0f / sqrtf(static_cast<float>(K)), scal + 5);
+                           2.0f / sqrtf(static_cast<float>(K)), tol, scal + 8 + it, stop);
       if (e != cudaSuccess) return e;
-      float res = 0.0f;
-      if ((e = cudaMemcpyAsync(&res, scal + 5, sizeof(float), cudaMemcpyDeviceToHost, s)) !=
-              cudaSuccess ||
-          (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return e;
-      if (residuals != nullptr) residuals[it] = res;
-      if (res <= tol) break;
+      if (it == iterations || it % kItersPerSync == kItersPerSync - 1) {
+        float res[kItersPerSync];
+        const int n = it + 1 - read;
+        if ((e = cudaMemcpyAsync(res, scal + 8 + read, n * sizeof(float), cudaMemcpyDeviceToHost,
+                                 s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+          return e;
+        bool done = it == iterations;
+        updates = it;
+        for (int i = 0; i < n; ++i) {
+          if (residuals != nullptr) residuals[read + i] = res[i];
+          if (res[i] <= tol) {
+            updates = read + i;
+            done = true;
+            break;
+          }
+        }
+        read = it + 1;
+        if (done) break;
+      }
     }
-    if (it == iterations) break;
-    const uint32_t* tmax = rows_of(t_slot);
+    uint32_t* mx = slot(it);
     if (it == 0) {
       // zf holds T0^T, and Z1 = T0: no product; Y1 = Y0 T0
-      if ((e = launch_square_pass(zf, K, K, tmax, tmax + K, &tts, nullptr, &zs, s)) !=
-              cudaSuccess ||
-          (e = launch_square_pass(yt, K, K, ymax, ymax, &ys, nullptr, nullptr, s)) != cudaSuccess ||
-          (e = product(ys, tts, 1.0f, 0.0f, yt, nullptr)) != cudaSuccess)
+      SquarePassArgs a[2];
+      a[0] = sym_pass(zf, mx, zs);
+      a[0].row = tts;
+      a[1].c = yf;
+      a[1].rmax = a[1].cmax = ymax;
+      a[1].row = ys;
+      const SquareArgs y1 = product(ys, tts, yf, mx + 2 * K);
+      const SquarePassArgs yp = sym_pass(yf, mx + 2 * K, ys);
+      if ((e = launch_square_pass(a, 2, K, stop, s)) != cudaSuccess ||
+          (e = launch_square(&y1, 1, sms, s)) != cudaSuccess ||
+          (e = launch_square_pass(&yp, 1, K, stop, s)) != cudaSuccess)
         return e;
     } else {
-      if ((e = launch_square_pass(yt, K, K, tmax, tmax + K, &ts, &tts, nullptr, s)) != cudaSuccess ||
-          (e = product(ts, zs, 1.0f, 0.0f, zf, nullptr)) != cudaSuccess)
-        return e;
-      const uint32_t* zmax = rows_of(slot - 1);
-      if ((e = product(ys, tts, 1.0f, 0.0f, yt, nullptr)) != cudaSuccess ||
-          (e = launch_square_pass(zf, K, K, zmax, zmax + K, nullptr, nullptr, &zs, s)) !=
-              cudaSuccess)
+      const SquareArgs zy[2] = {product(ts, zs, zf, mx), product(ys, tts, yf, mx + 2 * K)};
+      const SquarePassArgs ps[2] = {sym_pass(zf, mx, zs), sym_pass(yf, mx + 2 * K, ys)};
+      if ((e = launch_square(zy, 2, sms, s)) != cudaSuccess ||
+          (e = launch_square_pass(ps, 2, K, stop, s)) != cudaSuccess)
         return e;
     }
-    const uint32_t* y_rows = rows_of(slot - 1);
-    if ((e = launch_square_pass(yt, K, K, y_rows, y_rows + K, nullptr, nullptr, &ys, s)) !=
-        cudaSuccess)
-      return e;
-    identity = false;
-    if (iterations_done != nullptr) *iterations_done = it + 1;
   }
+  if (iterations_done != nullptr) *iterations_done = updates;
   // Z ~ (R/c)^-1/2:  R^-1/2 = Z / sqrt(c);  R^-1 = Z Z / c
-  if (identity) {
+  if (updates == 0) {
     scaled_identity_kernel<<<std::min(K, 4096), 256, 0, s>>>(K, inverse ? scal + 4 : scal + 3, m,
                                                              ldm);
     return cudaGetLastError();
@@ -425,7 +475,7 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
   a.c = m;
   a.ldc = ldm;
   a.status = status;
-  return launch_square(a, sms, s);
+  return launch_square(&a, 1, sms, s);
 }
 
 }  // namespace bergson

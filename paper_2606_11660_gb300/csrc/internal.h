@@ -235,7 +235,7 @@ cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* 
 size_t fisher_power_workspace(int64_t K);
 // At most `iterations` Newton-Schulz updates.  With residuals != nullptr or
 // tol > 0 the residual ||I - Z Y||_F / sqrt(K) of every iterate is read back
-// (one stream synchronisation per iterate) into residuals[0 ..] and the
+// (the stream is synchronised every few iterates) into residuals[0 ..] and the
 // iteration stops at the first iterate whose residual is <= tol;
 // *iterations_done receives the number of updates applied.
 cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t ldr, float lam,
@@ -249,7 +249,8 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
 // entry = 2^-exps[row] (hi + lo).
 struct SplitOperand {
   __half* planes = nullptr;
-  int* exps = nullptr;
+  int* exps = nullptr;             // [rows], or nullptr: exp0 for every row
+  int exp0 = 0;
   int rows = 0;
   int K = 0;
   int64_t ld = 0;
@@ -260,22 +261,32 @@ struct SquareArgs {
   float alpha = 1.0f;
   const float* alpha_s = nullptr;  // alpha' = alpha * (*alpha_s) when given
   float gamma = 0.0f;
-  float* c = nullptr;              // [x.rows, ldc]
-  int64_t ldc = 0;
+  float* c = nullptr;              // [x.rows, ldc], or nullptr: C goes to the splits of its rows
+  int64_t ldc = 0;                 //   and columns (at their exp0; x.rows and y.rows multiples
+  SplitOperand row_out, col_out;   //   of 4)
   uint32_t* row_max = nullptr;     // max |C[b, :]| and max |C[:, q]| as float bits (cleared
   uint32_t* col_max = nullptr;     //   before the launch), or both nullptr
-  uint32_t* zero_next = nullptr;   // x.rows + y.rows words to clear for a later product
+  uint32_t* zero_next = nullptr;   // n_zero words to clear for later products
+  int n_zero = 0;
+  const int* stop = nullptr;       // device flag: nonzero = compute and write nothing
   float* part = nullptr;           // square_part_floats() sums of (C - I)^2, or nullptr
   int* status = nullptr;
 };
-cudaError_t launch_square(const SquareArgs& a, int sms, cudaStream_t s);
+// One product, or two of the same shape, alpha, gamma and ldc (a[1] gives its
+// operands, c and maxima only).
+cudaError_t launch_square(const SquareArgs* a, int n, int sms, cudaStream_t s);
 int64_t square_part_floats(int M, int N);         // the most sums `part` may receive
-int square_part_count(int M, int N, int sms);     // the sums a plain product writes there
-// Splits of c's rows, columns and symmetric part (K x K; each may be nullptr)
-// scaled by its row and column maxima.
-cudaError_t launch_square_pass(const float* c, int64_t ldc, int K, const uint32_t* rmax,
-                               const uint32_t* cmax, const SplitOperand* row,
-                               const SplitOperand* col, const SplitOperand* sym, cudaStream_t s);
+int square_part_count(int M, int N, int sms);     // the sums one plain product writes there
+// One or two passes over K x K matrices c (row and column maxima given): the
+// splits of the rows and / or of the symmetric part.
+struct SquarePassArgs {
+  const float* c = nullptr;
+  const uint32_t* rmax = nullptr;
+  const uint32_t* cmax = nullptr;
+  SplitOperand row, sym;           // planes == nullptr: not written
+};
+cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int* stop,
+                               cudaStream_t s);
 // m = (c + c^T) / 2 * (*scale)
 cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
                                    int64_t ldm, cudaStream_t s);

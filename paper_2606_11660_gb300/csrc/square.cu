@@ -57,21 +57,31 @@ struct SqCfg {
   static constexpr int kCols = TN / 2;                     // accumulator columns per epilogue warp
 };
 
+// One product of a launch (a launch runs one or two of the same shape).
+struct SqProblem {
+  const int* ey;             // [M] scale exponents of y's rows, or nullptr: exp0_y for all
+  const int* ex;             // [N] likewise of x's rows
+  int exp0_y, exp0_x;
+  float* c;                  // [N, ldc]; nullptr: the splits below instead
+  uint32_t* row_max;         // [N] / [M] maxima of |C| over each b / each q (float bits), or
+  uint32_t* col_max;         //   nullptr
+};
+
 struct SqParams {
+  SqProblem pr[2];
+  int n_prob;
   int M, N, K;               // rows of y (q), rows of x (b), columns
   int n_mt, n_nt;            // tiles
-  int n_tiles;
+  int n_tiles;               // of one product
   int symmetric;             // x == y: tiles with some b <= q, mirrored into C[q, b]
-  const int* ey;             // [M] scale exponents of y's rows
-  const int* ex;             // [N] scale exponents of x's rows
   float alpha;
   const float* alpha_s;      // or nullptr
   float gamma;               // added on the diagonal
-  float* c;                  // [N, ldc]
   int64_t ldc;
-  uint32_t* row_max;         // [N] / [M] maxima of |C| over each b / each q (float bits), or
-  uint32_t* col_max;         //   nullptr
-  uint32_t* zero_next;       // [N + M] words cleared for a later product, or nullptr
+  SplitOperand row, col;     // splits of C's rows and columns at their exp0 (c == nullptr)
+  uint32_t* zero_next;       // words cleared for later products, or nullptr
+  int n_zero;
+  const int* stop;           // nonzero: nothing is computed or written (nullptr: never)
   float* part;               // [n_tiles, 16] sums of (C - I)^2 per tile and epilogue warp, or nullptr
   int* status;
   uint64_t timeout_ns;
@@ -114,13 +124,6 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap,
 __device__ __forceinline__ float pow2f(int e) {     // -126 <= e <= 127
   return __uint_as_float(static_cast<uint32_t>(e + 127) << 23);
 }
-// v 2^e for |e| <= 252, in two exact factors (results below the normal range
-// round as fp32 does).
-__device__ __forceinline__ float scale2(float v, int e) {
-  const int h = e >> 1;
-  return v * pow2f(h) * pow2f(e - h);
-}
-
 // Scale exponent of a row whose largest |entry| has the float bits `m`: the
 // scaled maximum lies in [2^14, 2^15).  Zero rows and rows with an infinity or
 // NaN keep 0 (their products are what the entries make them).
@@ -128,6 +131,45 @@ __device__ __forceinline__ int row_exponent(uint32_t m) {
   if (m == 0u || m >= 0x7f800000u) return 0;
   const int ex = max(static_cast<int>(m >> 23), 1) - 127;
   return min(14 - ex, 120);
+}
+
+// (hi, lo) of the scaled value: hi + lo = v up to 2^-23 |v|.
+__device__ __forceinline__ void split_half(float v, __half* hi, __half* lo) {
+  *hi = __float2half_rn(v);
+  *lo = __float2half_rn(v - __half2float(*hi));
+}
+__device__ __forceinline__ void split_half2(float a, float b, __half2* hi, __half2* lo) {
+  split_half(a, &hi->x, &lo->x);
+  split_half(b, &hi->y, &lo->y);
+}
+
+// Writes a warp's 32 x 32 output tile (tile[j * 33 + i] = C[bc + j, q0 + i]) to
+// the splits of C's rows and columns, two entries per lane and 64 bytes per
+// row and plane (sizes are multiples of 4).
+__device__ __forceinline__ void put_splits(const SqParams& p, const float* tile, int lane, int bc,
+                                           int nb, int q0) {
+  const int l2 = 2 * (lane & 15), odd = lane >> 4;
+  const int nq = min(32, p.M - q0);
+  const float sr = pow2f(p.row.exp0), sc = pow2f(p.col.exp0);
+  const int64_t rp = static_cast<int64_t>(p.row.rows) * p.row.ld;
+  const int64_t cp = static_cast<int64_t>(p.col.rows) * p.col.ld;
+#pragma unroll 4
+  for (int k = 0; k < 16; ++k) {
+    const int j = 2 * k + odd;
+    __half2 h, l;
+    if (j < nb && l2 < nq) {                       // row bc + j of C, columns q0 + l2, + 1
+      split_half2(tile[j * 33 + l2] * sr, tile[j * 33 + l2 + 1] * sr, &h, &l);
+      __half* d = p.row.planes + static_cast<int64_t>(bc + j) * p.row.ld + q0 + l2;
+      *reinterpret_cast<__half2*>(d) = h;
+      *reinterpret_cast<__half2*>(d + rp) = l;
+    }
+    if (j < nq && l2 < nb) {                       // column q0 + j of C, rows bc + l2, + 1
+      split_half2(tile[l2 * 33 + j] * sc, tile[(l2 + 1) * 33 + j] * sc, &h, &l);
+      __half* d = p.col.planes + static_cast<int64_t>(q0 + j) * p.col.ld + bc + l2;
+      *reinterpret_cast<__half2*>(d) = h;
+      *reinterpret_cast<__half2*>(d + cp) = l;
+    }
+  }
 }
 
 __device__ __forceinline__ bool sq_warp_wait(uint32_t bar, uint32_t parity, uint64_t tmo,
@@ -145,8 +187,10 @@ __device__ __forceinline__ bool sq_warp_wait(uint32_t bar, uint32_t parity, uint
 // `tempty`.  Every wait is bounded.
 template <int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
-    square_kernel(const __grid_constant__ CUtensorMap tm_y,
-                  const __grid_constant__ CUtensorMap tm_x, const SqParams p) {
+    square_kernel(const __grid_constant__ CUtensorMap tm_y0,
+                  const __grid_constant__ CUtensorMap tm_x0,
+                  const __grid_constant__ CUtensorMap tm_y1,
+                  const __grid_constant__ CUtensorMap tm_x1, const __grid_constant__ SqParams p) {
   using C = SqCfg<TN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -191,31 +235,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint64_t tmo = p.timeout_ns;
   if (p.zero_next != nullptr)
-    for (int i = blockIdx.x * kSqThreads + threadIdx.x; i < p.N + p.M; i += gridDim.x * kSqThreads)
+    for (int i = blockIdx.x * kSqThreads + threadIdx.x; i < p.n_zero; i += gridDim.x * kSqThreads)
       p.zero_next[i] = 0u;
+  const int n_all = p.stop != nullptr && *p.stop != 0 ? 0 : p.n_prob * p.n_tiles;
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      prefetch_tmap(&tm_y);
-      prefetch_tmap(&tm_x);
+      prefetch_tmap(&tm_y0);
+      prefetch_tmap(&tm_x0);
       const uint64_t pol = policy_evict_normal();
       int stage = 0;
       uint32_t ph = 0;
       uint32_t issued = 0, issued_par = 0;
       bool ok = true;
-      for (int t = cid; t < p.n_tiles && ok; t += n_cl) {
+      for (int t = cid; t < n_all && ok; t += n_cl) {
+        const bool second = t >= p.n_tiles;
+        const CUtensorMap* tm_y = second ? &tm_y1 : &tm_y0;
+        const CUtensorMap* tm_x = second ? &tm_x1 : &tm_x0;
         int mt, nt;
-        tile_of<TN>(p, t, &mt, &nt);
+        tile_of<TN>(p, second ? t - p.n_tiles : t, &mt, &nt);
         for (int kc = 0; kc < nK; ++kc) {
           if (!mbar_wait(smem_u32(&empty[stage]), ph ^ 1, tmo, s_abort)) { ok = false; break; }
           const uint32_t fb_local = smem_u32(&full[stage]);
           const uint32_t fb = mapa_shared(fb_local, 0);
           if (rank == 0) mbar_arrive_expect_tx(fb_local, 2 * C::kStageBytes);
           const uint32_t dst = sbase + stage * C::kStageBytes;
-          tma_load_3d_pair(dst, &tm_y, fb, kc * kSqK, mt * kSqM + static_cast<int>(rank) * 128,
+          tma_load_3d_pair(dst, tm_y, fb, kc * kSqK, mt * kSqM + static_cast<int>(rank) * 128,
                            pol);
-          tma_load_3d_pair(dst + C::kABytes, &tm_x, fb, kc * kSqK,
+          tma_load_3d_pair(dst + C::kABytes, tm_x, fb, kc * kSqK,
                            nt * TN + static_cast<int>(rank) * (TN / 2), pol);
           issued |= 1u << stage;
           issued_par = (issued_par & ~(1u << stage)) | (ph << stage);
@@ -245,9 +293,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
       int ab = 0;
       uint32_t aph = 0;
       bool ok = true;
-      for (int t = cid; t < p.n_tiles && ok; t += n_cl) {
-        int mt, nt;
-        tile_of<TN>(p, t, &mt, &nt);
+      for (int t = cid; t < n_all && ok; t += n_cl) {
         for (int c0 = 0; c0 < nK && ok; c0 += kChainStages) {
           const int c1 = min(nK, c0 + kChainStages);
           if (!mbar_wait(smem_u32(&tempty[ab]), aph ^ 1, tmo, s_abort)) { ok = false; break; }
@@ -292,9 +338,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
     int ab = 0;
     uint32_t aph = 0;
     bool aborted = false;
-    for (int t = cid; t < p.n_tiles && !aborted; t += n_cl) {
+    for (int t = cid; t < n_all && !aborted; t += n_cl) {
+      const SqProblem& pr = p.pr[t >= p.n_tiles ? 1 : 0];
       int mt, nt;
-      tile_of<TN>(p, t, &mt, &nt);
+      tile_of<TN>(p, t >= p.n_tiles ? t - p.n_tiles : t, &mt, &nt);
       float acc[C::kCols];               // 0 + v = v: the first chain lands unchanged
 #pragma unroll
       for (int j = 0; j < C::kCols; ++j) acc[j] = 0.0f;
@@ -327,7 +374,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
       const int q = q0 + lane;
       const bool qin = q < p.M;
       const int b0 = nt * TN + half * C::kCols;
-      const int eq = qin ? p.ey[q] : 0;
+      const int eq = pr.ey == nullptr ? pr.exp0_y : (qin ? pr.ey[q] : 0);
       const float uq1 = pow2f(-(eq >> 1)), uq2 = pow2f(-(eq - (eq >> 1)));
       uint32_t cmax = 0u;
       float ssq = 0.0f, comp = 0.0f;
@@ -335,13 +382,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
       for (int c = 0; c < C::kCols; c += 32) {
         const int bc = b0 + c;
         const int nb = min(32, p.N - bc);
-        const int eb = lane < nb ? p.ex[bc + lane] : 0;
+        const int eb = pr.ex == nullptr ? pr.exp0_x : (lane < nb ? pr.ex[bc + lane] : 0);
         const float ub1 = pow2f(-(eb >> 1)), ub2 = pow2f(-(eb - (eb >> 1)));
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 32; ++j) tile[j * 33 + lane] = acc[c + j];
         __syncwarp();
-        float* dst = p.c + static_cast<int64_t>(bc) * p.ldc + q;
+        float* dst = pr.c + static_cast<int64_t>(bc) * p.ldc + q;
 #pragma unroll 4
         for (int j = 0; j < 32; ++j, dst += p.ldc) {
           // acc 2^-(eq + eb): both factors stay within 2^+-120, and so do the halves
@@ -351,7 +398,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
           float v = al * (tile[j * 33 + lane] * f1 * f2);
           if (b == q) v += p.gamma;
           const bool in = qin && j < nb;
-          if (in && (!p.symmetric || b <= q)) *dst = v;
+          if (in && pr.c != nullptr && (!p.symmetric || b <= q)) *dst = v;
           tile[j * 33 + lane] = in ? v : 0.0f;
           cmax = max(cmax, in ? __float_as_uint(v) & 0x7fffffffu : 0u);
           const float r = in ? v - (b == q ? 1.0f : 0.0f) : 0.0f;
@@ -361,22 +408,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
           ssq = u;
         }
         __syncwarp();
-        if (p.row_max != nullptr) {
+        if (pr.c == nullptr) put_splits(p, tile, lane, bc, nb, q0);
+        if (pr.row_max != nullptr) {
           uint32_t m = 0u;
 #pragma unroll 8
           for (int i = 0; i < 32; ++i)
             m = max(m, __float_as_uint(tile[lane * 33 + i]) & 0x7fffffffu);
-          if (lane < nb) atomicMax(&p.row_max[bc + lane], m);
+          if (lane < nb) atomicMax(&pr.row_max[bc + lane], m);
         }
         if (p.symmetric && lane < nb) {                 // the mirror image C[q, b], b < q
-          float* mir = p.c + static_cast<int64_t>(q0) * p.ldc + bc + lane;
+          float* mir = pr.c + static_cast<int64_t>(q0) * p.ldc + bc + lane;
           const int nq = min(32, p.M - q0);
 #pragma unroll 4
           for (int i = 0; i < nq; ++i, mir += p.ldc)
             if (bc + lane < q0 + i) *mir = tile[lane * 33 + i];
         }
       }
-      if (p.col_max != nullptr && qin) atomicMax(&p.col_max[q], cmax);
+      if (pr.col_max != nullptr && qin) atomicMax(&pr.col_max[q], cmax);
       if (p.part != nullptr) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
@@ -395,25 +443,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
 
 // ------------------------------------------------------------ operand passes
 
-// (hi, lo) of the scaled value: hi + lo = v up to 2^-23 |v|.
-__device__ __forceinline__ void split_half(float v, __half* hi, __half* lo) {
-  *hi = __float2half_rn(v);
-  *lo = __float2half_rn(v - __half2float(*hi));
-}
-
 constexpr int kPassTile = 64;
 
-// Writes 64 values of one row of a split operand, two per lane.
+// Writes 64 values of one row of a split operand, two per lane, scaled by
+// f = 2^e (|e| <= 120: exact).
 __device__ __forceinline__ void put_row(const SplitOperand& o, int row, int col0, int lane, float a,
-                                        float b, int e) {
+                                        float b, float f) {
   const int c = col0 + 2 * lane;
   if (row >= o.rows || c >= o.K) return;
   __half2 h, l;
-  __half t;
-  split_half(scale2(a, e), &h.x, &t);
-  l.x = t;
-  split_half(scale2(b, e), &h.y, &t);
-  l.y = t;
+  split_half2(a * f, b * f, &h, &l);
   __half* hp = o.planes + static_cast<int64_t>(row) * o.ld + c;
   __half* lp = hp + static_cast<int64_t>(o.rows) * o.ld;
   if (c + 1 < o.K) {
@@ -425,30 +464,38 @@ __device__ __forceinline__ void put_row(const SplitOperand& o, int row, int col0
   }
 }
 
-// One pass over a K x K matrix c (row maxima rmax, column maxima cmax, float
-// bits) that writes any of: the split of its rows (o.row), of its columns
-// (o.col: the rows of c^T) and of the rows of its symmetric part
-// (c + c^T) / 2 (o.sym; scaled by the larger of the row's and the column's
-// maximum, a bound of that part's maximum).  One CTA per pair of 64 x 64
-// tiles (ti <= tj): each tile is read once, row by row, and everything is
-// written row by row.  Memory bound: 4 bytes read and 4 written per entry
-// and operand.
+// One pass over a K x K matrix c, or two of them (grid.z), with row maxima rmax
+// and column maxima cmax (float bits), that writes the split of its rows
+// (o.row) and / or of the rows of its symmetric part (c + c^T) / 2 (o.sym;
+// scaled by the larger of the row's and the column's maximum, a bound of that
+// part's maximum).  One CTA per pair of 64 x 64 tiles (ti <= tj): each tile is
+// read once, row by row, with all its loads in flight, and everything is
+// written row by row.  Memory bound: 4 bytes read and 4 written per entry and
+// operand.
 struct SquarePass {
   const float* c;
   int64_t ldc;
   int K;
   const uint32_t* rmax;
   const uint32_t* cmax;
-  SplitOperand row, col, sym;    // planes == nullptr: not written
+  SplitOperand row, sym;         // planes == nullptr: not written
 };
 
-__global__ void __launch_bounds__(256) square_pass_kernel(const SquarePass p) {
+struct SquarePasses {
+  SquarePass p[2];
+  const int* stop;               // nonzero: nothing is written (nullptr: never)
+};
+
+__global__ void __launch_bounds__(256)
+    square_pass_kernel(const __grid_constant__ SquarePasses pp) {
+  const SquarePass& p = pp.p[blockIdx.z];
   __shared__ float sa[kPassTile][kPassTile + 1], sb[kPassTile][kPassTile + 1];
-  __shared__ int sexp[3][2][kPassTile];         // row, col, sym exponents of both tiles' rows
+  __shared__ float sfac[2][2][kPassTile];       // row and sym scales of both tiles' rows
   const int ti = blockIdx.y, tj = blockIdx.x;
   if (ti > tj) return;
   griddep_launch_dependents();
   griddep_wait();
+  if (pp.stop != nullptr && *pp.stop != 0) return;
   const int i0 = ti * kPassTile, j0 = tj * kPassTile;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // every load of both tiles in flight before the first is used
@@ -465,13 +512,13 @@ __global__ void __launch_bounds__(256) square_pass_kernel(const SquarePass p) {
     const int side = threadIdx.x / kPassTile, r = threadIdx.x % kPassTile;
     const int row = (side ? j0 : i0) + r;
     const uint32_t rm = row < p.K ? p.rmax[row] : 0u, cm = row < p.K ? p.cmax[row] : 0u;
-    sexp[0][side][r] = row_exponent(rm);
-    sexp[1][side][r] = row_exponent(cm);
-    sexp[2][side][r] = row_exponent(max(rm, cm));
+    const int er = p.row.exps == nullptr ? p.row.exp0 : row_exponent(rm);
+    const int es = row_exponent(max(rm, cm));
+    sfac[0][side][r] = pow2f(er);
+    sfac[1][side][r] = 0.5f * pow2f(es);
     if (row < p.K && (side ? i0 : j0) == 0) {   // the tile at column 0 records its rows' exponents
-      if (p.row.planes != nullptr) p.row.exps[row] = sexp[0][side][r];
-      if (p.col.planes != nullptr) p.col.exps[row] = sexp[1][side][r];
-      if (p.sym.planes != nullptr) p.sym.exps[row] = sexp[2][side][r];
+      if (p.row.planes != nullptr && p.row.exps != nullptr) p.row.exps[row] = er;
+      if (p.sym.planes != nullptr) p.sym.exps[row] = es;
     }
   }
 #pragma unroll
@@ -492,10 +539,9 @@ __global__ void __launch_bounds__(256) square_pass_kernel(const SquarePass p) {
       const float a1 = side ? sb[r][2 * lane + 1] : sa[r][2 * lane + 1];
       const float t0 = side ? sa[2 * lane][r] : sb[2 * lane][r];        // the transposed entries
       const float t1 = side ? sa[2 * lane + 1][r] : sb[2 * lane + 1][r];
-      if (p.row.planes != nullptr) put_row(p.row, row, col0, lane, a0, a1, sexp[0][side][r]);
-      if (p.col.planes != nullptr) put_row(p.col, row, col0, lane, t0, t1, sexp[1][side][r]);
+      if (p.row.planes != nullptr) put_row(p.row, row, col0, lane, a0, a1, sfac[0][side][r]);
       if (p.sym.planes != nullptr)
-        put_row(p.sym, row, col0, lane, 0.5f * (a0 + t0), 0.5f * (a1 + t1), sexp[2][side][r]);
+        put_row(p.sym, row, col0, lane, a0 + t0, a1 + t1, sfac[1][side][r]);
     }
   }
 }
@@ -567,7 +613,7 @@ __global__ void __launch_bounds__(256) transpose_split_kernel(const float* __res
                                                               const uint32_t* __restrict__ cmax,
                                                               const SplitOperand o) {
   __shared__ float s[kPassTile][kPassTile + 1];
-  __shared__ int sexp[kPassTile];
+  __shared__ float sfac[kPassTile];
   griddep_launch_dependents();
   griddep_wait();
   const int i0 = blockIdx.x * kPassTile, k0 = blockIdx.y * kPassTile;
@@ -580,15 +626,16 @@ __global__ void __launch_bounds__(256) transpose_split_kernel(const float* __res
   }
   if (threadIdx.x < kPassTile) {
     const int k = k0 + threadIdx.x;
-    sexp[threadIdx.x] = row_exponent(k < K ? cmax[k] : 0u);
-    if (i0 == 0 && k < K) o.exps[k] = sexp[threadIdx.x];
+    const int e = row_exponent(k < K ? cmax[k] : 0u);
+    sfac[threadIdx.x] = pow2f(e);
+    if (i0 == 0 && k < K) o.exps[k] = e;
   }
 #pragma unroll
   for (int u = 0; u < 16; ++u) s[w + 8 * (u >> 1)][lane + 32 * (u & 1)] = v[u];
   __syncthreads();
 #pragma unroll 4
   for (int r = w; r < kPassTile; r += 8)
-    put_row(o, k0 + r, i0, lane, s[2 * lane][r], s[2 * lane + 1][r], sexp[r]);
+    put_row(o, k0 + r, i0, lane, s[2 * lane][r], s[2 * lane + 1][r], sfac[r]);
 }
 
 int64_t square_tiles(int M, int N, int tn, bool symmetric) {
@@ -601,29 +648,33 @@ int64_t square_tiles(int M, int N, int tn, bool symmetric) {
 // tile is half the products of a 256-wide one but keeps shared memory busier
 // than the tensor pipe (158 bytes per cycle wanted of 128) and pays the same
 // fill and epilogue, so it counts 0.65.
-int square_tile_width(int M, int N, int clusters, bool symmetric) {
-  const int64_t r256 = (square_tiles(M, N, 256, symmetric) + clusters - 1) / clusters;
-  const int64_t r128 = (square_tiles(M, N, 128, symmetric) + clusters - 1) / clusters;
+int square_tile_width(int M, int N, int n, int clusters, bool symmetric) {
+  const int64_t r256 = (n * square_tiles(M, N, 256, symmetric) + clusters - 1) / clusters;
+  const int64_t r128 = (n * square_tiles(M, N, 128, symmetric) + clusters - 1) / clusters;
   return static_cast<double>(r128) * 0.65 < static_cast<double>(r256) ? 128 : 256;
 }
 
 template <int TN>
-cudaError_t launch_square_t(const SplitOperand& y, const SplitOperand& x, SqParams p, int clusters,
-                            cudaStream_t s) {
+cudaError_t launch_square_t(const SquareArgs* a, int n, SqParams p, int clusters, cudaStream_t s) {
   using C = SqCfg<TN>;
-  CUtensorMap tm_y, tm_x;
-  if (encode_tmap_planes(&tm_y, y.planes, y.K, y.rows, y.ld, kSqK, 128) != CUDA_SUCCESS ||
-      encode_tmap_planes(&tm_x, x.planes, x.K, x.rows, x.ld, kSqK, TN / 2) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  CUtensorMap tm_y[2], tm_x[2];
+  for (int i = 0; i < 2; ++i) {
+    const SquareArgs& g = a[i < n ? i : 0];
+    if (encode_tmap_planes(&tm_y[i], g.y.planes, g.y.K, g.y.rows, g.y.ld, kSqK, 128) !=
+            CUDA_SUCCESS ||
+        encode_tmap_planes(&tm_x[i], g.x.planes, g.x.K, g.x.rows, g.x.ld, kSqK, TN / 2) !=
+            CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
   static PerDeviceOnce attr;
   const cudaError_t e = smem_attr_once(attr, square_kernel<TN>, C::kSmemBytes);
   if (e != cudaSuccess) return e;
   p.n_mt = (p.M + kSqM - 1) / kSqM;
   p.n_nt = (p.N + TN - 1) / TN;
   p.n_tiles = static_cast<int>(square_tiles(p.M, p.N, TN, p.symmetric != 0));
-  const int grid = 2 * std::max(1, std::min(clusters, p.n_tiles));
-  return launch_dependent(square_kernel<TN>, dim3(grid), dim3(kSqThreads), C::kSmemBytes, s, tm_y,
-                          tm_x, p);
+  const int grid = 2 * std::max(1, std::min(clusters, n * p.n_tiles));
+  return launch_dependent(square_kernel<TN>, dim3(grid), dim3(kSqThreads), C::kSmemBytes, s,
+                          tm_y[0], tm_x[0], tm_y[1], tm_x[1], p);
 }
 
 }  // namespace
@@ -636,48 +687,58 @@ int64_t square_part_floats(int M, int N) {
 int square_part_count(int M, int N, int sms) {
   const int clusters = std::max(1, sms / 2);
   return static_cast<int>(
-      16 * square_tiles(M, N, square_tile_width(M, N, clusters, false), false));
+      16 * square_tiles(M, N, square_tile_width(M, N, 1, clusters, false), false));
 }
 
-cudaError_t launch_square(const SquareArgs& a, int sms, cudaStream_t s) {
+cudaError_t launch_square(const SquareArgs* a, int n, int sms, cudaStream_t s) {
   SqParams p = {};
-  p.M = a.y.rows;
-  p.N = a.x.rows;
-  p.K = a.y.K;
-  p.symmetric = a.symmetric ? 1 : 0;
-  p.ey = a.y.exps;
-  p.ex = a.x.exps;
-  p.alpha = a.alpha;
-  p.alpha_s = a.alpha_s;
-  p.gamma = a.gamma;
-  p.c = a.c;
-  p.ldc = a.ldc;
-  p.row_max = a.row_max;
-  p.col_max = a.col_max;
-  p.zero_next = a.zero_next;
-  p.part = a.part;
-  p.status = a.status;
+  p.n_prob = n;
+  p.M = a->y.rows;
+  p.N = a->x.rows;
+  p.K = a->y.K;
+  p.symmetric = a->symmetric ? 1 : 0;
+  for (int i = 0; i < n; ++i) {
+    p.pr[i].ey = a[i].y.exps;
+    p.pr[i].ex = a[i].x.exps;
+    p.pr[i].exp0_y = a[i].y.exp0;
+    p.pr[i].exp0_x = a[i].x.exp0;
+    p.pr[i].c = a[i].c;
+    p.pr[i].row_max = a[i].row_max;
+    p.pr[i].col_max = a[i].col_max;
+  }
+  p.alpha = a->alpha;
+  p.alpha_s = a->alpha_s;
+  p.gamma = a->gamma;
+  p.ldc = a->ldc;
+  p.row = a->row_out;
+  p.col = a->col_out;
+  p.zero_next = a->zero_next;
+  p.n_zero = a->n_zero;
+  p.stop = a->stop;
+  p.part = a->part;
+  p.status = a->status;
   p.timeout_ns = kWaitTimeoutNs;
   const int clusters = std::max(1, sms / 2);
-  return square_tile_width(p.M, p.N, clusters, a.symmetric) == 256
-             ? launch_square_t<256>(a.y, a.x, p, clusters, s)
-             : launch_square_t<128>(a.y, a.x, p, clusters, s);
+  return square_tile_width(p.M, p.N, n, clusters, a->symmetric) == 256
+             ? launch_square_t<256>(a, n, p, clusters, s)
+             : launch_square_t<128>(a, n, p, clusters, s);
 }
 
-cudaError_t launch_square_pass(const float* c, int64_t ldc, int K, const uint32_t* rmax,
-                               const uint32_t* cmax, const SplitOperand* row,
-                               const SplitOperand* col, const SplitOperand* sym, cudaStream_t s) {
-  SquarePass p = {};
-  p.c = c;
-  p.ldc = ldc;
-  p.K = K;
-  p.rmax = rmax;
-  p.cmax = cmax;
-  if (row != nullptr) p.row = *row;
-  if (col != nullptr) p.col = *col;
-  if (sym != nullptr) p.sym = *sym;
+cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int* stop,
+                               cudaStream_t s) {
+  SquarePasses pp = {};
+  pp.stop = stop;
+  for (int i = 0; i < n; ++i) {
+    pp.p[i].c = a[i].c;
+    pp.p[i].ldc = K;
+    pp.p[i].K = K;
+    pp.p[i].rmax = a[i].rmax;
+    pp.p[i].cmax = a[i].cmax;
+    pp.p[i].row = a[i].row;
+    pp.p[i].sym = a[i].sym;
+  }
   const int t = (K + kPassTile - 1) / kPassTile;
-  return launch_dependent(square_pass_kernel, dim3(t, t), dim3(256), 0, s, p);
+  return launch_dependent(square_pass_kernel, dim3(t, t, n), dim3(256), 0, s, pp);
 }
 
 cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
