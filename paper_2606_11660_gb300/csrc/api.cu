@@ -477,7 +477,7 @@ CUresult encode_2d(CUtensorMap* tm, CUtensorMapDataType dt, const void* ptr, int
 
 struct ScoreLayout {
   int qt = 1;
-  size_t qh_off = 0, heap_off = 0, pace_off = 0, total = 0;
+  size_t qh_off = 0, heap_off = 0, pace_off = 0, pub_off = 0, total = 0;
 };
 
 ScoreLayout plan_score(int64_t K, int64_t Q, int64_t topk) {
@@ -493,6 +493,18 @@ ScoreLayout plan_score(int64_t K, int64_t Q, int64_t topk) {
   // the pair kernel's pacing words, one per CTA (timing only: never initialised)
   L.total = L.pace_off + round_up(static_cast<size_t>(kMaxScoreCTAs) * sizeof(unsigned long long),
                                   256);
+  // The published scores (16 bits per CTA and slot, up to kPlanCTAs CTAs) go where
+  // the lists of CTAs past those would: a region of 8 lists, large enough from
+  // topk = 5 on.
+  const size_t pub = static_cast<size_t>(kPlanCTAs) * L.qt * kScoreQT * sizeof(uint16_t);
+  if (static_cast<size_t>(kMaxScoreCTAs - kPlanCTAs) * topk * L.qt * kScoreQT *
+          sizeof(unsigned long long) >= pub) {
+    L.pub_off = L.heap_off + static_cast<size_t>(kPlanCTAs) * topk * L.qt * kScoreQT *
+                                 sizeof(unsigned long long);
+  } else {
+    L.pub_off = L.total;
+    L.total += round_up(pub, 256);
+  }
   return L;
 }
 
@@ -527,6 +539,23 @@ struct ScoreLaunchPlan {
   std::vector<ScoreLaunch> launches;
 };
 
+// The bound of the score kernels: each of a query's cpg CTAs publishes its j-th
+// best score of its first tile, and the r-th largest of those, r = ceil(topk /
+// j), is at most the k-th best of all rows.  j a little above topk / cpg passes
+// the fewest rows: at topk = 100 over 152 CTAs, j = 1 and r = 100 pass about 164
+// of the 39,000 first-tile rows; over 38 CTAs j = 4, r = 25 pass 186, j = 3 210
+// and j = 8 250.  Lists that can hold every row of their CTA need no bound.
+void score_bound_rule(int64_t rows, int bn, int cpg, int topk, int* j, int* r) {
+  *j = *r = 0;
+  const int64_t tiles = (rows + bn - 1) / bn;
+  if (cpg < 2 || (tiles + cpg - 1) / cpg * bn <= topk) return;
+  const int want = std::min(kScoreMaxJ, static_cast<int>(int64_t{topk} * 6 / (int64_t{cpg} * 5)) + 1);
+  const int need = (topk + want - 1) / want;
+  if (need > cpg) return;
+  *j = want;
+  *r = need;
+}
+
 // Launch sequence of bergson_score_topk for `ctas` resident CTAs (for the pair
 // kernel: 2 x its co-resident clusters).  Pure host logic.
 ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas,
@@ -542,10 +571,16 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
   if (Q <= 0 || (P.pair && sms < 2)) return P;
   int n_qg_total = static_cast<int>((Q + P.gsize - 1) / P.gsize);
   if (P.pair) n_qg_total = (n_qg_total + 1) & ~1;   // whole pairs of query groups
-  // Prefix pass (large stores only): the exact top-k of the first `prefix` rows
-  // lands in the outputs, and its k-th score seeds the full pass's threshold.
+  // Prefix pass (large stores whose kernels cannot bound the k-th best on their
+  // own: topk above 32 times the CTAs of a query group): the exact top-k of the
+  // first `prefix` rows lands in the outputs, and its k-th score seeds the full
+  // pass's threshold.
   const int64_t prefix_rows = round_up(static_cast<size_t>(kPrefixRowsPerTopk * topk), kScoreBN);
-  P.use_prefix = allow_prefix && N >= kPrefixMinFactor * prefix_rows && Q >= kPrefixMinQueries;
+  const int per_group = std::max(1, sms / std::min(sms, n_qg_total));
+  int bound_j = 0, bound_r = 0;
+  score_bound_rule(N, kScoreBN, per_group, static_cast<int>(topk), &bound_j, &bound_r);
+  P.use_prefix = allow_prefix && bound_j == 0 && N >= kPrefixMinFactor * prefix_rows &&
+                 Q >= kPrefixMinQueries;
   for (int pass = 0; pass < n_qg_total; pass += sms) {
     const int n_qg = std::min(sms, n_qg_total - pass);
     // The prefix is cut to whole rounds of store tiles over the CTAs of a
@@ -1077,28 +1112,27 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
   __half* qh = reinterpret_cast<__half*>(ws + L.qh_off);
   unsigned long long* heaps = reinterpret_cast<unsigned long long*>(ws + L.heap_off);
 
-  cudaError_t e = launch_normalize_queries(queries, static_cast<int>(Q), static_cast<int>(K), ld_q,
-                                           least, qh, s);
-  if (e != cudaSuccess) return fail_cuda(e, "query normalisation launch");
-
   // Many queries: clusters of two CTAs share each store tile (128 rows each).
   const bool pair = Q >= kPairMinQueries;
-  CUtensorMap tm_store, tm_q;
-  CUresult r1 = encode_2d(&tm_store, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, store, K, N, ld_store * 2,
-                          kChunk, pair ? kScoreBN / 2 : kScoreBN);
-  CUresult r2 = encode_2d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, qh, K, Q, K * 2, kChunk, kScoreQT);
-  if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS)
-    return fail(BERGSON_ECUDA, "tensor map encoding failed (%d %d)", (int)r1, (int)r2);
-
   int ctas = sm_count(dg.dev);
   if (pair) {
     int resident = 0;
-    e = score_pair_max_ctas(L.qt, std::max(1, std::min(ctas, kMaxScoreCTAs)), &resident);
+    const cudaError_t e = score_pair_max_ctas(L.qt, std::max(1, std::min(ctas, kMaxScoreCTAs)), &resident);
     if (e != cudaSuccess) return fail_cuda(e, "score kernel occupancy query");
     ctas = std::min(ctas, resident);
   }
   const ScoreLaunchPlan P = plan_score_launches(N, Q, topk, ctas, !update);
   if (P.launches.empty()) return fail(BERGSON_ECUDA, "no two-SM cluster fits the score kernel");
+  uint16_t* pub = reinterpret_cast<uint16_t*>(ws + L.pub_off);
+  const int pub_words = std::min(P.ctas, kPlanCTAs) * L.qt * kScoreQT;
+  cudaError_t e = launch_normalize_queries(queries, static_cast<int>(Q), static_cast<int>(K), ld_q,
+                                           least, qh, pub, pub_words, s);
+  if (e != cudaSuccess) return fail_cuda(e, "query normalisation launch");
+  CUtensorMap tm_store, tm_q;
+  int box = 0;
+  CUresult r = encode_2d(&tm_q, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, qh, K, Q, K * 2, kChunk,
+                         pair ? kScoreQT : score_query_rows(static_cast<int>(Q)));
+  if (r != CUDA_SUCCESS) return fail(BERGSON_ECUDA, "tensor map encoding failed (%d)", (int)r);
   for (const ScoreLaunch& l : P.launches) {
     ScoreParams p;
     p.N = static_cast<int>(l.rows);
@@ -1107,8 +1141,23 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
     p.topk = static_cast<int>(topk);
     p.n_qg = l.n_qg;
     p.qg_base = l.qg_base;
-    p.n_ntiles = l.n_tiles;
+    // The plan counts 256-row tiles; the launch evens them out over the CTAs.
+    const int per_group = P.ctas / l.n_qg;
+    p.bn = score_tile_rows(l.rows, per_group);
+    p.n_ntiles = static_cast<int>((l.rows + p.bn - 1) / p.bn);
+    const int cpg = std::max(1, std::min(per_group, p.n_ntiles));
+    const int grid = l.n_qg * cpg;
+    if (box != p.bn) {
+      box = p.bn;
+      r = encode_2d(&tm_store, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, store, K, N, ld_store * 2, kChunk,
+                    pair ? box / 2 : box);
+      if (r != CUDA_SUCCESS) return fail(BERGSON_ECUDA, "tensor map encoding failed (%d)", (int)r);
+    }
+    score_bound_rule(l.rows, p.bn, cpg, static_cast<int>(topk), &p.bound_j, &p.bound_r);
+    if (grid > kPlanCTAs) p.bound_j = p.bound_r = 0;      // no room for their words
+    p.stages = p.q_rows = 0;
     p.heaps = heaps;
+    p.pub = pub;
     p.tau0 = l.stage == 1 && (P.use_prefix || update) ? out_scores : nullptr;
     // a prefix pass leaves its scores in the search's own order; a prior
     // bottom-k state holds scores against q
@@ -1117,14 +1166,14 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
     p.timeout_ns = kWaitTimeoutNs;
     p.pace = pair ? reinterpret_cast<unsigned long long*>(ws + L.pace_off) : nullptr;
     p.pace_tag = pair ? next_pace_tag() : 0;
-    e = pair ? launch_score_pair(L.qt, tm_store, tm_q, p, l.grid, s)
-             : launch_score(L.qt, tm_store, tm_q, p, l.grid, s);
+    e = pair ? launch_score_pair(L.qt, tm_store, tm_q, p, grid, s)
+             : launch_score(tm_store, tm_q, p, grid, s);
     if (e != cudaSuccess) return fail_cuda(e, "score kernel launch");
     // The prefix pass's scores seed the full pass's thresholds, so only
     // the final merge converts them back for a bottom-k search.
     const bool final_merge = l.stage == 1;
-    e = launch_merge(heaps, l.grid, l.n_qg, L.qt, static_cast<int>(topk), l.q_begin, l.q_end,
-                     l.pass, least && final_merge, final_merge ? row_base : 0,
+    e = launch_merge(heaps, pub, grid > kPlanCTAs ? 0 : pub_words, grid, l.n_qg, L.qt, static_cast<int>(topk), l.q_begin, l.q_end,
+                     least && final_merge, final_merge ? row_base : 0,
                      update && final_merge ? out_scores : nullptr,
                      update && final_merge ? out_idx : nullptr, out_scores, out_idx, s);
     if (e != cudaSuccess) return fail_cuda(e, "merge kernel launch");

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
 
 // Fixed-order sum of part[0, n): compensated per thread, then a tree over the
 // threads of the single CTA.  Returned to thread 0.
-__device__ __forceinline__ float ordered_sum(const float* __restrict__ part, int n) {
+__device__ __forceinline__ float ordered_sum(const float* part, int n) {
   __shared__ float red[32];
   float t = 0.0f, comp = 0.0f;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -155,9 +155,8 @@ __global__ void __launch_bounds__(1024) frob_final_kernel(const float* __restric
 }
 
 // *out = scale * sqrt(sum of part[0, n_part)); *stop is set once that is <= tol.
-__global__ void __launch_bounds__(1024) frob_norm_kernel(const float* __restrict__ part, int n_part,
-                                                         float scale, float tol,
-                                                         float* __restrict__ out, int* stop) {
+__global__ void __launch_bounds__(1024) frob_norm_kernel(const float* part, int n_part, float scale,
+                                                         float tol, float* out, int* stop) {
   griddep_launch_dependents();
   griddep_wait();
   if (*stop != 0) return;

@@ -75,6 +75,7 @@ constexpr int kChunk = 64;           // bf16 elements per 128-byte swizzled row
 constexpr int kScoreBN = 256;        // store rows per score tile (tcgen05 N)
 constexpr int kScoreQT = 128;        // queries per query tile (tcgen05 M)
 constexpr int kMaxTopk = 1024;
+constexpr int kScoreMaxJ = 32;       // best first-tile scores a score epilogue thread can take
 constexpr uint64_t kWaitTimeoutNs = 4000000000ull;   // bounded device waits: 4 s
 constexpr int kPlanCTAs = 152;   // persistent CTAs work planners assume (one per SM of this part)
 
@@ -153,8 +154,14 @@ struct ScoreParams {
   int topk;
   int n_qg;             // query groups in this pass
   int qg_base;          // first query group of this pass
-  int n_ntiles;         // ceil(N / 256)
-  unsigned long long* heaps;  // [grid, topk, QT*128]
+  int bn;               // store rows per tile (a multiple of 16, at most 256)
+  int n_ntiles;         // ceil(N / bn)
+  int stages;           // single-CTA kernel (set by launch_score): ring stages
+  int q_rows;           //   and query rows loaded per stage
+  int bound_j;          // the bound on the final k-th best: each CTA publishes its bound_j-th
+  int bound_r;          //   best first-tile score, the bound_r-th largest is it (0: no bound)
+  unsigned long long* heaps;  // [grid, topk, QT*128] lists
+  uint16_t* pub;        // [n_qg, QT*128, grid / n_qg] published scores, cleared (see score.cu)
   const float* tau0;    // per query starting threshold at tau0[q * topk + topk - 1], or nullptr
   int tau0_negate;      // 1: the threshold is -tau0[...] (tau0 holds scores against q while
                         //    the search runs on -q: a bottom-k state)
@@ -203,24 +210,33 @@ struct StoreBlocks {
 cudaError_t launch_build_store_blocks(const float* proj, int B, int64_t ld_proj,
                                       const StoreBlocks& blocks, __half* store, int64_t ld_store,
                                       float* norms, cudaStream_t s);
+// Also clears pub_words of `pub` (the score kernels' published scores).
 cudaError_t launch_normalize_queries(const float* q, int Q, int K, int64_t ld_q, bool negate,
-                                     __half* qh, cudaStream_t s);
-cudaError_t launch_score(int qt, const CUtensorMap& tm_store, const CUtensorMap& tm_q,
-                         const ScoreParams& p, int grid, cudaStream_t s);
+                                     __half* qh, uint16_t* pub, int pub_words, cudaStream_t s);
+// Store rows per tile for `rows` store rows over `ctas_per_group` CTAs, and query
+// rows the single-CTA kernel loads (its tensor map's box).
+int score_tile_rows(int64_t rows, int ctas_per_group);
+int score_query_rows(int Q);
+// Up to 128 queries: one CTA per SM, store tensor map with p.bn-row boxes, query
+// tensor map with score_query_rows()-row boxes.
+cudaError_t launch_score(const CUtensorMap& tm_store, const CUtensorMap& tm_q, ScoreParams p,
+                         int grid, cudaStream_t s);
 // Two-SM variant (clusters of two CTAs, qt x 128 queries per CTA, 128 store
-// rows per CTA per tile): the store tensor map has 128-row boxes, grid and
+// rows per CTA per tile): the store tensor map has p.bn / 2-row boxes, grid and
 // n_qg are even.
 cudaError_t launch_score_pair(int qt, const CUtensorMap& tm_store, const CUtensorMap& tm_q,
                               const ScoreParams& p, int grid, cudaStream_t s);
 cudaError_t score_pair_max_ctas(int qt, int sms, int* ctas);
 constexpr int kPairMinQueries = 129;   // the pair kernel serves Q >= this
-// Final top-k of queries [q_begin, q_end) from the CTAs' heaps.  Heap rows
+// Final top-k of queries [q_begin, q_end) from the CTAs' lists; also clears `pub`
+// for the next launch.  List rows
 // are local to the scored rows; the results report row_base + row.  With
 // prior_scores / prior_idx (a previous [Q, topk] result over other rows, global
 // indices, ordered as this call's output) the prior entries take part in the
 // selection too; they may alias out_scores / out_idx.
-cudaError_t launch_merge(const unsigned long long* heaps, int grid, int n_qg, int qt, int topk,
-                         int q_begin, int q_end, int qg_base, bool negate, int64_t row_base,
+cudaError_t launch_merge(const unsigned long long* heaps, uint16_t* pub, int64_t pub_words,
+                         int grid, int n_qg, int qt, int topk,
+                         int q_begin, int q_end, bool negate, int64_t row_base,
                          const float* prior_scores, const int64_t* prior_idx, float* out_scores,
                          int64_t* out_idx, cudaStream_t s);
 

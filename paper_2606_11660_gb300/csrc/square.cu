@@ -547,10 +547,9 @@ __global__ void __launch_bounds__(256)
 }
 
 // m = (c + c^T) / 2 * (*scale)
-__global__ void __launch_bounds__(256) symmetric_scale_kernel(const float* __restrict__ c, int K,
-                                                              int64_t ldc,
-                                                              const float* __restrict__ scale,
-                                                              float* __restrict__ m, int64_t ldm) {
+__global__ void __launch_bounds__(256) symmetric_scale_kernel(const float* c, int K, int64_t ldc,
+                                                              const float* scale, float* m,
+                                                              int64_t ldm) {
   __shared__ float sa[32][33], sb[32][33];
   const int ti = blockIdx.y, tj = blockIdx.x;
   if (ti > tj) return;
@@ -610,7 +609,7 @@ __global__ void __launch_bounds__(256) column_max_kernel(const float* __restrict
 // The split of x^T (K rows of n entries) from x [n, ldx].
 __global__ void __launch_bounds__(256) transpose_split_kernel(const float* __restrict__ x, int n,
                                                               int K, int64_t ldx,
-                                                              const uint32_t* __restrict__ cmax,
+                                                              const uint32_t* cmax,
                                                               const SplitOperand o) {
   __shared__ float s[kPassTile][kPassTile + 1];
   __shared__ float sfac[kPassTile];

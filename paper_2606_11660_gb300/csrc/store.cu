@@ -107,18 +107,25 @@ __global__ void __launch_bounds__(kRowThreads) normalize_blocks_kernel(
 // Queries may have any row stride; they are read with scalar loads.  With
 // `negate` the row is written as -q / ||q|| (exactly the negation of the
 // unit row: fp16 rounding is symmetric), which turns a top-k search into a
-// bottom-k one.
+// bottom-k one.  The CTAs share the clearing of the score kernels' published
+// words.
 __global__ void __launch_bounds__(kRowThreads) normalize_queries_kernel(
-    const float* __restrict__ q, int K, int64_t ldq, int negate, __half* __restrict__ qh) {
+    const float* __restrict__ q, int K, int64_t ldq, int negate, __half* __restrict__ qh,
+    uint32_t* __restrict__ pub, int n_pub) {
   __shared__ float red[kRowThreads / 32];
+  griddep_launch_dependents();   // the score kernel streams the store meanwhile
+  for (int i = blockIdx.x * kRowThreads + threadIdx.x; i < n_pub; i += gridDim.x * kRowThreads)
+    pub[i] = 0u;
   const int64_t r = blockIdx.x;
   const float* qr = q + r * ldq;
   KahanSum ss;
+#pragma unroll 4
   for (int i = threadIdx.x; i < K; i += kRowThreads) ss.add(qr[i] * qr[i]);
   const float tot = block_sum(ss.s, red);
   const float inv = tot > 0.0f ? 1.0f / sqrtf(tot) : 0.0f;
   const float scale = negate ? -inv : inv;
   __half* out = qh + r * K;
+#pragma unroll 4
   for (int i = threadIdx.x; i < K; i += kRowThreads) out[i] = __float2half_rn(qr[i] * scale);
 }
 
@@ -140,9 +147,11 @@ cudaError_t launch_build_store_blocks(const float* proj, int B, int64_t ld_proj,
 }
 
 cudaError_t launch_normalize_queries(const float* q, int Q, int K, int64_t ld_q, bool negate,
-                                     __half* qh, cudaStream_t s) {
+                                     __half* qh, uint16_t* pub, int pub_words, cudaStream_t s) {
   if (Q == 0) return cudaSuccess;
-  normalize_queries_kernel<<<Q, kRowThreads, 0, s>>>(q, K, ld_q, negate ? 1 : 0, qh);
+  normalize_queries_kernel<<<Q, kRowThreads, 0, s>>>(q, K, ld_q, negate ? 1 : 0, qh,
+                                                     reinterpret_cast<uint32_t*>(pub),
+                                                     pub_words / 2);
   return cudaGetLastError();
 }
 
