@@ -25,8 +25,13 @@
 // Merge kernel: one CTA per query gathers the lists of the CTAs that covered
 // the query and sorts them by score descending, then row ascending (long
 // candidate sets go through an exact radix select first).
-// Measured (3 queries, 20,011 x 3072, top-10 / 100 queries, 250,007 x 12,288,
-// bottom-100): @@M@@.
+// Measured (one GB300, microseconds a call, with heaps / as here): 3 queries,
+// 20,011 x 3072, top-10 91 / 37; 100 queries, 250,007 x 12,288, bottom-100 1530 /
+// 897 (the store stream's time at 6.8 TB/s is 904); 64 queries, 100,003 x 1024,
+// top-500 2810 / 78; 1024 queries, 60,000 x 4096, top-100 1660 / 465 and 300,000 x
+// 2048, top-300 7960 / 1120; 4M x 8192 level (tensor bound).  Small calls pay for
+// code they run once (instruction fetch): fully unrolled searches of the bound
+// and of the candidates cost 5 to 15 us more.
 
 #include <algorithm>
 
@@ -187,7 +192,7 @@ __device__ __noinline__ static void heapify(unsigned long long* heap, int stride
 // rows of cpg words start at `pub`): per slot the r-th largest value, or NaN or
 // -inf while fewer than r are there.  One warp; lane i looks at CTAs i, i + 32,
 // ... of the group.  The slots' loads and reductions run side by side.
-constexpr int kBatch = 4;
+constexpr int kBatch = 8;
 __device__ __forceinline__ void slot_bounds(const uint16_t* pub, int cpg, int r, int lane,
                                             float* out) {
   uint32_t v[kBatch][5];                          // cpg <= 160
@@ -202,7 +207,7 @@ __device__ __forceinline__ void slot_bounds(const uint16_t* pub, int cpg, int r,
   uint32_t t[kBatch];
 #pragma unroll
   for (int s = 0; s < kBatch; ++s) t[s] = 0u;
-#pragma unroll 4
+#pragma unroll 1
   for (int bit = 15; bit >= 0; --bit) {
 #pragma unroll
     for (int s = 0; s < kBatch; ++s) {
@@ -244,13 +249,15 @@ __device__ __forceinline__ float nth_of_tile(uint32_t tbase, int rows, int j) {
   float top[J];
 #pragma unroll
   for (int i = 0; i < J; ++i) top[i] = -INFINITY;
+  // eight columns a time: unrolled over 32, the J = 32 network is 32 KB of code
+  // that each launch fetches for one use
 #pragma unroll 1
-  for (int c = 0; c * 32 < rows; ++c) {
-    float v[32];
-    tmem_ld32(tbase + c * 32, v);
-    const int nvalid = rows - c * 32;
+  for (int c = 0; c < rows; c += 8) {
+    float v[8];
+    tmem_ld8(tbase + c, v);
+    const int nvalid = rows - c;
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
+    for (int i = 0; i < 8; ++i)
       top_insert<J>(top, i < nvalid && v[i] == v[i] ? v[i] : -INFINITY);
   }
   return nth<J>(top, j);
@@ -357,14 +364,14 @@ __device__ __forceinline__ void score_epilogue(const ScoreParams& p, uint32_t tm
         __threadfence();
       }
     }
-    // The bound from the first tiles, and again before tiles 2, 8, 64, 512 from
+    // The bound from the first tiles, and again before tiles 2, 6, 20, ... from
     // the lists, which hold every row seen so far that matters: with t tiles
     // seen a tile adds about 1.3 topk / (cpg t) keys to a list, so the lists
-    // do not fill up unless a CTA's rows come in ascending order.  It takes 20 to
-    // 40 us, so only scans that go on for eight times as long do it.
-    const bool again = j_best > 0 &&
-                       (tile_no == 2 || tile_no == 8 || tile_no == 64 || tile_no == 512) &&
-                       n_my_tiles > 8 * tile_no;
+    // do not fill up unless a CTA's rows come in ascending order.  It takes 10 to
+    // 30 us, so only scans that go on for four times as long do it.
+    const bool again = j_best > 0 && n_my_tiles > 4 * tile_no &&
+                       (tile_no == 2 || tile_no == 6 || tile_no == 20 || tile_no == 60 ||
+                        tile_no == 200);
     if (again && live && cnt >= j_best) {
       const float x = j_best == 1   ? nth_of_list<1>(heap, stride, cnt, 1)
                       : j_best <= 8 ? nth_of_list<8>(heap, stride, cnt, j_best)
