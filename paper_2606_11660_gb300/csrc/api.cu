@@ -34,6 +34,7 @@ constexpr int kMaxDevices = 64;
 constexpr int kMaxTokenQueries = 256;                // per-token scores: queries per call
 constexpr int64_t kPrefixRowsPerTopk = 128;          // prefix pass: 128 * topk store rows
 constexpr int64_t kPrefixMinFactor = 8;              // ... only when N >= 8 * prefix
+constexpr int64_t kPrefixBoundFactor = 128;          // ... or this, where the kernels bound it
 constexpr int64_t kPrefixMinQueries = 129;           // ... and Q > 128 (fewer queries insert
                                                      // too little into their heaps to repay it)
 
@@ -571,16 +572,18 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
   if (Q <= 0 || (P.pair && sms < 2)) return P;
   int n_qg_total = static_cast<int>((Q + P.gsize - 1) / P.gsize);
   if (P.pair) n_qg_total = (n_qg_total + 1) & ~1;   // whole pairs of query groups
-  // Prefix pass (large stores whose kernels cannot bound the k-th best on their
-  // own: topk above 32 times the CTAs of a query group): the exact top-k of the
-  // first `prefix` rows lands in the outputs, and its k-th score seeds the full
-  // pass's threshold.
+  // Prefix pass (large stores): the exact top-k of the first `prefix` rows lands
+  // in the outputs, and its k-th score seeds the full pass's threshold.  Where
+  // the kernels bound the k-th best on their own (topk up to 32 times the CTAs
+  // of a query group), only scans of 128 times the prefix take it: it is level
+  // there (4M x 8192, 1024 queries: within 1%) and costs shorter scans its merge
+  // (187,044 rows, 157 queries: 244 us with it, 191 without).
   const int64_t prefix_rows = round_up(static_cast<size_t>(kPrefixRowsPerTopk * topk), kScoreBN);
   const int per_group = std::max(1, sms / std::min(sms, n_qg_total));
   int bound_j = 0, bound_r = 0;
   score_bound_rule(N, kScoreBN, per_group, static_cast<int>(topk), &bound_j, &bound_r);
-  P.use_prefix = allow_prefix && bound_j == 0 && N >= kPrefixMinFactor * prefix_rows &&
-                 Q >= kPrefixMinQueries;
+  const int64_t factor = bound_j == 0 ? kPrefixMinFactor : kPrefixBoundFactor;
+  P.use_prefix = allow_prefix && N >= factor * prefix_rows && Q >= kPrefixMinQueries;
   for (int pass = 0; pass < n_qg_total; pass += sms) {
     const int n_qg = std::min(sms, n_qg_total - pass);
     // The prefix is cut to whole rounds of store tiles over the CTAs of a
