@@ -174,10 +174,26 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr() if hasattr(t, "data_ptr") else int(t)
 
 
+_raw_stream = None
+
+
+def _current_stream() -> int:
+    """torch's current stream on the current device, without building the
+    Stream object that torch.cuda.current_stream() returns (3 us a call)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()                       # initialises CUDA
+        raw, dev = (getattr(torch._C, n, None)
+                    for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        _raw_stream = ((lambda: raw(dev())) if raw is not None and dev is not None
+                       else (lambda: torch.cuda.current_stream().cuda_stream))
+    return _raw_stream()
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -197,14 +213,14 @@ class Layer:
     bias_col_offset: Optional[int] = None     # set to also write the projected bias gradient
 
     def to_c(self) -> bergson_layer:
-        bias = self.bias_col_offset is not None
+        bias = self.bias_col_offset
+        # in the order of bergson_layer._fields_
         return bergson_layer(
-            A=_ptr(self.A), G=_ptr(self.G), d_in=int(self.A.shape[-1]), d_out=int(self.G.shape[-1]),
-            k_in=int(self.k_in), k_out=int(self.k_out), seed_in=int(self.seed_in),
-            seed_out=int(self.seed_out), proj_kind=int(self.proj_kind),
-            flags=BERGSON_LAYER_BIAS if bias else 0, r=_ptr(self.r), c=_ptr(self.c),
-            out_col_offset=int(self.out_col_offset),
-            bias_col_offset=int(self.bias_col_offset) if bias else 0)
+            _ptr(self.A), _ptr(self.G), int(self.A.shape[-1]), int(self.G.shape[-1]),
+            int(self.k_in), int(self.k_out), int(self.seed_in), int(self.seed_out),
+            int(self.proj_kind), 0 if bias is None else BERGSON_LAYER_BIAS,
+            None if self.r is None else _ptr(self.r), None if self.c is None else _ptr(self.c),
+            int(self.out_col_offset), 0 if bias is None else int(bias))
 
 
 def _layer_array(layers: Sequence) -> "ctypes.Array":

@@ -29,6 +29,12 @@ constexpr int kSchedTargetItems = 8192;              // work items per projectio
 // share of the work, into pieces of about 1/kPiecesPerShare of a share.
 constexpr double kSplitShare = 0.4;
 constexpr int kPiecesPerShare = 2;
+constexpr double kMinPieceUnits = 4.0;               // ... of at least 4 chunks of a tile
+constexpr double kFinePieceShare = 0.8;              // largest piece, in shares, before the minimum
+                                                     // piece size is lowered
+constexpr int kFineMaxK = 96;                        // k_in + k_out up to which it is
+constexpr double kFineSlotUnits = 64.0;              // shares below this (and few slots): slots of
+                                                     // one tile each
 constexpr int kMaxScoreCTAs = 160;                   // upper bound on persistent score CTAs
 constexpr int kMaxDevices = 64;
 constexpr int kMaxTokenQueries = 256;                // per-token scores: queries per call
@@ -238,7 +244,8 @@ int chunks_of(int64_t d) { return static_cast<int>((d + kChunk - 1) / kChunk); }
 // the items of a unit's layers for the same example and tiles are listed next
 // to each other (A-side pieces too), so the scheduler starts them together.
 // Cost unit: one 64-column chunk of one tile; the table runs largest first.
-void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bool allow_split) {
+void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bool allow_split,
+               bool fine) {
   if (g.n_slots == 0) return;
   int64_t total = 0, max_slot = 0;
   for (int li : g.layers) {
@@ -251,86 +258,145 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bo
   bool shared = false;
   for (const auto& u : g.units) shared = shared || u.second > 1;
   if (!split && !shared) return;
-  const double target = share / kPiecesPerShare;
+  // Tiles of a slot (the last slot of an example may have fewer).
+  const int slot_tiles = std::min(g.tpc, n_tiles);
+  const double target = std::max(share / kPiecesPerShare, kMinPieceUnits);
   // A piece stores and its slot's finisher reloads 4k fp32 bytes per token,
   // against 128 bytes per token and chunk streamed: pieces of at least 2k
   // chunks keep that under 1/32 of the piece's traffic.  (Fewer, larger
   // pieces measured faster: Llama-8B-shaped block 0.790 ms at a quarter of a
-  // share per piece, 0.770 ms at half.)
-  auto pieces = [&](int ch, int k) {
-    const int n = static_cast<int>(std::ceil(static_cast<double>(ch) * g.tpc / target));
-    return std::max(1, std::min(n, ch / (2 * k)));
+  // share per piece, 0.770 ms at half.)  Small launches, whose largest piece
+  // would then be most of a CTA's share or more, go down to 3k/8 chunks (an
+  // extra 1/6 of L2 traffic).  Measured together with slots of one tile and one
+  // launch less, us a call: 7 x 333 tokens of 8 modules (k = 32 x 16) 68 -> 54,
+  // 1 x 300 tokens of 4 modules (k = 16) 66 -> 32, 1 x 512 of a Llama-8B-shaped
+  // block 71 -> 63.  At k = 64 x 64 the finishers' sums outweigh it (98 -> 116
+  // with finer pieces), so k_in + k_out stays within kFineMaxK.
+  auto pieces = [&](int ch, int min_ch) {
+    const int n = static_cast<int>(std::ceil(static_cast<double>(ch) * slot_tiles / target));
+    return std::max(1, std::min(n, ch / min_ch));
   };
-  struct Entry {
-    WorkItem w;
+  int min_a = 2 * g.k_in, min_g = 2 * g.k_out;
+  if (split && fine && g.k_in + g.k_out <= kFineMaxK) {
+    double worst = 0.0;
+    for (int li : g.layers) {
+      const int ca = chunks_of(layers[li].d_in), cg = chunks_of(layers[li].d_out);
+      if (static_cast<double>(ca + cg) * slot_tiles <= share / kPiecesPerShare) continue;
+      const int na = pieces(ca, min_a), ng = pieces(cg, min_g);
+      worst = std::max(worst, static_cast<double>(std::max((ca + na - 1) / na, (cg + ng - 1) / ng)) *
+                                  slot_tiles);
+    }
+    if (worst > std::max(kFinePieceShare * share, kMinPieceUnits)) {
+      min_a = 3 * g.k_in / 8;
+      min_g = 3 * g.k_out / 8;
+    }
+  }
+  // Groups of entries of one cost: a unit's fused items, or one of its pieces,
+  // over every example and slot of `tiles` tiles.
+  struct Batch {
     int64_t key;
+    int unit, side, piece, j, tiles;           // j: layer of the unit (G side)
   };
-  std::vector<Entry> es;
+  struct UnitPlan {
+    bool cut = false;
+    int n_a = 0, sid0 = 0;
+    int64_t base0 = 0, slot_floats = 0;
+  };
+  std::vector<Batch> batches;
+  std::vector<UnitPlan> ups(g.units.size());
+  std::vector<int> n_g(g.layers.size(), 0);
+  std::vector<int64_t> off(g.layers.size(), 0);  // a layer's floats within its unit's slot
+  const int n_last = n_tiles - (g.n_chunks - 1) * g.tpc;        // tiles of an example's last slot
   int64_t base = 0;
   int n_split = 0;
-  for (const auto& u : g.units) {
-    const int m0 = u.first, cnt = u.second;
+  size_t n_entries = 0;
+  for (size_t ui = 0; ui < g.units.size(); ++ui) {
+    const int m0 = g.units[ui].first, cnt = g.units[ui].second;
+    UnitPlan& up = ups[ui];
     const int ca = chunks_of(layers[g.layers[m0]].d_in);
-    bool cut = false;
     int64_t worst = 0;
-    std::vector<int> cg(cnt), n_g(cnt, 0);
     for (int j = 0; j < cnt; ++j) {
-      cg[j] = chunks_of(layers[g.layers[m0 + j]].d_out);
-      worst = std::max<int64_t>(worst, ca + cg[j]);
-      cut = cut || (split && static_cast<double>(ca + cg[j]) * g.tpc > target);
+      const int cg = chunks_of(layers[g.layers[m0 + j]].d_out);
+      worst = std::max<int64_t>(worst, ca + cg);
+      up.cut = up.cut || (split && static_cast<double>(ca + cg) * slot_tiles > share / kPiecesPerShare);
     }
-    const int n_a = cut ? pieces(ca, g.k_in) : 0;
-    if (cut)
-      for (int j = 0; j < cnt; ++j) n_g[j] = pieces(cg[j], g.k_out);
-    std::vector<int> sid(cnt);
-    std::vector<int64_t> sbase(cnt);
+    const int kinds = g.n_chunks > 1 && n_last != g.tpc ? 2 : 1;
+    for (int kind = 0; kind < kinds; ++kind) {
+      const int tiles = kind == kinds - 1 ? (kinds == 1 ? std::min(g.tpc, n_tiles) : n_last) : g.tpc;
+      if (!up.cut) {
+        batches.push_back({worst * tiles, static_cast<int>(ui), 0, 0, 0, tiles});
+        continue;
+      }
+      up.n_a = pieces(ca, min_a);
+      for (int q = 0; q < up.n_a; ++q) {
+        const int c0 = static_cast<int>(static_cast<int64_t>(q) * ca / up.n_a);
+        const int c1 = static_cast<int>(static_cast<int64_t>(q + 1) * ca / up.n_a);
+        batches.push_back({int64_t{c1 - c0} * tiles, static_cast<int>(ui), 1, q, 0, tiles});
+      }
+      for (int j = 0; j < cnt; ++j) {
+        const int cg = chunks_of(layers[g.layers[m0 + j]].d_out);
+        n_g[m0 + j] = pieces(cg, min_g);
+        for (int q = 0; q < n_g[m0 + j]; ++q) {
+          const int c0 = static_cast<int>(static_cast<int64_t>(q) * cg / n_g[m0 + j]);
+          const int c1 = static_cast<int>(static_cast<int64_t>(q + 1) * cg / n_g[m0 + j]);
+          batches.push_back({int64_t{c1 - c0} * tiles, static_cast<int>(ui), 2, q, j, tiles});
+        }
+      }
+    }
+    n_entries += static_cast<size_t>(cnt) * B * g.n_chunks;
+    if (up.cut) {
+      n_entries -= static_cast<size_t>(cnt) * B * g.n_chunks;
+      up.sid0 = n_split;
+      up.base0 = base;
+      for (int j = 0; j < cnt; ++j) {
+        off[m0 + j] = up.slot_floats;
+        up.slot_floats +=
+            (int64_t{up.n_a} * g.k_in + int64_t{n_g[m0 + j]} * g.k_out) * g.tpc * kTileTokens;
+        n_entries += static_cast<size_t>(up.n_a + n_g[m0 + j]) * B * g.n_chunks;
+      }
+      base += up.slot_floats * B * g.n_chunks;
+      n_split += static_cast<int>(cnt * B * g.n_chunks);
+    }
+  }
+  std::stable_sort(batches.begin(), batches.end(),
+                   [](const Batch& x, const Batch& y) { return x.key > y.key; });
+  g.table.reserve(n_entries);
+  for (const Batch& bt : batches) {
+    const UnitPlan& up = ups[bt.unit];
+    const int m0 = g.units[bt.unit].first, cnt = g.units[bt.unit].second;
+    const int j0 = bt.side == 2 ? bt.j : 0, j1 = bt.side == 2 ? bt.j + 1 : cnt;
+    const int li0 = g.layers[m0 + j0];
+    const int ch = bt.side == 2 ? chunks_of(layers[li0].d_out) : chunks_of(layers[li0].d_in);
+    const int n = bt.side == 2 ? n_g[m0 + j0] : up.n_a;
+    const int c0 = bt.side ? static_cast<int>(static_cast<int64_t>(bt.piece) * ch / n) : 0;
+    const int c1 = bt.side ? static_cast<int>(static_cast<int64_t>(bt.piece + 1) * ch / n) : 0;
     for (int64_t b = 0; b < B; ++b) {
       for (int c = 0; c < g.n_chunks; ++c) {
-        const int tiles = std::min(n_tiles, (c + 1) * g.tpc) - c * g.tpc;
-        auto slot_of = [&](int j) {
-          return static_cast<int>((static_cast<int64_t>(m0 + j) * B + b) * g.n_chunks + c);
-        };
-        if (!cut) {
-          for (int j = 0; j < cnt; ++j)
-            es.push_back({WorkItem{slot_of(j), 0, 0, 0, 0, 0, 0, 0, 0}, worst * tiles});
-          continue;
-        }
-        for (int j = 0; j < cnt; ++j) {
-          sid[j] = n_split++;
-          sbase[j] = base;
-          base += (int64_t{n_a} * g.k_in + int64_t{n_g[j]} * g.k_out) * g.tpc * kTileTokens;
-        }
-        for (int q = 0; q < n_a; ++q) {             // A side: the unit's layers together
-          const int c0 = static_cast<int>(static_cast<int64_t>(q) * ca / n_a);
-          const int c1 = static_cast<int>(static_cast<int64_t>(q + 1) * ca / n_a);
-          for (int j = 0; j < cnt; ++j)
-            es.push_back({WorkItem{slot_of(j), 1, c0, c1, sid[j], n_a, n_g[j], q, sbase[j]},
-                          int64_t{c1 - c0} * tiles});
-        }
-        for (int j = 0; j < cnt; ++j) {
-          for (int q = 0; q < n_g[j]; ++q) {
-            const int c0 = static_cast<int>(static_cast<int64_t>(q) * cg[j] / n_g[j]);
-            const int c1 = static_cast<int>(static_cast<int64_t>(q + 1) * cg[j] / n_g[j]);
-            es.push_back({WorkItem{slot_of(j), 2, c0, c1, sid[j], n_a, n_g[j], q, sbase[j]},
-                          int64_t{c1 - c0} * tiles});
-          }
+        if (std::min(n_tiles, (c + 1) * g.tpc) - c * g.tpc != bt.tiles) continue;
+        const int64_t bc = b * g.n_chunks + c;
+        for (int j = j0; j < j1; ++j) {            // A side: the unit's layers together
+          const int slot = static_cast<int>((static_cast<int64_t>(m0 + j) * B + b) * g.n_chunks + c);
+          if (!up.cut)
+            g.table.push_back(WorkItem{slot, 0, 0, 0, 0, 0, 0, 0, 0});
+          else
+            g.table.push_back(WorkItem{slot, bt.side, c0, c1,
+                                       up.sid0 + static_cast<int>(bc * cnt + j), up.n_a,
+                                       n_g[m0 + j], bt.piece,
+                                       up.base0 + bc * up.slot_floats + off[m0 + j]});
         }
       }
     }
   }
-  std::stable_sort(es.begin(), es.end(),
-                   [](const Entry& x, const Entry& y) { return x.key > y.key; });
-  g.table.resize(es.size());
-  for (size_t i = 0; i < es.size(); ++i) g.table[i] = es[i].w;
-  g.n_items = static_cast<int>(es.size());
+  g.n_items = static_cast<int>(g.table.size());
   g.n_split = n_split;
   g.piece_floats = base;
 }
 
 // n_queries > 0 lays out per-token score partials [n_layers, n_queries, B, T]
-// instead of per-item projection partials.
-ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
-                        int64_t n_queries = 0) {
+// instead of per-item projection partials.  `fine` lets small launches be cut
+// more finely, which takes more workspace.
+ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                           int64_t n_queries, bool fine) {
   ProjLayout L;
   L.n_tiles = static_cast<int>((T + kTileTokens - 1) / kTileTokens);
   L.mod_slot.assign(n_layers, 0);
@@ -399,11 +465,20 @@ ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, in
     if (want < 1) want = 1;
     int tpc = static_cast<int>((L.n_tiles + want - 1) / want);
     tpc = (tpc + nt_per_group - 1) / nt_per_group * nt_per_group;
+    if (fine && tpc > 1 && mb * ((L.n_tiles + tpc - 1) / tpc) < 2 * kPlanCTAs) {
+      // few slots of a small launch: one tile each (more P' reads from L2, but
+      // more CTAs at work: 300 tokens of one example had 4 slots)
+      int64_t units_total = 0;
+      for (int li : g.layers)
+        units_total += int64_t{chunks_of(layers[li].d_in) + chunks_of(layers[li].d_out)} *
+                       L.n_tiles * B;
+      if (static_cast<double>(units_total) / kPlanCTAs < kFineSlotUnits) tpc = 1;
+    }
     g.tpc = tpc;
     g.n_chunks = (L.n_tiles + tpc - 1) / tpc;
     g.n_slots = static_cast<int>(mb * g.n_chunks);
     g.n_items = g.n_slots;
-    plan_work(layers, B, L.n_tiles, g, n_queries == 0);
+    plan_work(layers, B, L.n_tiles, g, n_queries == 0, fine);
   }
   size_t off = 0;
   L.mods_off = off;
@@ -452,6 +527,17 @@ ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, in
   return L;
 }
 
+// A finely cut launch may need more workspace than a coarse one; one that would
+// then pass the allocation-free call's static scratch stays coarse, so that
+// the call takes what it always took.
+ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                        int64_t n_queries = 0) {
+  ProjLayout L = plan_project_at(layers, n_layers, B, T, n_queries, true);
+  if (L.total > BERGSON_NOALLOC_SCRATCH_BYTES)
+    L = plan_project_at(layers, n_layers, B, T, n_queries, false);
+  return L;
+}
+
 CUresult encode_act(CUtensorMap* tm, const void* ptr, int64_t d, int64_t T, int64_t B) {
   cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(T),
                         static_cast<cuuint64_t>(B)};
@@ -479,6 +565,7 @@ CUresult encode_2d(CUtensorMap* tm, CUtensorMapDataType dt, const void* ptr, int
 struct ScoreLayout {
   int qt = 1;
   size_t qh_off = 0, heap_off = 0, pace_off = 0, pub_off = 0, total = 0;
+  size_t least = 0;            // without the published scores: a search then takes no bound
 };
 
 ScoreLayout plan_score(int64_t K, int64_t Q, int64_t topk) {
@@ -502,8 +589,9 @@ ScoreLayout plan_score(int64_t K, int64_t Q, int64_t topk) {
           sizeof(unsigned long long) >= pub) {
     L.pub_off = L.heap_off + static_cast<size_t>(kPlanCTAs) * topk * L.qt * kScoreQT *
                                  sizeof(unsigned long long);
+    L.least = L.total;
   } else {
-    L.pub_off = L.total;
+    L.least = L.pub_off = L.total;
     L.total += round_up(pub, 256);
   }
   return L;
@@ -823,7 +911,10 @@ static int run_projection(const bergson_layer* layers, int n_layers, int64_t B, 
     if (B > 0 && out == nullptr) return fail(BERGSON_EINVAL, "out is NULL");
   }
   if (out != nullptr && !aligned(out, 4)) return fail(BERGSON_EALIGN, "out must be 4-byte aligned");
-  const ProjLayout L = plan_project(layers, n_layers, B, T, token ? n_queries : 0);
+  ProjLayout L = plan_project(layers, n_layers, B, T, token ? n_queries : 0);
+  // a workspace that only a coarse cut fits takes that
+  if (ws_bytes < L.total)
+    L = plan_project_at(layers, n_layers, B, T, token ? n_queries : 0, false);
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
   if (ws_bytes < L.total)
@@ -887,23 +978,28 @@ static int run_projection(const bergson_layer* layers, int n_layers, int64_t B, 
   for (const Group& g : L.groups)
     if (!g.table.empty())
       std::memcpy(staging.data() + g.table_off, g.table.data(), sizeof(WorkItem) * g.table.size());
-  cudaError_t e = cudaMemcpyAsync(ws, staging.data(), staging.size(), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return fail_cuda(e, "staging copy");
+  // The records reach the workspace with P' generation (as its kernel's
+  // parameters) when they fit there, by a copy before it otherwise; the
+  // projection kernel is launched as that kernel's dependent and sets itself
+  // up while P' is generated.  The tile flags come from the same kernel.
+  cudaError_t e = cudaSuccess;
   const ModDesc* mods_dev = reinterpret_cast<const ModDesc*>(ws + L.mods_off);
-  const bool need_tiles = T > 0;
-  // Tile flags first, then P' right before the projection kernel, which is
-  // launched as its dependent and sets itself up while P' is generated.
-  uint8_t* tile_valid = nullptr;
-  if (mask != nullptr && need_tiles) {
-    tile_valid = ws + L.tv_off;
-    e = launch_tile_valid(mask, static_cast<int>(B), static_cast<int>(T), L.n_tiles, tile_valid, s);
-    if (e != cudaSuccess) return fail_cuda(e, "tile flag launch");
-  }
-  if (need_tiles) {
-    e = launch_prep(reinterpret_cast<const PrepSeg*>(ws + L.segs_off), 2 * n_layers, max_pairs,
-                    status, s);
-    if (e != cudaSuccess) return fail_cuda(e, "prep launch");
-  }
+  uint8_t* tile_valid = mask != nullptr && T > 0 ? ws + L.tv_off : nullptr;
+  PrepArgs pa;
+  pa.staging = staging.data();
+  pa.staging_bytes = staging.size();
+  pa.segs_off = L.segs_off;
+  pa.ws = ws;
+  pa.n_segs = T > 0 ? 2 * n_layers : 0;
+  pa.max_pairs = max_pairs;
+  pa.mask = T > 0 ? mask : nullptr;
+  pa.tile_valid = tile_valid;
+  pa.B = static_cast<int>(B);
+  pa.T = static_cast<int>(T);
+  pa.n_tiles = L.n_tiles;
+  pa.status = status;
+  e = launch_prep(pa, s);
+  if (e != cudaSuccess) return fail_cuda(e, "prep launch");
   const int sms = sm_count(dg.dev);
   for (size_t gi = 0; gi < L.groups.size(); ++gi) {
     const Group& g = L.groups[gi];
@@ -1099,8 +1195,9 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
   const ScoreLayout L = plan_score(K, Q, topk);
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
-  if (ws_bytes < L.total)
+  if (ws_bytes < L.least)
     return fail(BERGSON_EWORKSPACE, "workspace too small: %zu < %zu bytes", ws_bytes, L.total);
+  const bool room = ws_bytes >= L.total;       // for the published scores (topk < 5)
   if ((st = injected()) != BERGSON_OK) return st;
   if (Q == 0) return BERGSON_OK;
 
@@ -1127,7 +1224,7 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
   const ScoreLaunchPlan P = plan_score_launches(N, Q, topk, ctas, !update);
   if (P.launches.empty()) return fail(BERGSON_ECUDA, "no two-SM cluster fits the score kernel");
   uint16_t* pub = reinterpret_cast<uint16_t*>(ws + L.pub_off);
-  const int pub_words = std::min(P.ctas, kPlanCTAs) * L.qt * kScoreQT;
+  const int pub_words = room ? std::min(P.ctas, kPlanCTAs) * L.qt * kScoreQT : 0;
   cudaError_t e = launch_normalize_queries(queries, static_cast<int>(Q), static_cast<int>(K), ld_q,
                                            least, qh, pub, pub_words, s);
   if (e != cudaSuccess) return fail_cuda(e, "query normalisation launch");
@@ -1157,7 +1254,7 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
       if (r != CUDA_SUCCESS) return fail(BERGSON_ECUDA, "tensor map encoding failed (%d)", (int)r);
     }
     score_bound_rule(l.rows, p.bn, cpg, static_cast<int>(topk), &p.bound_j, &p.bound_r);
-    if (grid > kPlanCTAs) p.bound_j = p.bound_r = 0;      // no room for their words
+    if (grid > kPlanCTAs || !room) p.bound_j = p.bound_r = 0;   // no room for their words
     p.stages = p.q_rows = 0;
     p.heaps = heaps;
     p.pub = pub;
@@ -1255,7 +1352,7 @@ int bergson_score_topk_host(const void* host_store, int64_t N, int64_t K, int64_
   if (Q > 0 && (queries == nullptr || out_scores == nullptr || out_idx == nullptr))
     return fail(BERGSON_EINVAL, "queries, out_scores or out_idx is NULL");
   const size_t chunk_bytes = host_chunk_bytes(chunk_rows, K);
-  const size_t need = 2 * chunk_bytes + plan_score(K, Q, topk).total;
+  const size_t need = 2 * chunk_bytes + plan_score(K, Q, topk).least;
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
   if (ws_bytes < need)

@@ -177,13 +177,23 @@ int record_error(int code, const char* fmt, ...);
 
 // ---- launchers (return the launch error, if any) ----
 
+// P' generation, the host-built records and the tile flags of a projection call.
+struct PrepArgs {
+  const uint8_t* staging;     // host: module descriptors, PrepSegs, zeroed counters, work table
+  size_t staging_bytes;       // (a multiple of 16) -> ws[0, staging_bytes)
+  size_t segs_off;            // offset of the PrepSegs in staging
+  uint8_t* ws;
+  int n_segs;                 // 0: no P'
+  int64_t max_pairs;          // largest segment, entry pairs
+  const uint8_t* mask;        // [B, T], or nullptr: no tile flags
+  uint8_t* tile_valid;        // [B, n_tiles]
+  int B, T, n_tiles;
+  int* status;
+};
 // Both record BERGSON_EMOMENT in *status when a second-moment entry is not > 0.
-cudaError_t launch_prep(const PrepSeg* segs, int n_segs, int64_t max_pairs, int* status,
-                        cudaStream_t s);
+cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s);
 cudaError_t launch_projection_matrix(uint64_t seed, int d, int k, int kind, const float* moment,
                                      int* status, float* out, cudaStream_t s);
-cudaError_t launch_tile_valid(const uint8_t* mask, int B, int T, int n_tiles, uint8_t* tile_valid,
-                              cudaStream_t s);
 cudaError_t launch_wait_probe(int* status, uint64_t timeout_ns, cudaStream_t s);
 
 // token = false: per-example projected gradients (partials); token = true:

@@ -17,6 +17,9 @@
 // into two bf16 terms hi + lo, so A and G (exact bf16) meet a projection that
 // is accurate to ~2^-16 relative instead of bf16's 2^-8.
 
+#include <algorithm>
+#include <cstring>
+
 #include "bergson.h"
 #include "internal.h"
 #include "ptx.cuh"
@@ -111,12 +114,10 @@ __device__ __forceinline__ void prep_pair(const PrepSeg& sg, int i, int j, int* 
   store_hi_lo(sg.dst, (j + 1) * d + i, (sg.k + j + 1) * d + i, v1);
 }
 
-// blockIdx.y = segment; threads walk the segment's d*k/2 entry pairs with the
-// input index i fastest, so the transposed bf16 stores are coalesced.  The
-// index arithmetic is 32-bit when the segment allows it (the common case).
-__global__ void prep_kernel(const PrepSeg* __restrict__ segs, int* status) {
-  griddep_launch_dependents();   // the projection kernel may set itself up meanwhile
-  const PrepSeg sg = segs[blockIdx.y];
+// Threads walk a segment's d*k/2 entry pairs with the input index i fastest, so
+// the transposed bf16 stores are coalesced.  The index arithmetic is 32-bit
+// when the segment allows it (the common case).
+__device__ __forceinline__ void prep_segment(const PrepSeg& sg, int* status) {
   const int64_t npairs = static_cast<int64_t>(sg.d) * sg.k / 2;
   if (npairs <= 0x7fffffff) {
     const uint32_t n = static_cast<uint32_t>(npairs), d = static_cast<uint32_t>(sg.d);
@@ -126,6 +127,68 @@ __global__ void prep_kernel(const PrepSeg* __restrict__ segs, int* status) {
     for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < npairs;
          q += static_cast<int64_t>(gridDim.x) * blockDim.x)
       prep_pair(sg, static_cast<int>(q % sg.d), 2 * static_cast<int>(q / sg.d), status);
+  }
+}
+
+// tile_valid[b, t] bit q (q = 0..3) = 1 if any token of the 32-token slice
+// [128 t + 32 q, 128 t + 32 q + 32) of example b is valid.  One warp per tile.
+__device__ __forceinline__ void tile_flags(const uint8_t* __restrict__ mask, int B, int T,
+                                           int n_tiles, uint8_t* __restrict__ tile_valid) {
+  const int lane = threadIdx.x & 31;
+  const int n_warps = static_cast<int>(gridDim.x * blockDim.x) >> 5;
+  for (int64_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+       w < static_cast<int64_t>(B) * n_tiles; w += n_warps) {
+    const int64_t b = w / n_tiles;
+    const int t0 = static_cast<int>(w % n_tiles) * kTileTokens;
+    uint32_t bits = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = t0 + 32 * q + lane;
+      const int v = t < T && mask[b * T + t] != 0;
+      if (__any_sync(0xffffffffu, v)) bits |= 1u << q;
+    }
+    if (lane == 0) tile_valid[w] = static_cast<uint8_t>(bits);
+  }
+}
+
+// One launch before the projection kernel: blockIdx.y < n_segs generates that
+// segment's P', row n_segs the tile flags, and (when the host-built records
+// came as parameters, kBytes > 0) row n_segs + 1 writes them to the workspace.
+// A copy and a launch less than separate steps: 4 us of host time and 4 us of
+// device time per call on small batches.
+struct PrepCommon {
+  const uint8_t* mask;
+  uint8_t* tile_valid;
+  uint8_t* ws;
+  int64_t segs_off;
+  int B, T, n_tiles, n_segs;
+  int bytes;                   // of the records, a multiple of 16
+  int* status;
+};
+template <int kBytes>
+struct PrepParams : PrepCommon {
+  alignas(16) uint8_t staging[kBytes];
+};
+template <>
+struct PrepParams<0> : PrepCommon {};
+
+template <int kBytes>
+__global__ void prep_kernel(const __grid_constant__ PrepParams<kBytes> p) {
+  griddep_launch_dependents();   // the projection kernel may set itself up meanwhile
+  const int y = blockIdx.y;
+  if (y < p.n_segs) {
+    const uint8_t* base;
+    if constexpr (kBytes > 0) base = p.staging;
+    else base = p.ws;
+    const PrepSeg sg = reinterpret_cast<const PrepSeg*>(base + p.segs_off)[y];
+    prep_segment(sg, p.status);
+  } else if (y == p.n_segs) {
+    if (p.tile_valid != nullptr) tile_flags(p.mask, p.B, p.T, p.n_tiles, p.tile_valid);
+  } else if constexpr (kBytes > 0) {
+    const uint4* src = reinterpret_cast<const uint4*>(p.staging);
+    uint4* dst = reinterpret_cast<uint4*>(p.ws);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.bytes / 16; i += gridDim.x * blockDim.x)
+      dst[i] = src[i];
   }
 }
 
@@ -144,25 +207,6 @@ __global__ void projection_matrix_kernel(uint64_t seed, int d, int k, int kind,
   }
 }
 
-// tile_valid[b, t] bit q (q = 0..3) = 1 if any token of the 32-token slice
-// [128 t + 32 q, 128 t + 32 q + 32) of example b is valid.  One warp per tile.
-__global__ void tile_valid_kernel(const uint8_t* __restrict__ mask, int B, int T, int n_tiles,
-                                  uint8_t* __restrict__ tile_valid) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= B * n_tiles) return;
-  const int b = warp / n_tiles;
-  const int t0 = (warp % n_tiles) * kTileTokens;
-  uint32_t bits = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int t = t0 + 32 * q + lane;
-    const int v = t < T && mask[static_cast<int64_t>(b) * T + t] != 0;
-    if (__any_sync(0xffffffffu, v)) bits |= 1u << q;
-  }
-  if (lane == 0) tile_valid[warp] = static_cast<uint8_t>(bits);
-}
-
 // Waits on an mbarrier that nothing completes; exercises the timeout path.
 __global__ void wait_probe_kernel(int* status, uint64_t timeout_ns) {
   __shared__ __align__(8) uint64_t bar;
@@ -176,15 +220,48 @@ __global__ void wait_probe_kernel(int* status, uint64_t timeout_ns) {
   }
 }
 
-cudaError_t launch_prep(const PrepSeg* segs, int n_segs, int64_t max_pairs, int* status,
-                        cudaStream_t s) {
-  if (n_segs <= 0 || max_pairs <= 0) return cudaSuccess;
+namespace {
+
+template <int kBytes>
+cudaError_t launch_prep_t(const PrepArgs& a, cudaStream_t s) {
+  static thread_local PrepParams<kBytes> p;      // up to 28 KB: kept off the stack
+  p.mask = a.mask;
+  p.tile_valid = a.tile_valid;
+  p.ws = a.ws;
+  p.segs_off = static_cast<int64_t>(a.segs_off);
+  p.B = a.B;
+  p.T = a.T;
+  p.n_tiles = a.n_tiles;
+  p.n_segs = a.n_segs;
+  p.bytes = static_cast<int>(a.staging_bytes);
+  p.status = a.status;
+  if constexpr (kBytes > 0) std::memcpy(p.staging, a.staging, a.staging_bytes);
   const int threads = 256;
-  int64_t bx = (max_pairs + 4 * threads - 1) / (4 * threads);   // ~4 pairs per thread
-  if (bx > 4096) bx = 4096;
-  prep_kernel<<<dim3(static_cast<unsigned>(bx), static_cast<unsigned>(n_segs)), threads, 0, s>>>(
-      segs, status);
+  // ~4 pairs per thread, and enough CTAs for the flags (8 tiles each)
+  int64_t bx = (a.max_pairs + 4 * threads - 1) / (4 * threads);
+  if (a.tile_valid != nullptr)
+    bx = std::max<int64_t>(bx, std::min<int64_t>(
+                                   512, (static_cast<int64_t>(a.B) * a.n_tiles * 32 + threads - 1) /
+                                            threads));
+  bx = std::max<int64_t>(1, std::min<int64_t>(bx, 4096));
+  const int rows = a.n_segs + 1 + (kBytes > 0 ? 1 : 0);
+  prep_kernel<kBytes><<<dim3(static_cast<unsigned>(bx), static_cast<unsigned>(rows)), threads, 0,
+                        s>>>(p);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+// The records travel as kernel parameters up to 28 KB (a block or two of
+// modules); a parameter costs the host its copy, so small calls use a small one.
+cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
+  if (a.staging_bytes <= 4096) return launch_prep_t<4096>(a, s);
+  if (a.staging_bytes <= 28672) return launch_prep_t<28672>(a, s);
+  const cudaError_t e =
+      cudaMemcpyAsync(a.ws, a.staging, a.staging_bytes, cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  if (a.n_segs == 0 && a.tile_valid == nullptr) return cudaSuccess;
+  return launch_prep_t<0>(a, s);
 }
 
 cudaError_t launch_projection_matrix(uint64_t seed, int d, int k, int kind, const float* moment,
@@ -194,17 +271,6 @@ cudaError_t launch_projection_matrix(uint64_t seed, int d, int k, int kind, cons
   const int64_t blocks = (npairs + threads - 1) / threads;
   projection_matrix_kernel<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), threads, 0,
                              s>>>(seed, d, k, kind, moment, status, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tile_valid(const uint8_t* mask, int B, int T, int n_tiles, uint8_t* tile_valid,
-                              cudaStream_t s) {
-  const int64_t warps = static_cast<int64_t>(B) * n_tiles;
-  if (warps == 0) return cudaSuccess;
-  const int threads = 256;
-  const int64_t blocks = (warps * 32 + threads - 1) / threads;
-  tile_valid_kernel<<<static_cast<unsigned>(blocks), threads, 0, s>>>(mask, B, T, n_tiles,
-                                                                      tile_valid);
   return cudaGetLastError();
 }
 
