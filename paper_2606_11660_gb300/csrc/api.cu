@@ -260,7 +260,7 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bo
   if (!split && !shared) return;
   // Tiles of a slot (the last slot of an example may have fewer).
   const int slot_tiles = std::min(g.tpc, n_tiles);
-  const double target = std::max(share / kPiecesPerShare, kMinPieceUnits);
+  double target = std::max(share / kPiecesPerShare, kMinPieceUnits);
   // A piece stores and its slot's finisher reloads 4k fp32 bytes per token,
   // against 128 bytes per token and chunk streamed: pieces of at least 2k
   // chunks keep that under 1/32 of the piece's traffic.  (Fewer, larger
@@ -289,6 +289,22 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bo
     if (worst > std::max(kFinePieceShare * share, kMinPieceUnits)) {
       min_a = 3 * g.k_in / 8;
       min_g = 3 * g.k_out / 8;
+      // Rounding leaves a few pieces more than two a CTA, and a third round for
+      // them (a Llama-8B-shaped block of 512 tokens: 328 items, 24 CTAs busy 10
+      // us longer): slightly larger pieces fit two rounds.
+      const double least = target;
+      bool fits = false;
+      for (double f = 1.0; f < 1.45 && !fits; f += 0.1) {
+        target = f * least;
+        int64_t items = 0;
+        for (int li : g.layers) {
+          const int ca = chunks_of(layers[li].d_in), cg = chunks_of(layers[li].d_out);
+          const bool cut = static_cast<double>(ca + cg) * slot_tiles > share / kPiecesPerShare;
+          items += (cut ? pieces(ca, min_a) + pieces(cg, min_g) : 1) * B * g.n_chunks;
+        }
+        fits = items <= kPiecesPerShare * kPlanCTAs;
+      }
+      if (!fits) target = least;
     }
   }
   // Groups of entries of one cost: a unit's fused items, or one of its pieces,
