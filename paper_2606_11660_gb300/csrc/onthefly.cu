@@ -201,8 +201,12 @@ __device__ __forceinline__ XItem decode_xitem(const XGemmParams& p, int item) {
 // segments of a tile are its K slices; a segment's partial plane is its
 // cluster's rank among the clusters that meet the tile.  The cluster that
 // holds position g: ceil((g + 1) n / W) - 1.
+// (A 64-bit division is a couple of hundred instructions; the usual sizes fit 32.)
 __host__ __device__ __forceinline__ int seg_cluster_of(int64_t g, int64_t W, int n) {
-  return static_cast<int>(((g + 1) * n + W - 1) / W) - 1;
+  const int64_t a = (g + 1) * n + W - 1;
+  if (a < (int64_t{1} << 32))
+    return static_cast<int>(static_cast<uint32_t>(a) / static_cast<uint32_t>(W)) - 1;
+  return static_cast<int>(a / W) - 1;
 }
 __host__ __device__ __forceinline__ int seg_planes(int mt, int steps, int64_t W, int n) {
   const int64_t p0 = static_cast<int64_t>(mt) * steps;
@@ -218,16 +222,24 @@ struct SegIter {
     n = p.n_clusters;
     cid = c;
     W = static_cast<int64_t>(p.n_mtiles) * steps;
-    g = c * W / n;
-    g1 = (c + 1) * W / n;
+    const int64_t a = static_cast<int64_t>(c + 1) * W;
+    if (a < (int64_t{1} << 32)) {
+      g = static_cast<uint32_t>(c * W) / static_cast<uint32_t>(n);
+      g1 = static_cast<uint32_t>(a) / static_cast<uint32_t>(n);
+    } else {
+      g = c * W / n;
+      g1 = a / n;
+    }
     load();
   }
   __device__ __forceinline__ bool valid() const { return g < g1; }
   __device__ __forceinline__ void load() {
     if (g >= g1) return;
-    it.mt = static_cast<int>(g / steps);
+    it.mt = g < (int64_t{1} << 32)
+                ? static_cast<int>(static_cast<uint32_t>(g) / static_cast<uint32_t>(steps))
+                : static_cast<int>(g / steps);
     it.nt = 0;
-    it.s0 = static_cast<int>(g % steps);
+    it.s0 = static_cast<int>(g - static_cast<int64_t>(it.mt) * steps);
     const int64_t end = it.s0 + (g1 - g);
     it.s1 = end < steps ? static_cast<int>(end) : steps;
     it.z = cid - seg_cluster_of(static_cast<int64_t>(it.mt) * steps, W, n);
@@ -570,6 +582,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
+  // widest batch tile of this instantiation: unrolled code for no more columns
+  constexpr int kPad = kTwo ? 32 : kMaxPadN;
   const uint32_t sbase = smem_u32(smem);
   const int xbytes = p.n_pad * 128;
   // this CTA's y half, its half of B = [x_hi; x_lo], and with two issuers its
@@ -789,9 +803,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       const int q = it.mt * 2 * kXM + static_cast<int>(rank) * kXM + row;
       const int L = it.s1 - it.s0;
       const int n_ch = chain_count(L, p.sub);
-      float acc[kMaxPadN];          // 0 + v = v: the first chain lands unchanged
+      float acc[kPad];          // 0 + v = v: the first chain lands unchanged
 #pragma unroll
-      for (int j = 0; j < kMaxPadN; ++j) acc[j] = 0.0f;
+      for (int j = 0; j < kPad; ++j) acc[j] = 0.0f;
       for (int k = 0; k < n_ch; ++k) {
         if (!warp_wait(smem_u32(&tfull[ab]), aph, tmo, s_abort)) {
           raise_device_error(p.status, s_abort, kStatusTimeout);
@@ -801,7 +815,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
         tc_fence_after();
         const uint32_t tbase = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + ab * set_cols;
 #pragma unroll
-        for (int cb = 0; cb < kMaxPadN / 16; ++cb) {
+        for (int cb = 0; cb < kPad / 16; ++cb) {
           const int c = 16 * cb;
           if (c < p.n_pad) {
             // <x_b, y_q> ~= (y_hi + y_lo) x_hi + (y_hi + y_lo) x_lo; with two
@@ -830,7 +844,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       if (q < p.Q) {
         float* dst = p.partial + static_cast<int64_t>(it.z) * p.B * p.Q + q;
 #pragma unroll
-        for (int cb = 0; cb < kMaxPadN / 16; ++cb) {
+        for (int cb = 0; cb < kPad / 16; ++cb) {
           const int c = 16 * cb;
           if (c < p.n_pad) {
 #pragma unroll
@@ -857,33 +871,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // = s / sqrt(nx_b) / sqrt(ny_q), nx_b the sum over the row's chunks (in
 // order) of xnorm[b, c], ny_q the sum over the same planes of ynorm[z, q] (0
 // when either row is zero).  Otherwise scores[b, q] = s.
-__global__ void finish_kernel(const float* __restrict__ partial, int S, int B, int Q,
-                              const float* __restrict__ xnorm, int n_chunks,
-                              const float* __restrict__ ynorm, int seg_clusters, int steps,
-                              int y_rows, float* scores, int64_t ld) {
-  griddep_wait();                 // partials and norms come from earlier grids
+//
+// The planes' loads are issued kFinishBatch at a time before they are added in
+// order (one after another, the 20 planes and 20 norms of a 1024-query call were
+// 7 us of L2 latency), and a thread keeps its column's norm for all its rows.
+constexpr int kFinishBatch = 8;
+struct PlaneSum {                 // a sum over n planes, its first batch in flight
+  const float* src;
+  int64_t stride;
+  int n;
+  float v[kFinishBatch];
+  __device__ __forceinline__ void start(const float* src_, int64_t stride_, int n_) {
+    src = src_;
+    stride = stride_;
+    n = n_;
+    load(0);
+  }
+  __device__ __forceinline__ void load(int z0) {
+#pragma unroll
+    for (int z = 0; z < kFinishBatch; ++z)
+      if (z0 + z < n) v[z] = __ldcg(src + (z0 + z) * stride);
+  }
+  __device__ __forceinline__ float finish() {
+    float s = 0.0f;
+    for (int z0 = 0;;) {
+#pragma unroll
+      for (int z = 0; z < kFinishBatch; ++z)
+        if (z0 + z < n) s += v[z];
+      z0 += kFinishBatch;
+      if (z0 >= n) return s;
+      load(z0);
+    }
+  }
+};
+
+__global__ void __launch_bounds__(256) finish_kernel(const float* partial, int S, int B, int Q,
+                                                     const float* xnorm, int n_chunks,
+                                                     const float* ynorm, int seg_clusters,
+                                                     int steps, int y_rows, float* scores,
+                                                     int64_t ld) {
   const int64_t n = static_cast<int64_t>(B) * Q;
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;     // grid: (Q / 256, rows of b)
-  if (q >= Q) return;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;     // grid: (Q / 256, groups of b)
   // planes of this row's y tile: all S, or on pairs the tile's segments
   const int n_mtiles = (Q + y_rows - 1) / y_rows;
   const int planes = seg_clusters > 0 ? seg_planes(q / y_rows, steps,
                                                    static_cast<int64_t>(n_mtiles) * steps,
                                                    seg_clusters)
                                       : S;
+  griddep_wait();                 // partials and norms come from earlier grids
+  if (q >= Q) return;
+  float iy = 0.0f;
+  bool first = true;
   for (int b = blockIdx.y; b < B; b += gridDim.y) {
-    const int64_t i = static_cast<int64_t>(b) * Q + q;
-    float s = 0.0f;
-    for (int z = 0; z < planes; ++z) s += partial[z * n + i];
+    PlaneSum sum, sx, sy;
+    sum.start(partial + static_cast<int64_t>(b) * Q + q, n, planes);
     float* dst = scores + b * ld + q;
-    if (xnorm != nullptr) {
-      float nx = 0.0f, ny = 0.0f;
-      for (int c = 0; c < n_chunks; ++c) nx += xnorm[static_cast<int64_t>(b) * n_chunks + c];
-      for (int z = 0; z < planes; ++z) ny += ynorm[static_cast<int64_t>(z) * Q + q];
-      *dst = nx > 0.0f && ny > 0.0f ? s * (1.0f / sqrtf(nx)) * (1.0f / sqrtf(ny)) : 0.0f;
-    } else {
-      *dst = s;
+    if (xnorm == nullptr) {
+      *dst = sum.finish();
+      continue;
     }
+    sx.start(xnorm + static_cast<int64_t>(b) * n_chunks, 1, n_chunks);
+    if (first) {
+      sy.start(ynorm + q, Q, planes);
+      const float ny = sy.finish();
+      iy = ny > 0.0f ? 1.0f / sqrtf(ny) : 0.0f;
+      first = false;
+    }
+    const float nx = sx.finish(), s = sum.finish();
+    *dst = nx > 0.0f && iy > 0.0f ? s * (1.0f / sqrtf(nx)) * iy : 0.0f;
   }
 }
 
@@ -1056,7 +1111,9 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s) {
   }
   if (e != cudaSuccess) return e;
 
-  const dim3 fgrid((a.Q + 255) / 256, std::min(a.B, 65535));
+  // as many row groups as fill the SMs a few times over
+  const int fx = (a.Q + 255) / 256;
+  const dim3 fgrid(fx, std::max(1, std::min({a.B, 65535, (8 * kPlanCTAs + fx - 1) / fx})));
   const float* xn = a.unit ? xnorm : nullptr;
   return launch_dependent(finish_kernel, fgrid, dim3(256), 0, s, p.partial, pl.S, a.B, a.Q, xn,
                           pl.n_chunks, p.ynorm, pl.pair ? pl.n_clusters : 0, pl.steps, pl.y_rows,
