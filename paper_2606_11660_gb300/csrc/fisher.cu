@@ -21,9 +21,10 @@
 //
 // Measured (one GB300, n = 1024, 12 updates at K = 3072): 17.4 ms per fit and
 // power with tf32 parts on single CTAs, K slices through partial sums in
-// memory and separate transpose / symmetrise / norm passes; 5.6 ms as here.
-// Per update: 42 / 63 / 420 us at K = 256 / 1024 / 3072 (58 / 97 / 425 us with a
-// launch for every product and pass and T split by a pass of its own).
+// memory and separate transpose / symmetrise / norm passes; 5.4 ms as here.
+// Per update: 34 / 51 / 395 us at K = 256 / 1024 / 3072 (58 / 97 / 425 us with a
+// launch for every product and pass and T split by a pass of its own, entry by
+// entry).
 
 #include <algorithm>
 
