@@ -339,7 +339,9 @@ BERGSON_API int bergson_token_scores_workspace(const bergson_layer* layers, int 
  *            (64, 64), which stay on the CUDA cores.
  *   out      fp32 [n_queries, B, T] contiguous.
  * The workspace holds per-module partial scores (n_layers x n_queries x B x
- * T floats) that a final pass sums in module order.
+ * T floats) that a final pass sums in module order and, where a few wide
+ * layers would keep most of the GPU waiting, the token projections of their
+ * pieces (a workspace without room for these is served without pieces).
  * Other arguments as for bergson_project_grads.  Deterministic.
  * Errors: EINVAL, EALIGN, EUNSUPPORTED, EWORKSPACE, ECUDA.
  */

@@ -32,6 +32,16 @@ constexpr int kPiecesPerShare = 2;
 constexpr double kMinPieceUnits = 4.0;               // ... of at least 4 chunks of a tile
 constexpr double kFinePieceShare = 0.8;              // largest piece, in shares, before the minimum
                                                      // piece size is lowered
+// Token scores: pieces cost their slot's last one some 17 us (sums, query
+// blocks behind them) and 0.16 us a query, and save 0.35 us per unit by which
+// the largest slot exceeds a share.  With and without, us a call: a
+// Llama-8B-shaped block of 2 x 1024 tokens (excess 153) 69 / 106 with 1 query, 95
+// / 117 with 100; 1 x 300 tokens of it (263) 38 / 105; a 1.4B block of 5 x 700
+// (59, 64 queries) 93 / 78; 12 Pythia-160M modules, 3 x 200 (37, 40 queries)
+// 60 / 47.
+constexpr double kTokenSplitUnits = 64.0;
+constexpr double kTokenSplitPerQuery = 0.75;
+constexpr int kTokenSlotsPerCTA = 16;
 constexpr int kFineMaxK = 96;                        // k_in + k_out up to which it is
 constexpr double kFineSlotUnits = 64.0;              // shares below this (and few slots): slots of
                                                      // one tile each
@@ -240,12 +250,12 @@ int chunks_of(int64_t d) { return static_cast<int>((d + kChunk - 1) / kChunk); }
 // Builds a group's work table when its slots need more than "item i is slot i":
 // (1) cutting: when the launch is too coarse for the SMs to finish together
 // (largest slot above kSplitShare of one CTA's share), large slots are cut
-// into pieces (split = allowed only in projection mode); (2) shared inputs:
+// into pieces (token scores: see kTokenSplitUnits); (2) shared inputs:
 // the items of a unit's layers for the same example and tiles are listed next
 // to each other (A-side pieces too), so the scheduler starts them together.
 // Cost unit: one 64-column chunk of one tile; the table runs largest first.
-void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bool allow_split,
-               bool fine) {
+void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, int64_t n_queries,
+               bool token_split, bool fine) {
   if (g.n_slots == 0) return;
   int64_t total = 0, max_slot = 0;
   for (int li : g.layers) {
@@ -254,7 +264,10 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, bo
     max_slot = std::max<int64_t>(max_slot, c * std::min(g.tpc, n_tiles));
   }
   const double share = static_cast<double>(total) / kPlanCTAs;
-  const bool split = allow_split && static_cast<double>(max_slot) > kSplitShare * share;
+  const double excess = static_cast<double>(max_slot) - share;
+  const bool split = n_queries == 0 ? static_cast<double>(max_slot) > kSplitShare * share
+                                    : token_split && excess > kTokenSplitUnits +
+                                                                  kTokenSplitPerQuery * n_queries;
   bool shared = false;
   for (const auto& u : g.units) shared = shared || u.second > 1;
   if (!split && !shared) return;
@@ -467,6 +480,7 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
     }
     g.first_mod = slot;
     for (int li : g.layers) L.mod_slot[li] = slot++;
+    const bool token_tc = n_queries > 0 && fine && token_tc_queries(g.k_in, g.k_out) > 0;
     const int nt_per_group = (g.k_in + g.k_out <= 32) ? 4 : ((g.k_in + g.k_out <= 64) ? 2 : 1);
     const int64_t mb = static_cast<int64_t>(g.layers.size()) * B;
     if (L.n_tiles == 0 || mb == 0) {
@@ -490,11 +504,20 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
                        L.n_tiles * B;
       if (static_cast<double>(units_total) / kPlanCTAs < kFineSlotUnits) tpc = 1;
     }
+    // Token scores on the tensor cores take one tile at a time whatever the slot,
+    // so small slots cost an item's first query block each and even out the
+    // launch (as for collections / at most 4 / 16 slots a CTA, us a call): a
+    // Llama-8B-shaped block of 4 x 2048 tokens 385 / 222 / 222, of 8 x 4096 804 /
+    // 728 / 723; 16 Pythia-160M modules of 4 x 512 103 / 59 / 59, 48 of 8 x 2048
+    // 786 / 785 / 777 (789 with one-tile slots).
+    while (token_tc && tpc > 1 &&
+           mb * ((L.n_tiles + tpc - 1) / tpc) < kTokenSlotsPerCTA * kPlanCTAs)
+      tpc /= 2;
     g.tpc = tpc;
     g.n_chunks = (L.n_tiles + tpc - 1) / tpc;
     g.n_slots = static_cast<int>(mb * g.n_chunks);
     g.n_items = g.n_slots;
-    plan_work(layers, B, L.n_tiles, g, n_queries == 0, fine);
+    plan_work(layers, B, L.n_tiles, g, n_queries, token_tc, fine);
   }
   size_t off = 0;
   L.mods_off = off;
@@ -533,11 +556,12 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
         g.bias_off = off;
         off += round_up(static_cast<size_t>(g.n_slots) * kTileTokens * sizeof(float), 256);
       }
-      if (g.piece_floats > 0) {
-        g.piece_off = off;
-        off += round_up(static_cast<size_t>(g.piece_floats) * sizeof(float), 256);
-      }
     }
+  }
+  for (Group& g : L.groups) {
+    if (g.piece_floats == 0) continue;
+    g.piece_off = off;
+    off += round_up(static_cast<size_t>(g.piece_floats) * sizeof(float), 256);
   }
   L.total = off;
   return L;
@@ -549,7 +573,7 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
 ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
                         int64_t n_queries = 0) {
   ProjLayout L = plan_project_at(layers, n_layers, B, T, n_queries, true);
-  if (L.total > BERGSON_NOALLOC_SCRATCH_BYTES)
+  if (n_queries == 0 && L.total > BERGSON_NOALLOC_SCRATCH_BYTES)
     L = plan_project_at(layers, n_layers, B, T, n_queries, false);
   return L;
 }

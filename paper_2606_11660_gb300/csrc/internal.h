@@ -79,6 +79,17 @@ constexpr int kScoreMaxJ = 32;       // best first-tile scores a score epilogue 
 constexpr uint64_t kWaitTimeoutNs = 4000000000ull;   // bounded device waits: 4 s
 constexpr int kPlanCTAs = 152;   // persistent CTAs work planners assume (one per SM of this part)
 
+// Queries per block of token mode on the tensor cores (0: the (k_in, k_out)
+// does not fit and takes the CUDA cores).  TMEM, with one tile per group: the
+// two projection buffers (4 (k_in + k_out) columns), a~ hi / lo (2 k_in) and U
+// (k_out a query, at most 256).
+constexpr int token_tc_queries(int k_in, int k_out) {
+  const int avail = 512 - 4 * (k_in + k_out) - 2 * k_in;
+  const int cols = avail < 256 ? avail : 256;
+  const int q = cols > 0 ? cols / k_out : 0;
+  return q < 16 ? q : 16;
+}
+
 // Per-module launch record kept in workspace (global memory).  The tensor maps
 // are read by TMA straight from there, so the record is 64-byte aligned.
 struct ModDesc {
@@ -200,9 +211,6 @@ cudaError_t launch_wait_probe(int* status, uint64_t timeout_ns, cudaStream_t s);
 // per-token scores against p.queries (token_partials).
 cudaError_t launch_project(int k_in, int k_out, bool token, const ProjParams& p, int grid,
                           cudaStream_t s);
-// Queries whose blocks token mode holds in shared memory at once (more are
-// streamed through in blocks of this many).
-int token_query_capacity(int k_in, int k_out);
 cudaError_t launch_token_reduce(const float* token_partials, int n_mods, int Q, int B, int T,
                                 const uint8_t* mask, float* out, cudaStream_t s);
 cudaError_t launch_reduce(const ModDesc* mods, int n_mods, int k_in, int k_out, int B,

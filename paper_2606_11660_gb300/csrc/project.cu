@@ -54,10 +54,7 @@ struct ProjCfg {
   // cores (k_out FMAs per token and query instead of k_out (k_in + 1)).
   // TMEM with one tile per group: the two projection buffers (4 (k_in + k_out)
   // columns), a~ hi / lo (2 k_in) and U (kTcN <= 256) must fit in 512 columns.
-  static constexpr int kTcAvail = 512 - 4 * (KI + KO) - 2 * KI;
-  static constexpr int kTcNQa = kTcAvail > 0 ? kTcAvail / KO : 0;
-  static constexpr int kTcNQb = kTcNQa < 256 / KO ? kTcNQa : 256 / KO;
-  static constexpr int kTcNQ = kTcNQb < 16 ? kTcNQb : 16;
+  static constexpr int kTcNQ = token_tc_queries(KI, KO);
   static constexpr bool kTC = TOKEN && kTcNQ >= 1;
   static constexpr int kTcN = kTcNQ * KO;
   static constexpr int kTcAtoms = (KI + 31) / 32;              // 128-byte K atoms of a B row
@@ -275,8 +272,15 @@ __device__ __forceinline__ void tmem_store_row(uint32_t taddr, const float* v) {
   }
 }
 
-template <int KI, int KO, bool TOKEN>
+// Modes of the kernel.  Token scores without pieces are a mode of their own: the
+// same code with the pieces' branches in it runs 2 to 20% slower (48 modules,
+// 8 x 2048 tokens, 64 queries 784 -> 801 us; 4 x 2047 tokens, 200 queries 729 ->
+// 883 us: all 255 registers in use, the query blocks' loads issued later).
+constexpr int kModeProject = 0, kModeToken = 1, kModeTokenPieces = 2;
+template <int KI, int KO, int MODE>
 __global__ void __launch_bounds__(192, 1) project_kernel(const ProjParams p) {
+  constexpr bool TOKEN = MODE != kModeProject;
+  constexpr bool kPieces = MODE != kModeToken;
   using C = ProjCfg<KI, KO, TOKEN>;
   constexpr int NT = C::NT;
   extern __shared__ uint8_t smem_raw[];
@@ -501,7 +505,7 @@ __global__ void __launch_bounds__(192, 1) project_kernel(const ProjParams p) {
       bool finisher = false;       // last piece of its slot: contracts the summed pieces
       const int64_t stride_a = static_cast<int64_t>(p.tpc) * kTileTokens * KI;
       const int64_t stride_g = static_cast<int64_t>(p.tpc) * kTileTokens * KO;
-      if constexpr (!TOKEN) {
+      if constexpr (kPieces) {
         if (ic.side != 0) {
           // A piece: store this side's token projections of the slot's tiles.
           float* dst = p.piece_buf + ic.base +
@@ -593,7 +597,12 @@ __global__ void __launch_bounds__(192, 1) project_kernel(const ProjParams p) {
           const uint32_t lane_base = static_cast<uint32_t>(32 * quarter) << 16;
           float va[KI];
           float vg[KO];
-          {
+          if (kPieces && finisher) {
+            const int64_t tok = static_cast<int64_t>(g - ic.t_begin) * kTileTokens + row;
+            sum_token_rows<KI>(p.piece_buf + ic.base + tok * KI, stride_a, ic.n_a, va);
+            sum_token_rows<KO>(p.piece_buf + ic.base + ic.n_a * stride_a + tok * KO, stride_g,
+                               ic.n_g, vg);
+          } else {
             const uint32_t taddr = tmem + lane_base + ab * C::kTmemPerBuf;
             tmem_ld_hilo<KI>(taddr, va);
             tmem_ld_hilo<KO>(taddr + 2 * KI, vg);
@@ -610,9 +619,11 @@ __global__ void __launch_bounds__(192, 1) project_kernel(const ProjParams p) {
           }
           tmem_st_wait();
           tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&tempty[ab]));
-          if (++ab == 2) { ab = 0; aph ^= 1; }
+          if (!kPieces || !finisher) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tempty[ab]));
+            if (++ab == 2) { ab = 0; aph ^= 1; }
+          }
           const int t = g * kTileTokens + row;
           const bool in_range = t < p.T;
           const bool valid =
@@ -925,25 +936,22 @@ __global__ void __launch_bounds__(256) token_reduce_kernel(const float* tp, int 
   }
 }
 
-template <int KI, int KO, bool TOKEN>
+template <int KI, int KO, int MODE>
 cudaError_t launch_project_t(const ProjParams& p, int grid, cudaStream_t s) {
-  using C = ProjCfg<KI, KO, TOKEN>;
+  using C = ProjCfg<KI, KO, MODE != kModeProject>;
   static PerDeviceOnce attr;
-  const cudaError_t e = smem_attr_once(attr, project_kernel<KI, KO, TOKEN>, C::kSmemBytes);
+  const cudaError_t e = smem_attr_once(attr, project_kernel<KI, KO, MODE>, C::kSmemBytes);
   if (e != cudaSuccess) return e;
-  return launch_dependent(project_kernel<KI, KO, TOKEN>, dim3(grid), dim3(192), C::kSmemBytes, s,
+  return launch_dependent(project_kernel<KI, KO, MODE>, dim3(grid), dim3(192), C::kSmemBytes, s,
                           p);
 }
 
 template <int KI, int KO>
 cudaError_t launch_project_mode(bool token, const ProjParams& p, int grid, cudaStream_t s) {
-  return token ? launch_project_t<KI, KO, true>(p, grid, s)
-               : launch_project_t<KI, KO, false>(p, grid, s);
-}
-
-template <int KI, int KO>
-constexpr int token_capacity_of() {
-  return ProjCfg<KI, KO, true>::kQB;
+  if (!token) return launch_project_t<KI, KO, kModeProject>(p, grid, s);
+  if constexpr (token_tc_queries(KI, KO) > 0)
+    if (p.piece_buf != nullptr) return launch_project_t<KI, KO, kModeTokenPieces>(p, grid, s);
+  return launch_project_t<KI, KO, kModeToken>(p, grid, s);
 }
 
 }  // namespace
@@ -965,19 +973,6 @@ cudaError_t launch_project(int k_in, int k_out, bool token, const ProjParams& p,
   BERGSON_PROJ_DISPATCH(64, 32, (launch_project_mode<64, 32>(token, p, grid, s)))
   BERGSON_PROJ_DISPATCH(64, 64, (launch_project_mode<64, 64>(token, p, grid, s)))
   return cudaErrorInvalidValue;
-}
-
-int token_query_capacity(int k_in, int k_out) {
-  BERGSON_PROJ_DISPATCH(16, 16, (token_capacity_of<16, 16>()))
-  BERGSON_PROJ_DISPATCH(16, 32, (token_capacity_of<16, 32>()))
-  BERGSON_PROJ_DISPATCH(16, 64, (token_capacity_of<16, 64>()))
-  BERGSON_PROJ_DISPATCH(32, 16, (token_capacity_of<32, 16>()))
-  BERGSON_PROJ_DISPATCH(32, 32, (token_capacity_of<32, 32>()))
-  BERGSON_PROJ_DISPATCH(32, 64, (token_capacity_of<32, 64>()))
-  BERGSON_PROJ_DISPATCH(64, 16, (token_capacity_of<64, 16>()))
-  BERGSON_PROJ_DISPATCH(64, 32, (token_capacity_of<64, 32>()))
-  BERGSON_PROJ_DISPATCH(64, 64, (token_capacity_of<64, 64>()))
-  return 0;
 }
 
 cudaError_t launch_token_reduce(const float* token_partials, int n_mods, int Q, int B, int T,

@@ -16,7 +16,7 @@ DEV = "cuda"
 @pytest.mark.parametrize("B,T,shift", [(1, 1, 0), (3, 7, 0), (3, 7, 1), (2, 130, 0), (4, 33, 1)])
 def test_module_sums(n_mods, B, T, shift):
     specs = [wl.ModuleSpec(f"m{i}", 16, 24) for i in range(n_mods)]
-    gl, ol, ld = make_layers(specs, B, T, [(16, 16)], base_seed=3, data_seed=n_mods, rc=True)
+    gl, ol, ld = make_layers(specs, B, T, [(16, 16)] * n_mods, base_seed=3, data_seed=n_mods, rc=True)
     g = wl.generator(9, "cpu")
     queries = torch.randn((3, ld), generator=g)
     mask = (torch.rand((B, T), generator=g) > 0.3).to(torch.uint8)
