@@ -29,6 +29,12 @@ constexpr int kSchedTargetItems = 8192;              // work items per projectio
 // share of the work, into pieces of about 1/kPiecesPerShare of a share.
 constexpr double kSplitShare = 0.4;
 constexpr int kPiecesPerShare = 2;
+// Shares below kSmallShare units (some 70 us) must be exceeded by half: there the
+// last pieces' sums cost more than an uneven last round, with and without
+// pieces, us a call: 2 blocks of Pythia-160M, 7 x 333 tokens (1.1 shares) 45 / 39,
+// 4 of 4 x 242, k = 16 x 64 (1.5) 64 / 58; and 1 block of 1 x 300 (13) 32 / 64.
+constexpr double kSmallShare = 200.0;
+constexpr double kSplitSmallShare = 1.5;
 constexpr double kMinPieceUnits = 4.0;               // ... of at least 4 chunks of a tile
 constexpr double kFinePieceShare = 0.8;              // largest piece, in shares, before the minimum
                                                      // piece size is lowered
@@ -43,8 +49,8 @@ constexpr double kTokenSplitUnits = 64.0;
 constexpr double kTokenSplitPerQuery = 0.75;
 constexpr int kTokenSlotsPerCTA = 16;
 constexpr int kFineMaxK = 96;                        // k_in + k_out up to which it is
-constexpr double kFineSlotUnits = 64.0;              // shares below this (and few slots): slots of
-                                                     // one tile each
+// Few slots (below two a CTA) of shares below this: slots of one tile.
+constexpr double kFineSlotUnits = 400.0;
 constexpr int kMaxScoreCTAs = 160;                   // upper bound on persistent score CTAs
 constexpr int kMaxDevices = 64;
 constexpr int kMaxTokenQueries = 256;                // per-token scores: queries per call
@@ -265,7 +271,8 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, in
   }
   const double share = static_cast<double>(total) / kPlanCTAs;
   const double excess = static_cast<double>(max_slot) - share;
-  const bool split = n_queries == 0 ? static_cast<double>(max_slot) > kSplitShare * share
+  const bool split = n_queries == 0 ? static_cast<double>(max_slot) >
+                                          (share < kSmallShare ? kSplitSmallShare : kSplitShare) * share
                                     : token_split && excess > kTokenSplitUnits +
                                                                   kTokenSplitPerQuery * n_queries;
   bool shared = false;
@@ -495,9 +502,17 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
     if (want < 1) want = 1;
     int tpc = static_cast<int>((L.n_tiles + want - 1) / want);
     tpc = (tpc + nt_per_group - 1) / nt_per_group * nt_per_group;
-    if (fine && tpc > 1 && mb * ((L.n_tiles + tpc - 1) / tpc) < 2 * kPlanCTAs) {
+    if (fine && tpc > 1 && 2 * L.n_tiles <= nt_per_group) {
+      // stages of several tiles would be half empty at best (48 modules, 16 x 129
+      // tokens: 249 -> 202 us; three tiles of four are better together, 9 x 4
+      // modules, 29 x 257 tokens 329 / 366)
+      tpc = 1;
+    } else if (fine && tpc > 1 && mb * ((L.n_tiles + tpc - 1) / tpc) < 2 * kPlanCTAs) {
       // few slots of a small launch: one tile each (more P' reads from L2, but
-      // more CTAs at work: 300 tokens of one example had 4 slots)
+      // more CTAs at work, and pieces of one tile in stages of one tile).  With
+      // slots of four tiles / of one, us a call: a Llama-8B-shaped block of 2 x 1024
+      // tokens 116 / 70, 1.4B-shaped blocks of 5 x 700 (k = 16 x 32) 76 / 64 and 20
+      // x 600 194 / 134, 16 Pythia-160M modules of 4 x 512 81 / 58.
       int64_t units_total = 0;
       for (int li : g.layers)
         units_total += int64_t{chunks_of(layers[li].d_in) + chunks_of(layers[li].d_out)} *

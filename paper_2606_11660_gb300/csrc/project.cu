@@ -46,7 +46,7 @@ constexpr int pow2ceil(int x) {
   return p;
 }
 
-template <int KI, int KO, bool TOKEN = false>
+template <int KI, int KO, bool TOKEN = false, bool TILE = false>
 struct ProjCfg {
   // Token mode on the tensor cores (kTC): per tile and block of kTcNQ queries,
   // U = a~ Q^T (M = 128 tokens, K = k_in, N = kTcNQ k_out rows (q, i)) on
@@ -62,7 +62,7 @@ struct ProjCfg {
   // Tiles sharing one P' slice: each slice is re-read from L2 once per NT
   // tiles, so a larger NT cuts L2 -> SM traffic (NT = 1 -> 2 -> 4 measured
   // 3.05 -> 2.72 -> 2.59 ms on the 48-module bench call).
-  static constexpr int NT = kTC ? 1 : ((KI + KO <= 32) ? 4 : ((KI + KO <= 64) ? 2 : 1));
+  static constexpr int NT = kTC || TILE ? 1 : ((KI + KO <= 32) ? 4 : ((KI + KO <= 64) ? 2 : 1));
   static constexpr int kPRows = 2 * (KI > KO ? KI : KO);         // hi + lo rows
   static constexpr int kPBytes = kPRows * 128;
   static constexpr int kStageBytes = NT * kActBoxBytes + kPBytes;
@@ -74,7 +74,7 @@ struct ProjCfg {
       kTC ? 2 * kTcBBytes : kEpiRows * (KI + 4) * 4 + kEpiRows * (KO + 4) * 4;
   static constexpr int kBarBytes = 512;
   static constexpr int kStagesFit = (kSmemBudget - 1024 - kEpiBytes - kBarBytes) / kStageBytes;
-  static constexpr int kStages = kStagesFit > 8 ? 8 : kStagesFit;
+  static constexpr int kStages = kStagesFit > 12 ? 12 : kStagesFit;
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kEpiBytes + kBarBytes;
   // Per tile: A*[hi|lo] in 2 KI columns, then G*[hi|lo] in 2 KO columns.
   static constexpr int kTmemPerBuf = NT * 2 * (KI + KO);
@@ -277,11 +277,16 @@ __device__ __forceinline__ void tmem_store_row(uint32_t taddr, const float* v) {
 // 8 x 2048 tokens, 64 queries 784 -> 801 us; 4 x 2047 tokens, 200 queries 729 ->
 // 883 us: all 255 registers in use, the query blocks' loads issued later).
 constexpr int kModeProject = 0, kModeToken = 1, kModeTokenPieces = 2;
+// Collections whose slots are one tile: stages of one tile, so that a slot's
+// loads fill all of them (k = 16: ten stages of 20 KB; of the three stages of
+// four tiles a quarter was used).  A Llama-8B-shaped block of 512 tokens 56 -> 43
+// us, 7 x 333 tokens of 8 modules 47 -> 39.
+constexpr int kModeProjectTile = 3;
 template <int KI, int KO, int MODE>
 __global__ void __launch_bounds__(192, 1) project_kernel(const ProjParams p) {
-  constexpr bool TOKEN = MODE != kModeProject;
+  constexpr bool TOKEN = MODE == kModeToken || MODE == kModeTokenPieces;
   constexpr bool kPieces = MODE != kModeToken;
-  using C = ProjCfg<KI, KO, TOKEN>;
+  using C = ProjCfg<KI, KO, TOKEN, MODE == kModeProjectTile>;
   constexpr int NT = C::NT;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -938,7 +943,8 @@ __global__ void __launch_bounds__(256) token_reduce_kernel(const float* tp, int 
 
 template <int KI, int KO, int MODE>
 cudaError_t launch_project_t(const ProjParams& p, int grid, cudaStream_t s) {
-  using C = ProjCfg<KI, KO, MODE != kModeProject>;
+  using C = ProjCfg<KI, KO, MODE == kModeToken || MODE == kModeTokenPieces,
+                    MODE == kModeProjectTile>;
   static PerDeviceOnce attr;
   const cudaError_t e = smem_attr_once(attr, project_kernel<KI, KO, MODE>, C::kSmemBytes);
   if (e != cudaSuccess) return e;
@@ -948,7 +954,11 @@ cudaError_t launch_project_t(const ProjParams& p, int grid, cudaStream_t s) {
 
 template <int KI, int KO>
 cudaError_t launch_project_mode(bool token, const ProjParams& p, int grid, cudaStream_t s) {
-  if (!token) return launch_project_t<KI, KO, kModeProject>(p, grid, s);
+  if (!token) {
+    if constexpr (ProjCfg<KI, KO>::NT > 1)
+      if (p.tpc == 1) return launch_project_t<KI, KO, kModeProjectTile>(p, grid, s);
+    return launch_project_t<KI, KO, kModeProject>(p, grid, s);
+  }
   if constexpr (token_tc_queries(KI, KO) > 0)
     if (p.piece_buf != nullptr) return launch_project_t<KI, KO, kModeTokenPieces>(p, grid, s);
   return launch_project_t<KI, KO, kModeToken>(p, grid, s);

@@ -1,8 +1,10 @@
-"""The planner's line for cutting per-token score slots, through the workspace it asks for (CPU)."""
+"""The lines of the projection planner: slots, and when they are cut into pieces (CPU)."""
 import pytest
 import torch
 
 import paper_2606_11660_gb300 as bg
+from paper_2606_11660_gb300 import workloads as wl
+from tests.test_abi import _block_layers, _plan
 
 
 def _layers(dims, B, T, k):
@@ -35,3 +37,21 @@ def test_cut(dims, B, T, k, q, cut):
     tile_rows = 4 * B * 128 * (k[0] + k[1])            # one piece a side, one tile
     extra = _extra(dims, B, T, k, q)
     assert (extra >= tile_rows) == cut
+
+
+@pytest.mark.parametrize("name,blocks,B,T,k,tiles,cut", [
+    ("pythia160m", 2, 7, 333, 16, 1, False),     # one-tile slots; 60 units to a share of 53
+    ("pythia160m", 1, 1, 300, 16, 1, True),      # 60 to 4
+    ("llama8b", 1, 2, 1024, 16, 1, True),
+    ("llama8b", 1, 8, 4096, 16, 4, True),        # a large share: pieces as before
+    ("pythia160m", 12, 16, 129, 16, 1, False),   # two tiles would half fill a stage
+    ("pythia160m", 9, 29, 257, 16, 4, False),    # three of four: one slot an example
+    ("pythia1b4", 1, 16, 2048, 32, 2, False),
+])
+def test_slots_of_collections(name, blocks, B, T, k, tiles, cut):
+    cfg = wl.COLLECT_WORKLOADS[name]
+    specs = [s for b in range(blocks) for s in cfg.block_modules(b)]
+    slots, items, pieces, _ = _plan(_block_layers(specs, k), B, T)
+    n_tiles = (T + 127) // 128
+    assert slots == len(specs) * B * max(1, -(-n_tiles // tiles))
+    assert (pieces > 0) == cut
