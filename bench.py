@@ -342,7 +342,7 @@ def bench_collection(args, world, dev, peaks, peak_kind):
     proj_ms = statistics.mean(a.elapsed_time(b) for a, b in pairs)
     achieved = alg_bytes / (proj_ms * 1e-3) / 1e9
     traffic = profiled_traffic("project_kernel_pythia160m.md", "project.cu")
-    launches_per_step = 1 + 1 + 2 + 1   # prep, tile flags, projection, reduce, store
+    launches_per_step = 1 + 2 + 1   # prep (with the tile flags), projection, reduce, store
     res = {
         "value": cfg.B * world * args.steps / (elapsed_ms * 1e-3),
         "ms_per_step": elapsed_ms / args.steps,
@@ -413,8 +413,8 @@ def bench_onthefly(args, world, dev, state, peaks):
                          "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4),
                          "kernel": "bergson_score_grads call (split, tcgen05 3xTF32 product, "
                                    "finish)", "algorithmic_bytes_per_call": alg},
-            # tile flags, prep, projection, reduce; row split, product, finish
-            "gpu_launches": (4 + 3) * args.steps,
+            # prep, projection, reduce; row split, product, finish
+            "gpu_launches": (3 + 3) * args.steps,
             "what": "bergson_project_grads + bergson_score_grads (cosine vs 1024 fp32 queries, "
                     "no store) per batch"}
 
@@ -454,7 +454,7 @@ def bench_tokens(args, world, dev, state, peaks):
             "roofline": {"bound": "hbm", "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"],
                          "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4),
                          "traffic": profiled_traffic("token_kernel_pythia160m.md", "project.cu")},
-            "gpu_launches": 4 * args.steps,          # tile flags, prep, projection, token sum
+            "gpu_launches": 3 * args.steps,          # prep, projection, token sum
             "what": f"bergson_token_scores: per-token scores of all 65,536 tokens x 48 modules "
                     f"against {Q} query rows in one pass over A and G"}
 

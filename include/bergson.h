@@ -394,7 +394,7 @@ BERGSON_API int bergson_aggregate_rows(const float* rows, int64_t n, int64_t K, 
  * (or bergson_score_grads) as usual.  All matrices are fp32 row-major with
  * 16-byte aligned rows (leading dimensions multiples of 4); K % 4 == 0,
  * K <= 65536.  Workspaces: bergson_fisher_fit_workspace(n, K),
- * bergson_fisher_preconditioner_workspace(K) (4 K^2 floats) and, for
+ * bergson_fisher_preconditioner_workspace(K) (about 6 K^2 floats) and, for
  * precondition_rows, bergson_score_grads_workspace(B, K, K).
  * Errors: EINVAL, EALIGN, EWORKSPACE, ECUDA.
  */
@@ -549,9 +549,10 @@ BERGSON_API int bergson_debug_project_plan(const bergson_layer* layers, int n_la
  * launches (each followed by a merge); the first min(max_launches,
  * *n_launches) are written to out as rows of 12 int64:
  *   pass, stage (0 = prefix threshold pass, 1 = full pass), store rows,
- *   query groups, first query group, CTAs per group, grid, store tiles,
- *   first query, end query (of the merge), pair (1 = clusters of two CTAs),
- *   128-query tiles per CTA.
+ *   query groups, first query group, CTAs per group, grid, store tiles of 256
+ *   rows (a launch may even these out into smaller ones), first query, end
+ *   query (of the merge), pair (1 = clusters of two CTAs), 128-query tiles per
+ *   CTA.
  * Host only: enqueues nothing.  Errors: EINVAL.
  */
 BERGSON_API int bergson_debug_score_plan(int64_t N, int64_t K, int64_t Q, int64_t topk, int ctas,
@@ -559,7 +560,7 @@ BERGSON_API int bergson_debug_score_plan(int64_t N, int64_t K, int64_t Q, int64_
 
 /*
  * Test aid for the planner of the skinny tcgen05 product behind
- * bergson_score_grads, bergson_precondition_rows and the Fisher products
+ * bergson_score_grads and bergson_precondition_rows
  * (C[b, q] = <x_b, y_q> for B rows x, Q rows y of length K).  Writes 19 int64
  * to out (n_out >= 19): batch rows per tile, batch tiles, y tiles, 32-column
  * steps, K slices, pipeline stages, column chunks of the row split, CTA pairs
