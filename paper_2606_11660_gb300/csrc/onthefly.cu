@@ -872,15 +872,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // order) of xnorm[b, c], ny_q the sum over the same planes of ynorm[z, q] (0
 // when either row is zero).  Otherwise scores[b, q] = s.
 //
-// The planes' loads are issued kFinishBatch at a time before they are added in
-// order (one after another, the 20 planes and 20 norms of a 1024-query call were
-// 7 us of L2 latency), and a thread keeps its column's norm for all its rows.
-constexpr int kFinishBatch = 8;
+// The planes' loads are issued kBatch at a time before they are added in order
+// (one after another, the 20 planes and 20 norms of a 1024-query call were 7 us
+// of L2 latency), and a thread keeps its column's norm for all its rows.  A
+// batch that fits the planes leaves fewest idle slots, and short ones keep five
+// CTAs an SM.  us a call, one load at a time / always 8 / as here: 166 x 48 x 1796
+// cosine (57 planes) 21.0 / 22.8 / 20.3; 168 x 2384 x 2384 (4) 32.0 / 33.0 / 31.0; 100 x
+// 300 x 5000 cosine 24.9 / 22.8 / 20.8; 32 x 12,288 x 12,288 127.3 / 126.6 / 125.4.
+template <int kBatch>
 struct PlaneSum {                 // a sum over n planes, its first batch in flight
   const float* src;
   int64_t stride;
   int n;
-  float v[kFinishBatch];
+  float v[kBatch];
   __device__ __forceinline__ void start(const float* src_, int64_t stride_, int n_) {
     src = src_;
     stride = stride_;
@@ -889,23 +893,24 @@ struct PlaneSum {                 // a sum over n planes, its first batch in fli
   }
   __device__ __forceinline__ void load(int z0) {
 #pragma unroll
-    for (int z = 0; z < kFinishBatch; ++z)
+    for (int z = 0; z < kBatch; ++z)
       if (z0 + z < n) v[z] = __ldcg(src + (z0 + z) * stride);
   }
   __device__ __forceinline__ float finish() {
     float s = 0.0f;
     for (int z0 = 0;;) {
 #pragma unroll
-      for (int z = 0; z < kFinishBatch; ++z)
+      for (int z = 0; z < kBatch; ++z)
         if (z0 + z < n) s += v[z];
-      z0 += kFinishBatch;
+      z0 += kBatch;
       if (z0 >= n) return s;
       load(z0);
     }
   }
 };
 
-__global__ void __launch_bounds__(256) finish_kernel(const float* partial, int S, int B, int Q,
+template <int kBatch>
+__global__ void __launch_bounds__(256, kBatch <= 8 ? 5 : 2) finish_kernel(const float* partial, int S, int B, int Q,
                                                      const float* xnorm, int n_chunks,
                                                      const float* ynorm, int seg_clusters,
                                                      int steps, int y_rows, float* scores,
@@ -923,7 +928,8 @@ __global__ void __launch_bounds__(256) finish_kernel(const float* partial, int S
   float iy = 0.0f;
   bool first = true;
   for (int b = blockIdx.y; b < B; b += gridDim.y) {
-    PlaneSum sum, sx, sy;
+    PlaneSum<kBatch> sum, sy;
+    PlaneSum<kBatch <= 8 ? 4 : kBatch> sx;
     sum.start(partial + static_cast<int64_t>(b) * Q + q, n, planes);
     float* dst = scores + b * ld + q;
     if (xnorm == nullptr) {
@@ -1115,7 +1121,11 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s) {
   const int fx = (a.Q + 255) / 256;
   const dim3 fgrid(fx, std::max(1, std::min({a.B, 65535, (8 * kPlanCTAs + fx - 1) / fx})));
   const float* xn = a.unit ? xnorm : nullptr;
-  return launch_dependent(finish_kernel, fgrid, dim3(256), 0, s, p.partial, pl.S, a.B, a.Q, xn,
+  const auto finish = pl.S <= 4    ? finish_kernel<4>
+                      : pl.S <= 8  ? finish_kernel<8>
+                      : pl.S <= 12 ? finish_kernel<12>
+                                   : finish_kernel<16>;
+  return launch_dependent(finish, fgrid, dim3(256), 0, s, p.partial, pl.S, a.B, a.Q, xn,
                           pl.n_chunks, p.ynorm, pl.pair ? pl.n_clusters : 0, pl.steps, pl.y_rows,
                           a.scores, a.ld_scores);
 }
