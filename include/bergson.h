@@ -549,14 +549,26 @@ BERGSON_API int bergson_debug_project_plan(const bergson_layer* layers, int n_la
  * launches (each followed by a merge); the first min(max_launches,
  * *n_launches) are written to out as rows of 12 int64:
  *   pass, stage (0 = prefix threshold pass, 1 = full pass), store rows,
- *   query groups, first query group, CTAs per group, grid, store tiles of 256
- *   rows (a launch may even these out into smaller ones), first query, end
- *   query (of the merge), pair (1 = clusters of two CTAs), 128-query tiles per
- *   CTA.
+ *   query groups, first query group, then CTAs per group, grid and store tiles
+ *   for tiles of 256 rows (what is launched, with tiles evened out over the
+ *   CTAs: bergson_debug_score_launches), first query, end query (of the merge),
+ *   pair (1 = clusters of two CTAs), 128-query tiles per CTA.
  * Host only: enqueues nothing.  Errors: EINVAL.
  */
 BERGSON_API int bergson_debug_score_plan(int64_t N, int64_t K, int64_t Q, int64_t topk, int ctas,
                                          int64_t* out, int max_launches, int* n_launches);
+
+/*
+ * The same launches as they are made (for a workspace of
+ * bergson_score_topk_workspace bytes), as rows of 8 int64: store rows, query
+ * groups, store rows per tile, store tiles, CTAs per group, grid, and the bound
+ * j, r each of a group's CTAs takes on the final k-th best (its j-th best
+ * first-tile score is published, the r-th largest of those is the bound; 0, 0:
+ * none).  Host only: enqueues nothing.  Errors: EINVAL.
+ */
+BERGSON_API int bergson_debug_score_launches(int64_t N, int64_t K, int64_t Q, int64_t topk,
+                                             int ctas, int64_t* out, int max_launches,
+                                             int* n_launches);
 
 /*
  * Test aid for the planner of the skinny tcgen05 product behind

@@ -19,7 +19,8 @@ from .binding import (  # noqa: F401
     bergson_build_store_blocks, bergson_score_topk_update, bergson_score_topk_update_workspace,
     bergson_score_topk_host, bergson_score_topk_host_workspace,
     bergson_debug_attr_once,
-    bergson_debug_project_plan, bergson_debug_score_plan, bergson_debug_xgemm_plan,
+    bergson_debug_project_plan, bergson_debug_score_launches, bergson_debug_score_plan,
+    bergson_debug_xgemm_plan,
     bergson_debug_wait_probe, bergson_last_error, bergson_module_seeds, bergson_project_grads,
     bergson_project_grads_noalloc, bergson_project_grads_workspace, bergson_projection_matrix, bergson_score_topk,
     bergson_score_bottomk,

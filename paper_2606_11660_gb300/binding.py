@@ -50,7 +50,8 @@ EXPORTED = (
     "bergson_projection_matrix",
     "bergson_module_seeds", "bergson_sync_status", "bergson_last_error", "bergson_version",
     "bergson_debug_wait_probe", "bergson_debug_inject_status", "bergson_debug_project_plan",
-    "bergson_debug_score_plan", "bergson_debug_xgemm_plan", "bergson_project_grads_noalloc",
+    "bergson_debug_score_plan", "bergson_debug_score_launches", "bergson_debug_xgemm_plan",
+    "bergson_project_grads_noalloc",
     "bergson_score_grads_workspace", "bergson_score_grads", "bergson_token_scores_workspace",
     "bergson_token_scores", "bergson_aggregate_rows_workspace", "bergson_aggregate_rows",
     "bergson_fisher_fit_workspace", "bergson_fisher_fit", "bergson_fisher_preconditioner_workspace",
@@ -124,6 +125,8 @@ def lib() -> ctypes.CDLL:
         "bergson_debug_project_plan": (i32, [lp, i32, i64, i64, i64p, i64p, i64p, i64p]),
         "bergson_debug_score_plan": (i32, [i64, i64, i64, i64, i32, i64p, i32,
                                            ctypes.POINTER(i32)]),
+        "bergson_debug_score_launches": (i32, [i64, i64, i64, i64, i32, i64p, i32,
+                                               ctypes.POINTER(i32)]),
         "bergson_debug_xgemm_plan": (i32, [i64, i64, i64, i64p, i32]),
         "bergson_debug_attr_once": (i32, [i32, i32, i32, i64p, ctypes.POINTER(i32)]),
         "bergson_project_grads_noalloc": (i32, [lp, i32, i64, i64, vp, vp, i64, vp]),
@@ -511,16 +514,28 @@ SCORE_PLAN_COLUMNS = ("pass", "stage", "rows", "n_qg", "qg_base", "cpg", "grid",
                       "q_begin", "q_end", "pair", "qt")
 
 
+SCORE_LAUNCH_COLUMNS = ("rows", "n_qg", "bn", "n_tiles", "cpg", "grid", "bound_j", "bound_r")
+
+
+def _score_rows(fn: str, columns, N: int, K: int, Q: int, topk: int, ctas: int) -> list[dict]:
+    call = getattr(lib(), fn)
+    args = (int(N), int(K), int(Q), int(topk), int(ctas))
+    n, w = ctypes.c_int32(), len(columns)
+    _check(call(*args, None, 0, ctypes.byref(n)))
+    buf = (ctypes.c_int64 * (w * max(1, n.value)))()
+    _check(call(*args, buf, n.value, ctypes.byref(n)))
+    return [dict(zip(columns, buf[w * i:w * i + w])) for i in range(n.value)]
+
+
 def bergson_debug_score_plan(N: int, K: int, Q: int, topk: int, ctas: int) -> list[dict]:
     """The score launches (one dict per launch, keys SCORE_PLAN_COLUMNS) the
     scorer's planner makes for `ctas` resident CTAs; host only."""
-    n = ctypes.c_int32()
-    _check(lib().bergson_debug_score_plan(int(N), int(K), int(Q), int(topk), int(ctas), None, 0,
-                                          ctypes.byref(n)))
-    buf = (ctypes.c_int64 * (12 * max(1, n.value)))()
-    _check(lib().bergson_debug_score_plan(int(N), int(K), int(Q), int(topk), int(ctas), buf,
-                                          n.value, ctypes.byref(n)))
-    return [dict(zip(SCORE_PLAN_COLUMNS, buf[12 * i:12 * i + 12])) for i in range(n.value)]
+    return _score_rows("bergson_debug_score_plan", SCORE_PLAN_COLUMNS, N, K, Q, topk, ctas)
+
+
+def bergson_debug_score_launches(N: int, K: int, Q: int, topk: int, ctas: int) -> list[dict]:
+    """The same launches with their tiles, grid and bound (keys SCORE_LAUNCH_COLUMNS); host only."""
+    return _score_rows("bergson_debug_score_launches", SCORE_LAUNCH_COLUMNS, N, K, Q, topk, ctas)
 
 
 XGEMM_PLAN_FIELDS = ("n_pad", "n_ntiles", "n_mtiles", "steps", "S", "stages", "n_chunks",

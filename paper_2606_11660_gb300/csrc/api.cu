@@ -668,9 +668,12 @@ struct ScoreLaunch {
   int64_t rows = 0;        // store rows this launch scores (a prefix, or N)
   int n_qg = 0;            // query groups of this pass
   int qg_base = 0;         // first query group of this pass
+  int bn = 0;              // store rows per tile
+  int n_tiles = 0;         // tiles of `rows`
   int cpg = 0;             // CTAs per query group
   int grid = 0;            // n_qg * cpg
-  int n_tiles = 0;         // 256-row store tiles of `rows`
+  int bound_j = 0;         // the kernel's bound (score_bound_rule; 0: none)
+  int bound_r = 0;
   int q_begin = 0, q_end = 0;   // queries this launch's merge writes
 };
 
@@ -701,9 +704,10 @@ void score_bound_rule(int64_t rows, int bn, int cpg, int topk, int* j, int* r) {
 }
 
 // Launch sequence of bergson_score_topk for `ctas` resident CTAs (for the pair
-// kernel: 2 x its co-resident clusters).  Pure host logic.
+// kernel: 2 x its co-resident clusters); `room`: the workspace holds the
+// published scores.  Pure host logic.
 ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas,
-                                    bool allow_prefix = true) {
+                                    bool allow_prefix = true, bool room = true) {
   ScoreLaunchPlan P;
   const ScoreLayout L = plan_score(0, Q, topk);
   P.pair = Q >= kPairMinQueries;
@@ -741,9 +745,12 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
       l.rows = stage == 0 ? prefix : N;
       l.n_qg = n_qg;
       l.qg_base = pass;
-      l.n_tiles = static_cast<int>((l.rows + kScoreBN - 1) / kScoreBN);
+      l.bn = score_tile_rows(l.rows, sms / n_qg);
+      l.n_tiles = static_cast<int>((l.rows + l.bn - 1) / l.bn);
       l.cpg = std::max(1, std::min(sms / n_qg, l.n_tiles));
       l.grid = n_qg * l.cpg;
+      if (room && l.grid <= kPlanCTAs)         // more CTAs have no room for their words
+        score_bound_rule(l.rows, l.bn, l.cpg, static_cast<int>(topk), &l.bound_j, &l.bound_r);
       l.q_begin = pass * P.gsize;
       l.q_end = static_cast<int>(std::min<int64_t>(Q, static_cast<int64_t>(pass + n_qg) * P.gsize));
       P.launches.push_back(l);
@@ -867,9 +874,28 @@ int bergson_debug_score_plan(int64_t N, int64_t K, int64_t Q, int64_t topk, int 
   const int n = out == nullptr ? 0 : std::min(max_launches, *n_launches);
   for (int i = 0; i < n; ++i) {
     const ScoreLaunch& l = P.launches[i];
-    const int64_t row[12] = {l.pass, l.stage, l.rows, l.n_qg, l.qg_base, l.cpg,
-                             l.grid, l.n_tiles, l.q_begin, l.q_end, P.pair ? 1 : 0, P.qt};
+    const int tiles = static_cast<int>((l.rows + kScoreBN - 1) / kScoreBN);   // whole tiles
+    const int cpg = std::max(1, std::min(P.ctas / l.n_qg, tiles));
+    const int64_t row[12] = {l.pass, l.stage, l.rows, l.n_qg, l.qg_base, cpg,
+                             l.n_qg * cpg, tiles, l.q_begin, l.q_end, P.pair ? 1 : 0, P.qt};
     for (int c = 0; c < 12; ++c) out[static_cast<int64_t>(i) * 12 + c] = row[c];
+  }
+  return BERGSON_OK;
+}
+
+int bergson_debug_score_launches(int64_t N, int64_t K, int64_t Q, int64_t topk, int ctas,
+                                 int64_t* out, int max_launches, int* n_launches) {
+  if (n_launches == nullptr) return fail(BERGSON_EINVAL, "n_launches is NULL");
+  const int st = validate_score_sizes(N, K, Q, topk);
+  if (st != BERGSON_OK) return st;
+  if (ctas < 1) return fail(BERGSON_EINVAL, "ctas must be >= 1");
+  const ScoreLaunchPlan P = plan_score_launches(N, Q, topk, ctas);
+  *n_launches = static_cast<int>(P.launches.size());
+  const int n = out == nullptr ? 0 : std::min(max_launches, *n_launches);
+  for (int i = 0; i < n; ++i) {
+    const ScoreLaunch& l = P.launches[i];
+    const int64_t row[8] = {l.rows, l.n_qg, l.bn, l.n_tiles, l.cpg, l.grid, l.bound_j, l.bound_r};
+    for (int c = 0; c < 8; ++c) out[static_cast<int64_t>(i) * 8 + c] = row[c];
   }
   return BERGSON_OK;
 }
@@ -1276,7 +1302,7 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
     if (e != cudaSuccess) return fail_cuda(e, "score kernel occupancy query");
     ctas = std::min(ctas, resident);
   }
-  const ScoreLaunchPlan P = plan_score_launches(N, Q, topk, ctas, !update);
+  const ScoreLaunchPlan P = plan_score_launches(N, Q, topk, ctas, !update, room);
   if (P.launches.empty()) return fail(BERGSON_ECUDA, "no two-SM cluster fits the score kernel");
   uint16_t* pub = reinterpret_cast<uint16_t*>(ws + L.pub_off);
   const int pub_words = room ? std::min(P.ctas, kPlanCTAs) * L.qt * kScoreQT : 0;
@@ -1296,20 +1322,16 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
     p.topk = static_cast<int>(topk);
     p.n_qg = l.n_qg;
     p.qg_base = l.qg_base;
-    // The plan counts 256-row tiles; the launch evens them out over the CTAs.
-    const int per_group = P.ctas / l.n_qg;
-    p.bn = score_tile_rows(l.rows, per_group);
-    p.n_ntiles = static_cast<int>((l.rows + p.bn - 1) / p.bn);
-    const int cpg = std::max(1, std::min(per_group, p.n_ntiles));
-    const int grid = l.n_qg * cpg;
+    p.bn = l.bn;
+    p.n_ntiles = l.n_tiles;
     if (box != p.bn) {
       box = p.bn;
       r = encode_2d(&tm_store, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, store, K, N, ld_store * 2, kChunk,
                     pair ? box / 2 : box);
       if (r != CUDA_SUCCESS) return fail(BERGSON_ECUDA, "tensor map encoding failed (%d)", (int)r);
     }
-    score_bound_rule(l.rows, p.bn, cpg, static_cast<int>(topk), &p.bound_j, &p.bound_r);
-    if (grid > kPlanCTAs || !room) p.bound_j = p.bound_r = 0;   // no room for their words
+    p.bound_j = l.bound_j;
+    p.bound_r = l.bound_r;
     p.stages = p.q_rows = 0;
     p.heaps = heaps;
     p.pub = pub;
@@ -1321,14 +1343,15 @@ static int run_score(const void* store, int64_t N, int64_t K, int64_t ld_store,
     p.timeout_ns = kWaitTimeoutNs;
     p.pace = pair ? reinterpret_cast<unsigned long long*>(ws + L.pace_off) : nullptr;
     p.pace_tag = pair ? next_pace_tag() : 0;
-    e = pair ? launch_score_pair(L.qt, tm_store, tm_q, p, grid, s)
-             : launch_score(tm_store, tm_q, p, grid, s);
+    e = pair ? launch_score_pair(L.qt, tm_store, tm_q, p, l.grid, s)
+             : launch_score(tm_store, tm_q, p, l.grid, s);
     if (e != cudaSuccess) return fail_cuda(e, "score kernel launch");
     // The prefix pass's scores seed the full pass's thresholds, so only
     // the final merge converts them back for a bottom-k search.
     const bool final_merge = l.stage == 1;
-    e = launch_merge(heaps, pub, grid > kPlanCTAs ? 0 : pub_words, grid, l.n_qg, L.qt, static_cast<int>(topk), l.q_begin, l.q_end,
-                     least && final_merge, final_merge ? row_base : 0,
+    e = launch_merge(heaps, pub, l.grid > kPlanCTAs ? 0 : pub_words, l.grid, l.n_qg, L.qt,
+                     static_cast<int>(topk), l.q_begin, l.q_end, least && final_merge,
+                     final_merge ? row_base : 0,
                      update && final_merge ? out_scores : nullptr,
                      update && final_merge ? out_idx : nullptr, out_scores, out_idx, s);
     if (e != cudaSuccess) return fail_cuda(e, "merge kernel launch");
