@@ -745,7 +745,7 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
       l.rows = stage == 0 ? prefix : N;
       l.n_qg = n_qg;
       l.qg_base = pass;
-      l.bn = score_tile_rows(l.rows, sms / n_qg);
+      l.bn = score_tile_rows(l.rows, sms / n_qg, P.pair);
       l.n_tiles = static_cast<int>((l.rows + l.bn - 1) / l.bn);
       l.cpg = std::max(1, std::min(sms / n_qg, l.n_tiles));
       l.grid = n_qg * l.cpg;

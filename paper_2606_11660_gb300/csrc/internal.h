@@ -165,7 +165,7 @@ struct ScoreParams {
   int topk;
   int n_qg;             // query groups in this pass
   int qg_base;          // first query group of this pass
-  int bn;               // store rows per tile (a multiple of 16, at most 256)
+  int bn;               // store rows per tile (a multiple of 16, on pairs of 32; at most 256)
   int n_ntiles;         // ceil(N / bn)
   int stages;           // single-CTA kernel (set by launch_score): ring stages
   int q_rows;           //   and query rows loaded per stage
@@ -233,7 +233,7 @@ cudaError_t launch_normalize_queries(const float* q, int Q, int K, int64_t ld_q,
                                      __half* qh, uint16_t* pub, int pub_words, cudaStream_t s);
 // Store rows per tile for `rows` store rows over `ctas_per_group` CTAs, and query
 // rows the single-CTA kernel loads (its tensor map's box).
-int score_tile_rows(int64_t rows, int ctas_per_group);
+int score_tile_rows(int64_t rows, int ctas_per_group, bool pair);
 int score_query_rows(int Q);
 // Up to 128 queries: one CTA per SM, store tensor map with p.bn-row boxes, query
 // tensor map with score_query_rows()-row boxes.

@@ -1117,13 +1117,15 @@ __global__ void __launch_bounds__(512) merge_kernel(const unsigned long long* li
 // Store rows per tile of a launch that scores `rows` rows with `ctas_per_group`
 // CTAs per query group: the whole rounds of 256-row tiles that the rows need,
 // shared out evenly (a last round that is nearly empty would cost as much as a
-// full one), in steps of 16 (what one MMA takes).  Not below 64: smaller MMAs
-// take as long to issue as that one, and a tile's fixed costs weigh more.
-int score_tile_rows(int64_t rows, int ctas_per_group) {
+// full one), in steps of what one MMA takes: N of 16 at M = 128 on one CTA, of 32
+// at M = 256 over a pair.  Not below 64: smaller MMAs take as long to issue as
+// that one, and a tile's fixed costs weigh more.
+int score_tile_rows(int64_t rows, int ctas_per_group, bool pair) {
+  const int64_t step = pair ? 32 : 16;
   const int64_t per_round = static_cast<int64_t>(std::max(1, ctas_per_group)) * kScoreBN;
   const int64_t rounds = (rows + per_round - 1) / per_round;
   const int64_t tiles = rounds * std::max(1, ctas_per_group);
-  const int64_t bn = ((rows + tiles - 1) / tiles + 15) / 16 * 16;
+  const int64_t bn = ((rows + tiles - 1) / tiles + step - 1) / step * step;
   return static_cast<int>(std::max<int64_t>(64, std::min<int64_t>(kScoreBN, bn)));
 }
 

@@ -30,10 +30,11 @@ def _launches(N, Q, topk, ctas):
 def check(N, Q, topk, ctas):
     for p, l in _launches(N, Q, topk, ctas):
         assert (l["rows"], l["n_qg"]) == (p["rows"], p["n_qg"])
-        # tiles cover the rows in steps one MMA takes, and no CTA has one round more than
+        # tiles cover the rows in steps one MMA takes (N of 16 at M = 128, of 32 at the pairs'
+        # M = 256), and no CTA has one round more than
         # with tiles of 256 rows
         per_group = (min(ctas, 160) & (~1 if p["pair"] else ~0)) // l["n_qg"]
-        assert 64 <= l["bn"] <= 256 and l["bn"] % 16 == 0
+        assert 64 <= l["bn"] <= 256 and l["bn"] % (32 if p["pair"] else 16) == 0
         assert l["n_tiles"] == -(-l["rows"] // l["bn"])
         assert -(-l["n_tiles"] // per_group) <= -(-l["rows"] // (256 * per_group))
         assert 1 <= l["cpg"] <= min(l["n_tiles"], per_group)
