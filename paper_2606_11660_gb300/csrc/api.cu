@@ -809,11 +809,13 @@ CUresult encode_tmap_2d(CUtensorMap* tm, CUtensorMapDataType dt, const void* ptr
 CUresult encode_tmap_planes(CUtensorMap* tm, const void* ptr, int64_t inner, int64_t outer,
                             int64_t ld, int box_inner, int box_outer) {
   if (encode_fn() == nullptr) return CUDA_ERROR_NOT_SUPPORTED;
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(outer), 2};
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(outer),
+                        SplitOperand::kPlanes};
   cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld * 2), static_cast<cuuint64_t>(outer * ld * 2)};
-  cuuint32_t box[3] = {static_cast<cuuint32_t>(box_inner), static_cast<cuuint32_t>(box_outer), 2};
+  cuuint32_t box[3] = {static_cast<cuuint32_t>(box_inner), static_cast<cuuint32_t>(box_outer),
+                       SplitOperand::kPlanes};
   cuuint32_t es[3] = {1, 1, 1};
-  return encode_fn()(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(ptr), dims, strides,
+  return encode_fn()(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides,
                      box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }

@@ -12,19 +12,17 @@
 //           the on-the-fly scores).
 //
 // All products are "NT" (C = A B^T, the reduction index contiguous in both
-// operands) on the pair kernel of square.cu, whose operands are fp16 hi + lo
-// planes with per-row scales: every matrix of the iteration is split once, by
-// the pass that also symmetrises it (the product takes the row and column
-// maxima that pass scales by), or by the product itself (T).  Products of the
-// iteration are symmetric in exact arithmetic; each update is re-symmetrised
-// so that rounding cannot build up an antisymmetric part.
+// operands) on the pair kernel of square.cu, whose operands are three bf16
+// planes: every matrix of the iteration is split once, by the pass that also
+// symmetrises it, or by the product itself (T).  Products of the iteration are
+// symmetric in exact arithmetic; each update is re-symmetrised so that rounding
+// cannot build up an antisymmetric part.
 //
 // Measured (one GB300, n = 1024, 12 updates at K = 3072): 17.4 ms per fit and
 // power with tf32 parts on single CTAs, K slices through partial sums in
-// memory and separate transpose / symmetrise / norm passes; 5.4 ms as here.
-// Per update: 34 / 51 / 395 us at K = 256 / 1024 / 3072 (58 / 97 / 425 us with a
-// launch for every product and pass and T split by a pass of its own, entry by
-// entry).
+// memory and separate transpose / symmetrise / norm passes; 8.2 ms as here.
+// Per update: 63 / 116 / 1220 us at K = 256 / 1024 / 3072 before, 34 / 66 / 653
+// here.
 
 #include <algorithm>
 
@@ -56,17 +54,15 @@ __global__ void mixed_trace_kernel(const float* __restrict__ r1, const float* __
 }
 
 // Row i of out = lam R1 + (1 - lam) R2 + damping * trace / K * I (R2 may be
-// null: R1 + ...), its largest |entry| (float bits) and its compensated sum of
-// squares.  One CTA per row (grid stride).
+// null: R1 + ...) and its compensated sum of squares.  One CTA per row (grid
+// stride).
 __global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
                                                   const float* __restrict__ r2, int64_t ld, int K,
                                                   float lam, float damping,
                                                   const float* __restrict__ scal,
                                                   float* __restrict__ out,
-                                                  uint32_t* __restrict__ rmax,
                                                   float* __restrict__ part) {
-  __shared__ float red_s[8];
-  __shared__ uint32_t red_m[8];
+  __shared__ float red[8];
   const float d = damping * scal[0] / static_cast<float>(K);
   for (int i = blockIdx.x; i < K; i += gridDim.x) {
     const float4* a = reinterpret_cast<const float4*>(r1 + static_cast<int64_t>(i) * ld);
@@ -74,7 +70,6 @@ __global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
         r2 != nullptr ? reinterpret_cast<const float4*>(r2 + static_cast<int64_t>(i) * ld) : nullptr;
     float4* o = reinterpret_cast<float4*>(out + static_cast<int64_t>(i) * K);
     float s = 0.0f, comp = 0.0f;
-    uint32_t m = 0u;
     for (int j = threadIdx.x; j < K / 4; j += 256) {
       float4 v = a[j];
       if (b != nullptr) {
@@ -91,8 +86,6 @@ __global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
         if ((i & 3) == 3) v.w += d;
       }
       o[j] = v;
-      m = max(max(m, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
-              max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
       const float y = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w - comp;
       const float t = s + y;
       comp = (t - s) - y;
@@ -100,22 +93,13 @@ __global__ void __launch_bounds__(256) mix_kernel(const float* __restrict__ r1,
     }
 #pragma unroll
     for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-    m = __reduce_max_sync(0xffffffffu, m);
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-      red_s[threadIdx.x >> 5] = s;
-      red_m[threadIdx.x >> 5] = m;
-    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
       float t = 0.0f;
-      uint32_t mm = 0u;
-      for (int w = 0; w < 8; ++w) {
-        t += red_s[w];
-        mm = max(mm, red_m[w]);
-      }
+      for (int w = 0; w < 8; ++w) t += red[w];
       part[i] = t;
-      rmax[i] = mm;
     }
   }
 }
@@ -169,26 +153,18 @@ __global__ void __launch_bounds__(1024) frob_norm_kernel(const float* part, int 
   }
 }
 
-// The first iterate without products: Y0 = R / c (in place in y), its row
-// maxima rescaled the same way, and t = T0^T = 1.5 I - 0.5 Y0 (Z0 = I) with its
-// row and column maxima (cleared before) and, per tile, the sum of
-// (T0 - I)^2.  64 x 64 tiles.
+// The first iterate without products: Y0 = R / c (in place in y), t = T0^T =
+// 1.5 I - 0.5 Y0 (Z0 = I) and, per tile, the sum of (T0 - I)^2.  64 x 64 tiles.
 __global__ void __launch_bounds__(256) ns_first_kernel(float* __restrict__ y, int K,
                                                        const float* __restrict__ scal,
-                                                       uint32_t* __restrict__ ymax,
                                                        float* __restrict__ t,
-                                                       uint32_t* __restrict__ rmax,
-                                                       uint32_t* __restrict__ cmax,
                                                        float* __restrict__ part) {
-  __shared__ uint32_t scol[64];
   __shared__ float red[8];
   griddep_launch_dependents();
   griddep_wait();
   const float inv_c = scal[2];
   const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x < 64) scol[threadIdx.x] = 0u;
-  __syncthreads();
   float s = 0.0f;
   float v[16];
 #pragma unroll
@@ -196,39 +172,22 @@ __global__ void __launch_bounds__(256) ns_first_kernel(float* __restrict__ y, in
     const int i = i0 + w + 8 * (k >> 1), j = j0 + lane + 32 * (k & 1);
     v[k] = (i < K && j < K) ? y[static_cast<int64_t>(i) * K + j] * inv_c : 0.0f;
   }
-  uint32_t cm[2] = {0u, 0u};
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = i0 + w + 8 * r;
-    uint32_t m = 0u;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = j0 + lane + 32 * h;
-      if (i < K && j < K) {
-        const int64_t e = static_cast<int64_t>(i) * K + j;
-        y[e] = v[2 * r + h];
-        const float u = (i == j ? 1.5f : 0.0f) - 0.5f * v[2 * r + h];
-        t[e] = u;
-        const float d = u - (i == j ? 1.0f : 0.0f);
-        s += d * d;
-        const uint32_t b = __float_as_uint(u) & 0x7fffffffu;
-        m = max(m, b);
-        cm[h] = max(cm[h], b);
-      }
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0 && i < K) {
-      atomicMax(&rmax[i], m);
-      if (j0 == 0) ymax[i] = __float_as_uint(__uint_as_float(ymax[i]) * inv_c);
+  for (int k = 0; k < 16; ++k) {
+    const int i = i0 + w + 8 * (k >> 1), j = j0 + lane + 32 * (k & 1);
+    if (i < K && j < K) {
+      const int64_t e = static_cast<int64_t>(i) * K + j;
+      y[e] = v[k];
+      const float u = (i == j ? 1.5f : 0.0f) - 0.5f * v[k];
+      t[e] = u;
+      const float d = u - (i == j ? 1.0f : 0.0f);
+      s += d * d;
     }
   }
-  atomicMax(&scol[lane], cm[0]);
-  atomicMax(&scol[lane + 32], cm[1]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) red[w] = s;
   __syncthreads();
-  if (threadIdx.x < 64 && j0 + threadIdx.x < K) atomicMax(&cmax[j0 + threadIdx.x], scol[threadIdx.x]);
   if (threadIdx.x == 0) {
     float a = 0.0f;
     for (int x = 0; x < 8; ++x) a += red[x];
@@ -251,27 +210,25 @@ int64_t split_ld(int64_t K) { return (K + 7) / 8 * 8; }
 
 // Carves a split operand of `rows` rows of K entries out of ws at *off.
 size_t split_bytes(int64_t rows, int64_t K) {
-  return round_up256(2 * static_cast<size_t>(rows) * split_ld(K) * sizeof(__half)) +
-         round_up256(static_cast<size_t>(rows) * sizeof(int));
+  return round_up256(SplitOperand::kPlanes * static_cast<size_t>(rows) * split_ld(K) *
+                     sizeof(__nv_bfloat16));
 }
 SplitOperand take_split(uint8_t* ws, size_t* off, int rows, int K) {
   SplitOperand o;
   o.rows = rows;
   o.K = K;
   o.ld = split_ld(K);
-  o.planes = reinterpret_cast<__half*>(ws + *off);
-  o.exps = reinterpret_cast<int*>(
-      ws + *off + round_up256(2 * static_cast<size_t>(rows) * o.ld * sizeof(__half)));
+  o.planes = reinterpret_cast<__nv_bfloat16*>(ws + *off);
   *off += split_bytes(rows, K);
   return o;
 }
 
-// T = 1.5 I - 0.5 Z Y has its spectrum in [1, 1.5] (in [1.5 - cond/2, 1.5] at
-// worst before an iteration diverges), so its rows' maxima are known without
-// looking: entries up to 127 fit in fp16 at this exponent, and an entry's lo
-// part is exact to 2^-34, far below the 2^-24 of T's diagonal.  So the product
-// itself writes the splits of T and T^T, with no fp32 T and no pass over it.
-constexpr int kTExp = 9;
+// The Z and Y products of an update go in one launch, which takes a matrix more
+// of workspace, while one of them leaves half the SMs idle (25 of 256 x 256 tiles
+// for 76 clusters at K = 1280).  From there on they follow each other, and the Y
+// product's result takes the room of T, which only the Z product reads.
+constexpr int kTogetherK = 1280;
+bool zy_together(int64_t K) { return K <= kTogetherK; }
 
 // Iterates enqueued between two read-backs of their residuals.  Everything after
 // the first one within the tolerance finds the stop flag set and does nothing,
@@ -290,7 +247,7 @@ size_t part_floats(int64_t K) {
 }  // namespace
 
 size_t fisher_fit_workspace(int64_t n, int64_t K) {
-  return split_bytes(K, n) + round_up256(static_cast<size_t>(K) * sizeof(uint32_t));
+  return split_bytes(K, n);
 }
 
 cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* r, int64_t ldr,
@@ -298,8 +255,7 @@ cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* 
   uint8_t* base = reinterpret_cast<uint8_t*>(ws);
   size_t off = 0;
   const SplitOperand xt = take_split(base, &off, K, n);
-  uint32_t* cmax = reinterpret_cast<uint32_t*>(base + off);
-  const cudaError_t e = launch_transpose_split(x, n, K, ldx, cmax, xt, s);
+  const cudaError_t e = launch_transpose_split(x, n, K, ldx, xt, s);
   if (e != cudaSuccess) return e;
   SquareArgs a;
   a.x = xt;
@@ -314,7 +270,7 @@ cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* 
 
 size_t fisher_power_workspace(int64_t K) {
   const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
-  return 2 * kk + 4 * split_bytes(K, K) + round_up256(9 * static_cast<size_t>(K) * sizeof(uint32_t)) +
+  return (zy_together(K) ? 2 : 1) * kk + 4 * split_bytes(K, K) +
          round_up256(part_floats(K) * sizeof(float)) + kScalBytes;
 }
 
@@ -322,59 +278,51 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
                                 float damping, int inverse, int iterations, float tol,
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
                                 float* ws, int* status, int sms, cudaStream_t s) {
-  // Two fp32 matrices (the Z and Y products) and the splits of Z, Y, T and T^T.
+  // The splits of Z, Y, T and T^T and the fp32 Z and Y products.
   uint8_t* base = reinterpret_cast<uint8_t*>(ws);
   const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
-  float* yf = reinterpret_cast<float*>(base);
-  float* zf = reinterpret_cast<float*>(base + kk);
-  size_t off = 2 * kk;
+  size_t off = 0;
   const SplitOperand zs = take_split(base, &off, K, K);
   const SplitOperand ys = take_split(base, &off, K, K);
-  SplitOperand ts = take_split(base, &off, K, K);
-  SplitOperand tts = take_split(base, &off, K, K);
-  ts.exps = tts.exps = nullptr;
-  ts.exp0 = tts.exp0 = kTExp;
-  // Maxima in two slots: rows and columns of the Z product, then of the Y
-  // product (K words each).  The T product between two uses of a slot clears it.
-  uint32_t* maxima = reinterpret_cast<uint32_t*>(base + off);
-  uint32_t* ymax = maxima + 8 * static_cast<int64_t>(K);      // row maxima of R, then of Y0
-  const size_t max_bytes = 9 * static_cast<size_t>(K) * sizeof(uint32_t);
-  off += round_up256(max_bytes);
+  const SplitOperand ts = take_split(base, &off, K, K);
+  const SplitOperand tts = take_split(base, &off, K, K);
+  float* zf = reinterpret_cast<float*>(base + off);
+  off += kk;
+  const bool together = zy_together(K);
+  float* yf = reinterpret_cast<float*>(ts.planes);
+  if (together) {
+    yf = reinterpret_cast<float*>(base + off);
+    off += kk;
+  }
   float* part = reinterpret_cast<float*>(base + off);
   off += round_up256(part_floats(K) * sizeof(float));
   float* scal = reinterpret_cast<float*>(base + off);  // trace, c, 1/c, 1/sqrt(c), 1/c, -, stop
   int* stop = reinterpret_cast<int*>(scal + 6);
-  auto slot = [&](int it) { return maxima + 4 * static_cast<int64_t>(it & 1) * K; };
-  auto product = [&](const SplitOperand& x, const SplitOperand& y, float* c, uint32_t* max) {
+  auto product = [&](const SplitOperand& x, const SplitOperand& y, float* c) {
     SquareArgs a;
     a.x = x;
     a.y = y;
     a.c = c;
     a.ldc = K;
-    a.row_max = max;
-    a.col_max = max + K;
     a.stop = stop;
     a.status = status;
     return a;
   };
-  auto sym_pass = [&](const float* c, const uint32_t* max, const SplitOperand& o) {
+  auto sym_pass = [&](const float* c, const SplitOperand& o) {
     SquarePassArgs a;
     a.c = c;
-    a.rmax = max;
-    a.cmax = max + K;
     a.sym = o;
     return a;
   };
   const bool track = residuals != nullptr || tol > 0.0f;
   if (iterations_done != nullptr) *iterations_done = 0;
-  cudaError_t e = cudaMemsetAsync(maxima, 0, max_bytes, s);
-  if (e != cudaSuccess) return e;
   mixed_trace_kernel<<<1, 1024, 0, s>>>(r1, r2, ldr, K, lam, scal);
-  mix_kernel<<<std::min(K, 4096), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, yf, ymax, part);
+  mix_kernel<<<std::min(K, 4096), 256, 0, s>>>(r1, r2, ldr, K, lam, damping, scal, yf, part);
   frob_final_kernel<<<1, 1024, 0, s>>>(part, K, scal, stop);
   const int t64 = (K + 63) / 64;
-  ns_first_kernel<<<dim3(t64, t64), 256, 0, s>>>(yf, K, scal, ymax, zf, slot(0), slot(0) + K, part);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  ns_first_kernel<<<dim3(t64, t64), 256, 0, s>>>(yf, K, scal, zf, part);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   const int n_part = square_part_count(K, K, sms);
   int updates = 0;               // updates applied (Z is still I at 0)
   int read = 0;                  // residuals read back
@@ -401,8 +349,6 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
       t.gamma = 1.5f;
       t.row_out = ts;
       t.col_out = tts;
-      t.zero_next = slot(it);              // read last by the passes of update it - 2
-      t.n_zero = 4 * K;
       t.part = track ? part : nullptr;
       t.stop = stop;
       t.status = status;
@@ -436,25 +382,24 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
         if (done) break;
       }
     }
-    uint32_t* mx = slot(it);
     if (it == 0) {
       // zf holds T0^T, and Z1 = T0: no product; Y1 = Y0 T0
       SquarePassArgs a[2];
-      a[0] = sym_pass(zf, mx, zs);
+      a[0] = sym_pass(zf, zs);
       a[0].row = tts;
       a[1].c = yf;
-      a[1].rmax = a[1].cmax = ymax;
       a[1].row = ys;
-      const SquareArgs y1 = product(ys, tts, yf, mx + 2 * K);
-      const SquarePassArgs yp = sym_pass(yf, mx + 2 * K, ys);
+      const SquareArgs y1 = product(ys, tts, yf);
+      const SquarePassArgs yp = sym_pass(yf, ys);
       if ((e = launch_square_pass(a, 2, K, stop, s)) != cudaSuccess ||
           (e = launch_square(&y1, 1, sms, s)) != cudaSuccess ||
           (e = launch_square_pass(&yp, 1, K, stop, s)) != cudaSuccess)
         return e;
     } else {
-      const SquareArgs zy[2] = {product(ts, zs, zf, mx), product(ys, tts, yf, mx + 2 * K)};
-      const SquarePassArgs ps[2] = {sym_pass(zf, mx, zs), sym_pass(yf, mx + 2 * K, ys)};
-      if ((e = launch_square(zy, 2, sms, s)) != cudaSuccess ||
+      const SquareArgs zy[2] = {product(ts, zs, zf), product(ys, tts, yf)};
+      const SquarePassArgs ps[2] = {sym_pass(zf, zs), sym_pass(yf, ys)};
+      if ((e = launch_square(zy, together ? 2 : 1, sms, s)) != cudaSuccess ||
+          (!together && (e = launch_square(zy + 1, 1, sms, s)) != cudaSuccess) ||
           (e = launch_square_pass(ps, 2, K, stop, s)) != cudaSuccess)
         return e;
     }

@@ -278,13 +278,11 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
                                 float* ws, int* status, int sms, cudaStream_t s);
 
 // Square fp32-accurate products (square.cu).  An operand of `rows` rows of K
-// entries, split into two fp16 planes (hi rows, then lo rows; leading
-// dimension ld, a multiple of 8) with a power-of-two scale per row:
-// entry = 2^-exps[row] (hi + lo).
+// entries, split into three bf16 planes (`rows` rows each, leading dimension ld, a
+// multiple of 8) whose sum is the entry.
 struct SplitOperand {
-  __half* planes = nullptr;
-  int* exps = nullptr;             // [rows], or nullptr: exp0 for every row
-  int exp0 = 0;
+  static constexpr int kPlanes = 3;
+  __nv_bfloat16* planes = nullptr;
   int rows = 0;
   int K = 0;
   int64_t ld = 0;
@@ -296,27 +294,21 @@ struct SquareArgs {
   const float* alpha_s = nullptr;  // alpha' = alpha * (*alpha_s) when given
   float gamma = 0.0f;
   float* c = nullptr;              // [x.rows, ldc], or nullptr: C goes to the splits of its rows
-  int64_t ldc = 0;                 //   and columns (at their exp0; x.rows and y.rows multiples
-  SplitOperand row_out, col_out;   //   of 4)
-  uint32_t* row_max = nullptr;     // max |C[b, :]| and max |C[:, q]| as float bits (cleared
-  uint32_t* col_max = nullptr;     //   before the launch), or both nullptr
-  uint32_t* zero_next = nullptr;   // n_zero words to clear for later products
-  int n_zero = 0;
+  int64_t ldc = 0;                 //   and columns (x.rows and y.rows multiples of 4)
+  SplitOperand row_out, col_out;
   const int* stop = nullptr;       // device flag: nonzero = compute and write nothing
   float* part = nullptr;           // square_part_floats() sums of (C - I)^2, or nullptr
   int* status = nullptr;
 };
 // One product, or two of the same shape, alpha, gamma and ldc (a[1] gives its
-// operands, c and maxima only).
+// operands and c only).
 cudaError_t launch_square(const SquareArgs* a, int n, int sms, cudaStream_t s);
 int64_t square_part_floats(int M, int N);         // the most sums `part` may receive
 int square_part_count(int M, int N, int sms);     // the sums one plain product writes there
-// One or two passes over K x K matrices c (row and column maxima given): the
-// splits of the rows and / or of the symmetric part.
+// One or two passes over K x K matrices c: the splits of the rows and / or of the
+// symmetric part.
 struct SquarePassArgs {
   const float* c = nullptr;
-  const uint32_t* rmax = nullptr;
-  const uint32_t* cmax = nullptr;
   SplitOperand row, sym;           // planes == nullptr: not written
 };
 cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int* stop,
@@ -324,8 +316,8 @@ cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int*
 // m = (c + c^T) / 2 * (*scale)
 cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
                                    int64_t ldm, cudaStream_t s);
-// The split of x^T from x [n, ldx]; cmax: K words of scratch.
-cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx, uint32_t* cmax,
+// The split of x^T from x [n, ldx].
+cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx,
                                    const SplitOperand& o, cudaStream_t s);
 
 // Skinny fp32 product C[b, q] = <x_b, y_q> on the tensor cores (on-the-fly
@@ -372,8 +364,8 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s);
 CUresult encode_tmap_2d(CUtensorMap* tm, CUtensorMapDataType dt, const void* ptr, int64_t inner,
                         int64_t outer, int64_t row_bytes, int box_inner, int box_outer);
 
-// 3-D tiled tensor map of a split operand's two fp16 planes, box {box_inner,
-// box_outer, 2}, 128-byte swizzle.
+// 3-D tiled tensor map of a split operand's planes, box {box_inner, box_outer,
+// planes}, 128-byte swizzle.
 CUresult encode_tmap_planes(CUtensorMap* tm, const void* ptr, int64_t inner, int64_t outer,
                             int64_t ld, int box_inner, int box_outer);
 

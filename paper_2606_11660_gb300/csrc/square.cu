@@ -1,30 +1,28 @@
 // Square products of the Fisher preconditioner (C[b, q] = <x_b, y_q> for two
 // operands of thousands of rows, fp32 accuracy) on the tensor cores.
 //
-// Operands are split once, by the pass that writes them, into two fp16 planes
-// with a power-of-two scale per row:
-//   x_b = 2^-e_b (hi + lo),  e_b such that max |x_b| 2^e_b lies in [2^14, 2^15),
-//   hi = fp16(x 2^e), lo = fp16(x 2^e - hi)        (both rounded to nearest),
-// which leaves |x - hi - lo| <= 2^-23 |x|, or 2^-40 of the row's largest entry
-// where lo becomes subnormal, and the product is taken as
-//   <x, y> ~= <x_lo, y_hi> + <x_hi, y_lo> + <x_hi, y_hi>,
-// the three-product scheme of Ootomo and Yokota (2022) with fp16 parts.  fp16
-// parts hold the same 11 + 11 bits as tf32 parts, at twice the MMA rate, half
-// the operand bytes (4 per entry for both planes) and half as many truncating
-// accumulations per column.
+// Operands are split once, by the pass that writes them, into three bf16 planes
+//   x = x0 + x1 + x2,  x0 = bf16(x), x1 = bf16(x - x0), x2 = bf16(x - x0 - x1)
+// (each rounded to nearest), which hold all 24 bits of every entry at any
+// magnitude, and the product is taken as the six terms down to 2^-16,
+//   <x, y> ~= <x0, y0> + <x0, y1> + <x1, y0> + <x1, y1> + <x0, y2> + <x2, y0>
+// (Ootomo and Yokota 2022 with bf16 parts; what is left out is below 2^-25).
+// Two fp16 planes with a scale per row take half the MMAs, but keep those bits
+// only down to 2^-17 of a row's largest entry: entries of M = R^-1/2 that are
+// small beside the diagonal (columns of R that differ by e^4: half of them) lost
+// every digit.
 //
 // Bound: the tensor pipe.  CTA pairs take 256 x 256 output tiles (M = 256 rows
 // of y over the pair, N = 256 rows of x, K = 16 per MMA): a 64-column stage is
-// 64 KB per CTA for 12 MMAs of 128 cycles, 43 bytes of L2 reads per SM and
-// cycle, and 104 of the 128 bytes of shared-memory bandwidth (operand reads 64,
-// TMA writes 40), which a single-CTA 128 x 256 tile (160 with its reads) would
-// not fit.
+// 96 KB per CTA for 24 MMAs of 128 cycles, 32 bytes of L2 reads per SM and cycle.
+// A Newton-Schulz update (three products and their passes) at K = 256 / 1024 /
+// 3072: 34 / 66 / 653 us; 35 / 52 / 408 with two fp16 planes.
 //
 // The tensor cores' fp32 accumulation rounds toward zero, so an accumulation
-// chain covers at most kChainStages 64-column stages (48 MMAs, the small lo
-// terms of each 16 columns first); the epilogue adds the chains in registers
-// with IEEE adds, in order, while the next chain runs in the other half of
-// TMEM.  No partial sums go to memory.
+// chain is one stage or half of one, its smallest terms first: four MMAs (two)
+// round a sum of full size.  The epilogue adds the chains in registers with IEEE
+// adds, in order, while the next chain runs in the other half of TMEM.  No
+// partial sums go to memory.
 
 #include <algorithm>
 
@@ -36,8 +34,14 @@ namespace bergson {
 namespace {
 
 constexpr int kSqM = 256;                 // rows of y per tile (128 per CTA)
-constexpr int kSqK = 64;                  // fp16 columns per stage: one 128-byte row
-constexpr int kChainStages = 4;           // stages per accumulation chain
+constexpr int kSqK = 64;                  // bf16 columns per stage: one 128-byte row
+constexpr int kPlanes = SplitOperand::kPlanes;
+// Columns up to which a stage is two accumulation chains of 32 columns: there a
+// chain is a larger part of the sum.  M = R^-1/2 of K columns of unequal scale
+// (e^1), error against fp64 as a multiple of that with tf32 parts and chains of 32
+// columns or more, one chain / two: K = 128 1.28 / 0.79, 384 1.64 / 0.91, 512 0.89 /
+// 0.53, 1024 0.2.  Two cost 42 -> 48 us an update at K = 512, 66 -> 78 at K = 1024.
+constexpr int kShortChainK = 512;
 constexpr int kSqThreads = 64 + 256;      // producer, MMA, 8 epilogue warps
 constexpr int kSqBarBytes = 256;
 constexpr int kSqSmemBudget = 232448;
@@ -48,8 +52,8 @@ constexpr uint64_t kSqDrainTimeoutNs = 2000000000ull;
 template <int TN_>
 struct SqCfg {
   static constexpr int TN = TN_;                           // rows of x per tile
-  static constexpr int kABytes = 2 * 128 * 128;            // y: hi and lo planes, 128 rows
-  static constexpr int kBBytes = 2 * (TN / 2) * 128;       // x: this CTA's half of the N side
+  static constexpr int kABytes = kPlanes * 128 * 128;      // y: 128 rows of each plane
+  static constexpr int kBBytes = kPlanes * (TN / 2) * 128; // x: this CTA's half of the N side
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kStages = (kSqSmemBudget - 1024 - kSqBarBytes - kOutBytes) / kStageBytes;
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kSqBarBytes + kOutBytes;
@@ -57,19 +61,10 @@ struct SqCfg {
   static constexpr int kCols = TN / 2;                     // accumulator columns per epilogue warp
 };
 
-// One product of a launch (a launch runs one or two of the same shape).
-struct SqProblem {
-  const int* ey;             // [M] scale exponents of y's rows, or nullptr: exp0_y for all
-  const int* ex;             // [N] likewise of x's rows
-  int exp0_y, exp0_x;
-  float* c;                  // [N, ldc]; nullptr: the splits below instead
-  uint32_t* row_max;         // [N] / [M] maxima of |C| over each b / each q (float bits), or
-  uint32_t* col_max;         //   nullptr
-};
-
 struct SqParams {
-  SqProblem pr[2];
-  int n_prob;
+  float* c[2];               // [N, ldc] of each product; nullptr: the splits below instead
+  int n_prob;                // products of the launch (one, or two of the same shape)
+  int chains;                // accumulation chains per stage, 1 or 2
   int M, N, K;               // rows of y (q), rows of x (b), columns
   int n_mt, n_nt;            // tiles
   int n_tiles;               // of one product
@@ -78,9 +73,7 @@ struct SqParams {
   const float* alpha_s;      // or nullptr
   float gamma;               // added on the diagonal
   int64_t ldc;
-  SplitOperand row, col;     // splits of C's rows and columns at their exp0 (c == nullptr)
-  uint32_t* zero_next;       // words cleared for later products, or nullptr
-  int n_zero;
+  SplitOperand row, col;     // splits of C's rows and columns (c == nullptr)
   const int* stop;           // nonzero: nothing is computed or written (nullptr: never)
   float* part;               // [n_tiles, 16] sums of (C - I)^2 per tile and epilogue warp, or nullptr
   int* status;
@@ -111,7 +104,7 @@ __device__ __forceinline__ void tile_of(const SqParams& p, int i, int* mt, int* 
   *nt = r / gm;
 }
 
-// TMA load of a {64 columns, rows, 2 planes} box for a CTA pair's barrier.
+// TMA load of a {64 columns, rows, planes} box for a CTA pair's barrier.
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap, uint32_t bar,
                                                  int c0, int c1, uint64_t policy) {
   asm volatile(
@@ -121,34 +114,30 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap,
       : "memory");
 }
 
-__device__ __forceinline__ float pow2f(int e) {     // -126 <= e <= 127
-  return __uint_as_float(static_cast<uint32_t>(e + 127) << 23);
-}
-// Scale exponent of a row whose largest |entry| has the float bits `m`: the
-// scaled maximum lies in [2^14, 2^15).  Zero rows and rows with an infinity or
-// NaN keep 0 (their products are what the entries make them).
-__device__ __forceinline__ int row_exponent(uint32_t m) {
-  if (m == 0u || m >= 0x7f800000u) return 0;
-  const int ex = max(static_cast<int>(m >> 23), 1) - 127;
-  return min(14 - ex, 120);
-}
-
-// (hi, lo) of two scaled values: hi + lo = v up to 2^-23 |v|.
-__device__ __forceinline__ void split_half2(float a, float b, __half2* hi, __half2* lo) {
-  *hi = __floats2half2_rn(a, b);
-  const float2 h = __half22float2(*hi);
-  *lo = __floats2half2_rn(a - h.x, b - h.y);
+// The planes of two values.
+__device__ __forceinline__ void split_bf16x2(float a, float b, __nv_bfloat162* out) {
+#pragma unroll
+  for (int i = 0; i < kPlanes; ++i) {
+    out[i] = __floats2bfloat162_rn(a, b);
+    const float2 h = __bfloat1622float2(out[i]);
+    a -= h.x;
+    b -= h.y;
+  }
 }
 
-// The split of v[0..3] f at columns col.. of a row (4 | col: 8-byte aligned).
-__device__ __forceinline__ void put_four(const SplitOperand& o, int row, int col, float4 v, float f) {
-  __half2 h[2], l[2];
-  split_half2(v.x * f, v.y * f, &h[0], &l[0]);
-  split_half2(v.z * f, v.w * f, &h[1], &l[1]);
-  __half* d = o.planes + static_cast<int64_t>(row) * o.ld + col;
-  *reinterpret_cast<uint2*>(d) = *reinterpret_cast<const uint2*>(h);
-  *reinterpret_cast<uint2*>(d + static_cast<int64_t>(o.rows) * o.ld) =
-      *reinterpret_cast<const uint2*>(l);
+// The split of v at columns col.. of a row (4 | col: 8-byte aligned).
+__device__ __forceinline__ void put_four(const SplitOperand& o, int row, int col, float4 v) {
+  __nv_bfloat162 lo[kPlanes], hi[kPlanes];
+  split_bf16x2(v.x, v.y, lo);
+  split_bf16x2(v.z, v.w, hi);
+  __nv_bfloat16* d = o.planes + static_cast<int64_t>(row) * o.ld + col;
+#pragma unroll
+  for (int i = 0; i < kPlanes; ++i, d += static_cast<int64_t>(o.rows) * o.ld) {
+    uint2 w;
+    w.x = *reinterpret_cast<const uint32_t*>(&lo[i]);
+    w.y = *reinterpret_cast<const uint32_t*>(&hi[i]);
+    *reinterpret_cast<uint2*>(d) = w;
+  }
 }
 
 // Writes a warp's 32 x 32 output tile (tile[j * 33 + i] = C[bc + j, q0 + i]) to
@@ -158,16 +147,15 @@ __device__ __forceinline__ void put_splits(const SqParams& p, const float* tile,
                                            int nb, int q0) {
   const int l4 = 4 * (lane & 7);
   const int nq = min(32, p.M - q0);
-  const float sr = pow2f(p.row.exp0), sc = pow2f(p.col.exp0);
 #pragma unroll 2
   for (int j = lane >> 3; j < 32; j += 4) {
     if (j < nb && l4 < nq) {                       // row bc + j of C, columns q0 + l4, ..
       const float* v = tile + j * 33 + l4;
-      put_four(p.row, bc + j, q0 + l4, make_float4(v[0], v[1], v[2], v[3]), sr);
+      put_four(p.row, bc + j, q0 + l4, make_float4(v[0], v[1], v[2], v[3]));
     }
     if (j < nq && l4 < nb) {                       // column q0 + j of C, rows bc + l4, ..
       const float* v = tile + l4 * 33 + j;
-      put_four(p.col, q0 + j, bc + l4, make_float4(v[0], v[33], v[66], v[99]), sc);
+      put_four(p.col, q0 + j, bc + l4, make_float4(v[0], v[33], v[66], v[99]));
     }
   }
 }
@@ -177,6 +165,25 @@ __device__ __forceinline__ bool sq_warp_wait(uint32_t bar, uint32_t parity, uint
   bool ok = true;
   if ((threadIdx.x & 31) == 0) ok = mbar_wait_inline(bar, parity, tmo, abort_flag);
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+}
+
+// The MMAs of one chain of 16 kMmas columns, the terms y_i x_j smallest first
+// (descriptors hold addresses in 16 bytes: 16 bf16 = 2).  Unrolled: in a loop an
+// MMA of N = 128 is issued later than the pipe could take it (K = 1024: 64 -> 80 us
+// an update).
+template <int TN, int kMmas>
+__device__ __forceinline__ void issue_chain(uint32_t d, uint64_t y, uint64_t x, uint32_t idesc) {
+  using C = SqCfg<TN>;
+  constexpr int kTerms = 6;
+  constexpr uint8_t kI[kTerms] = {2, 0, 1, 1, 0, 0}, kJ[kTerms] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+  for (int t = 0; t < kTerms; ++t) {
+    const uint64_t yi = y + kI[t] * (C::kABytes / kPlanes / 16);
+    const uint64_t xj = x + kJ[t] * (C::kBBytes / kPlanes / 16);
+#pragma unroll
+    for (int kk = 0; kk < kMmas; ++kk)
+      umma_f16_pair(d, yi + 2 * kk, xj + 2 * kk, idesc, t != 0 || kk != 0);
+  }
 }
 
 // C[b, q] = alpha' <x_b, y_q> + gamma [b == q] over persistent CTA pairs.
@@ -228,15 +235,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
     tmem_alloc_pair(smem_u32(s_tmem), C::kTmemCols);
     tmem_relinquish_pair();
   }
-  griddep_wait();                // operands, exponents and maxima come from earlier grids
+  griddep_wait();                // the operands come from earlier grids
   tc_fence_before();
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
   const uint64_t tmo = p.timeout_ns;
-  if (p.zero_next != nullptr)
-    for (int i = blockIdx.x * kSqThreads + threadIdx.x; i < p.n_zero; i += gridDim.x * kSqThreads)
-      p.zero_next[i] = 0u;
   const int n_all = p.stop != nullptr && *p.stop != 0 ? 0 : p.n_prob * p.n_tiles;
 
   if (warp == 0) {
@@ -287,38 +291,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA)
     if (rank == 0 && lane == 0) {
-      const uint32_t idesc = make_idesc_f16(kSqM, TN, false);
+      const uint32_t idesc = make_idesc_f16(kSqM, TN, true);
       int stage = 0;
       uint32_t ph = 0;
       int ab = 0;
       uint32_t aph = 0;
       bool ok = true;
       for (int t = cid; t < n_all && ok; t += n_cl) {
-        for (int c0 = 0; c0 < nK && ok; c0 += kChainStages) {
-          const int c1 = min(nK, c0 + kChainStages);
-          if (!mbar_wait(smem_u32(&tempty[ab]), aph ^ 1, tmo, s_abort)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t d = tmem + ab * TN;
-          for (int kc = c0; kc < c1; ++kc) {
-            if (!mbar_wait(smem_u32(&full[stage]), ph, tmo, s_abort)) { ok = false; break; }
+        for (int kc = 0; kc < nK; ++kc) {
+          if (!mbar_wait(smem_u32(&full[stage]), ph, tmo, s_abort)) { ok = false; break; }
+          const uint32_t sa = sbase + stage * C::kStageBytes;
+          const uint64_t y = sw128_desc(sa), x = sw128_desc(sa + C::kABytes);
+          for (int ch = 0; ch < p.chains && ok; ++ch) {
+            if (!mbar_wait(smem_u32(&tempty[ab]), aph ^ 1, tmo, s_abort)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t sa = sbase + stage * C::kStageBytes;
-            const uint64_t yh = sw128_desc(sa), yl = sw128_desc(sa + C::kABytes / 2);
-            const uint64_t xh = sw128_desc(sa + C::kABytes);
-            const uint64_t xl = sw128_desc(sa + C::kABytes + C::kBBytes / 2);
-#pragma unroll
-            for (int kk = 0; kk < kSqK / 16; ++kk) {   // 16 fp16 = 32 bytes: +2 in the address field
-              const uint64_t o = 2 * kk;
-              umma_f16_pair(d, yl + o, xh + o, idesc, kc != c0 || kk != 0);
-              umma_f16_pair(d, yh + o, xl + o, idesc, 1u);
-              umma_f16_pair(d, yh + o, xh + o, idesc, 1u);
-            }
-            umma_commit_pair(smem_u32(&empty[stage]), 0x3);
-            if (++stage == C::kStages) { stage = 0; ph ^= 1; }
+            const uint32_t d = tmem + ab * TN;
+            if (p.chains == 1) issue_chain<TN, kSqK / 16>(d, y, x, idesc);
+            else issue_chain<TN, kSqK / 32>(d, y + kSqK / 16 * ch, x + kSqK / 16 * ch, idesc);
+            if (ch == p.chains - 1) umma_commit_pair(smem_u32(&empty[stage]), 0x3);
+            umma_commit_pair(smem_u32(&tfull[ab]), 0x3);
+            if (++ab == 2) { ab = 0; aph ^= 1; }
           }
-          if (!ok) break;
-          umma_commit_pair(smem_u32(&tfull[ab]), 0x3);
-          if (++ab == 2) { ab = 0; aph ^= 1; }
+          if (++stage == C::kStages) { stage = 0; ph ^= 1; }
         }
       }
       if (!ok) raise_device_error(p.status, s_abort, kStatusTimeout);
@@ -339,13 +333,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
     uint32_t aph = 0;
     bool aborted = false;
     for (int t = cid; t < n_all && !aborted; t += n_cl) {
-      const SqProblem& pr = p.pr[t >= p.n_tiles ? 1 : 0];
+      float* out = p.c[t >= p.n_tiles ? 1 : 0];
       int mt, nt;
       tile_of<TN>(p, t >= p.n_tiles ? t - p.n_tiles : t, &mt, &nt);
       float acc[C::kCols];               // 0 + v = v: the first chain lands unchanged
 #pragma unroll
       for (int j = 0; j < C::kCols; ++j) acc[j] = 0.0f;
-      for (int c0 = 0; c0 < nK; c0 += kChainStages) {
+      for (int ch = 0; ch < p.chains * nK; ++ch) {
         if (!sq_warp_wait(smem_u32(&tfull[ab]), aph, tmo, s_abort)) {
           raise_device_error(p.status, s_abort, kStatusTimeout);
           aborted = true;
@@ -374,33 +368,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
       const int q = q0 + lane;
       const bool qin = q < p.M;
       const int b0 = nt * TN + half * C::kCols;
-      const int eq = pr.ey == nullptr ? pr.exp0_y : (qin ? pr.ey[q] : 0);
-      const float uq1 = pow2f(-(eq >> 1)), uq2 = pow2f(-(eq - (eq >> 1)));
-      uint32_t cmax = 0u;
       float ssq = 0.0f, comp = 0.0f;
 #pragma unroll
       for (int c = 0; c < C::kCols; c += 32) {
         const int bc = b0 + c;
         const int nb = min(32, p.N - bc);
-        const int eb = pr.ex == nullptr ? pr.exp0_x : (lane < nb ? pr.ex[bc + lane] : 0);
-        const float ub1 = pow2f(-(eb >> 1)), ub2 = pow2f(-(eb - (eb >> 1)));
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 32; ++j) tile[j * 33 + lane] = acc[c + j];
         __syncwarp();
-        float* dst = pr.c + static_cast<int64_t>(bc) * p.ldc + q;
+        float* dst = out + static_cast<int64_t>(bc) * p.ldc + q;
 #pragma unroll 4
         for (int j = 0; j < 32; ++j, dst += p.ldc) {
-          // acc 2^-(eq + eb): both factors stay within 2^+-120, and so do the halves
-          const float f1 = uq1 * __shfl_sync(0xffffffffu, ub1, j);
-          const float f2 = uq2 * __shfl_sync(0xffffffffu, ub2, j);
           const int b = bc + j;
-          float v = al * (tile[j * 33 + lane] * f1 * f2);
+          float v = al * tile[j * 33 + lane];
           if (b == q) v += p.gamma;
           const bool in = qin && j < nb;
-          if (in && pr.c != nullptr && (!p.symmetric || b <= q)) *dst = v;
+          if (in && out != nullptr && (!p.symmetric || b <= q)) *dst = v;
           tile[j * 33 + lane] = in ? v : 0.0f;
-          cmax = max(cmax, in ? __float_as_uint(v) & 0x7fffffffu : 0u);
           const float r = in ? v - (b == q ? 1.0f : 0.0f) : 0.0f;
           const float y = r * r - comp;
           const float u = ssq + y;
@@ -408,23 +393,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
           ssq = u;
         }
         __syncwarp();
-        if (pr.c == nullptr) put_splits(p, tile, lane, bc, nb, q0);
-        if (pr.row_max != nullptr) {
-          uint32_t m = 0u;
-#pragma unroll 8
-          for (int i = 0; i < 32; ++i)
-            m = max(m, __float_as_uint(tile[lane * 33 + i]) & 0x7fffffffu);
-          if (lane < nb) atomicMax(&pr.row_max[bc + lane], m);
-        }
+        if (out == nullptr) put_splits(p, tile, lane, bc, nb, q0);
         if (p.symmetric && lane < nb) {                 // the mirror image C[q, b], b < q
-          float* mir = pr.c + static_cast<int64_t>(q0) * p.ldc + bc + lane;
+          float* mir = out + static_cast<int64_t>(q0) * p.ldc + bc + lane;
           const int nq = min(32, p.M - q0);
 #pragma unroll 4
           for (int i = 0; i < nq; ++i, mir += p.ldc)
             if (bc + lane < q0 + i) *mir = tile[lane * 33 + i];
         }
       }
-      if (pr.col_max != nullptr && qin) atomicMax(&pr.col_max[q], cmax);
       if (p.part != nullptr) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
@@ -445,43 +422,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
 
 constexpr int kPassTile = 64;
 
-// Writes 64 values of one row of a split operand, two per lane, scaled by
-// f = 2^e (|e| <= 120: exact).
+// Writes 64 values of one row of a split operand, two per lane.
 __device__ __forceinline__ void put_row(const SplitOperand& o, int row, int col0, int lane, float a,
-                                        float b, float f) {
+                                        float b) {
   const int c = col0 + 2 * lane;
   if (row >= o.rows || c >= o.K) return;
-  __half2 h, l;
-  split_half2(a * f, b * f, &h, &l);
-  __half* hp = o.planes + static_cast<int64_t>(row) * o.ld + c;
-  __half* lp = hp + static_cast<int64_t>(o.rows) * o.ld;
-  if (c + 1 < o.K) {
-    *reinterpret_cast<__half2*>(hp) = h;
-    *reinterpret_cast<__half2*>(lp) = l;
-  } else {
-    *hp = h.x;
-    *lp = l.x;
+  __nv_bfloat162 v[kPlanes];
+  split_bf16x2(a, b, v);
+  __nv_bfloat16* d = o.planes + static_cast<int64_t>(row) * o.ld + c;
+#pragma unroll
+  for (int i = 0; i < kPlanes; ++i, d += static_cast<int64_t>(o.rows) * o.ld) {
+    if (c + 1 < o.K) *reinterpret_cast<__nv_bfloat162*>(d) = v[i];
+    else *d = v[i].x;
   }
 }
 
-// One pass over a K x K matrix c, or two of them (grid.y), with row maxima rmax
-// and column maxima cmax (float bits), that writes the split of its rows
-// (o.row) and / or of the rows of its symmetric part (c + c^T) / 2 (o.sym;
-// scaled by the larger of the row's and the column's maximum, a bound of that
-// part's maximum).  Memory bound: 4 bytes read and 4 written per entry and
-// operand.  One CTA per pair of 64 x 64 tiles (ti <= tj); a thread takes a 4 x 4
-// block of the upper tile and the mirrored block of the lower one as eight
-// 16-byte loads, adds them across the diagonal in registers and writes both
-// 8 bytes a row and plane.  A warp's blocks are 4 x 8, so every access covers
-// whole 32-byte sectors.  Two operands at K = 3072 (151 MB): 31 us; 64 us with 64 x
-// 64 tiles transposed through shared memory entry by entry (105 instructions per
-// 64 entries).
+// One pass over a K x K matrix c, or two of them (grid.y), that writes the split
+// of its rows (o.row) and / or of the rows of its symmetric part (c + c^T) / 2
+// (o.sym).  Memory bound: 4 bytes read and 6 written per entry and operand.  One
+// CTA per pair of 64 x 64 tiles (ti <= tj); a thread takes a 4 x 4 block of the
+// upper tile and the mirrored block of the lower one as eight 16-byte loads,
+// adds them across the diagonal in registers and writes both 8 bytes a row and
+// plane.  A warp's blocks are 4 x 8, so every access covers whole 32-byte
+// sectors.
 struct SquarePass {
   const float* c;
   int64_t ldc;
   int K;
-  const uint32_t* rmax;
-  const uint32_t* cmax;
   SplitOperand row, sym;         // planes == nullptr: not written
 };
 
@@ -512,42 +479,28 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int u = 0; u < 4; ++u)
     b[u] = *reinterpret_cast<const float4*>(p.c + static_cast<int64_t>(j + u) * p.ldc + i);
-  const uint4 rmi = *reinterpret_cast<const uint4*>(p.rmax + i);
-  const uint4 cmi = *reinterpret_cast<const uint4*>(p.cmax + i);
-  const uint4 rmj = *reinterpret_cast<const uint4*>(p.rmax + j);
-  const uint4 cmj = *reinterpret_cast<const uint4*>(p.cmax + j);
   const bool lower = ti != tj;                 // on the diagonal another thread holds the mirror
   if (p.row.planes != nullptr) {
-    const uint32_t ri[4] = {rmi.x, rmi.y, rmi.z, rmi.w}, rj[4] = {rmj.x, rmj.y, rmj.z, rmj.w};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int ei = p.row.exps == nullptr ? p.row.exp0 : row_exponent(ri[u]);
-      const int ej = p.row.exps == nullptr ? p.row.exp0 : row_exponent(rj[u]);
-      put_four(p.row, i + u, j, a[u], pow2f(ei));
-      if (lower) put_four(p.row, j + u, i, b[u], pow2f(ej));
-      if (i == 0 && p.row.exps != nullptr) p.row.exps[j + u] = ej;   // the blocks at column 0
+      put_four(p.row, i + u, j, a[u]);
+      if (lower) put_four(p.row, j + u, i, b[u]);
     }
   }
   if (p.sym.planes != nullptr) {
-    const uint32_t mi[4] = {max(rmi.x, cmi.x), max(rmi.y, cmi.y), max(rmi.z, cmi.z),
-                            max(rmi.w, cmi.w)};
-    const uint32_t mj[4] = {max(rmj.x, cmj.x), max(rmj.y, cmj.y), max(rmj.z, cmj.z),
-                            max(rmj.w, cmj.w)};
-    const float4 s[4] = {
-        make_float4(a[0].x + b[0].x, a[0].y + b[1].x, a[0].z + b[2].x, a[0].w + b[3].x),
-        make_float4(a[1].x + b[0].y, a[1].y + b[1].y, a[1].z + b[2].y, a[1].w + b[3].y),
-        make_float4(a[2].x + b[0].z, a[2].y + b[1].z, a[2].z + b[2].z, a[2].w + b[3].z),
-        make_float4(a[3].x + b[0].w, a[3].y + b[1].w, a[3].z + b[2].w, a[3].w + b[3].w)};
-    const float4 t[4] = {make_float4(s[0].x, s[1].x, s[2].x, s[3].x),
-                         make_float4(s[0].y, s[1].y, s[2].y, s[3].y),
-                         make_float4(s[0].z, s[1].z, s[2].z, s[3].z),
-                         make_float4(s[0].w, s[1].w, s[2].w, s[3].w)};
+    float s[4][4];                             // s[u][v]: entry (i + u, j + v), and (j + v, i + u)
+    const float au[4][4] = {{a[0].x, a[0].y, a[0].z, a[0].w}, {a[1].x, a[1].y, a[1].z, a[1].w},
+                            {a[2].x, a[2].y, a[2].z, a[2].w}, {a[3].x, a[3].y, a[3].z, a[3].w}};
+    const float bu[4][4] = {{b[0].x, b[0].y, b[0].z, b[0].w}, {b[1].x, b[1].y, b[1].z, b[1].w},
+                            {b[2].x, b[2].y, b[2].z, b[2].w}, {b[3].x, b[3].y, b[3].z, b[3].w}};
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) s[u][v] = 0.5f * (au[u][v] + bu[v][u]);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int ei = row_exponent(mi[u]), ej = row_exponent(mj[u]);
-      put_four(p.sym, i + u, j, s[u], 0.5f * pow2f(ei));
-      if (lower) put_four(p.sym, j + u, i, t[u], 0.5f * pow2f(ej));
-      if (i == 0) p.sym.exps[j + u] = ej;
+      put_four(p.sym, i + u, j, make_float4(s[u][0], s[u][1], s[u][2], s[u][3]));
+      if (lower) put_four(p.sym, j + u, i, make_float4(s[0][u], s[1][u], s[2][u], s[3][u]));
     }
   }
 }
@@ -575,52 +528,12 @@ __global__ void __launch_bounds__(256) symmetric_scale_kernel(const float* c, in
   }
 }
 
-// cmax[k] = max over i of |x[i, k]| (float bits; cleared before).  Grid:
-// (columns / 1024, slabs of kMaxRows rows); four columns per thread (K % 4 ==
-// 0 and 16-byte aligned rows, or one column at a time).
-constexpr int kMaxRows = 16;
-__global__ void __launch_bounds__(256) column_max_kernel(const float* __restrict__ x, int n, int K,
-                                                         int64_t ldx, int vec,
-                                                         uint32_t* __restrict__ cmax) {
-  const int i0 = blockIdx.y * kMaxRows, i1 = min(n, i0 + kMaxRows);
-  if (vec) {
-    const int k = (blockIdx.x * 256 + threadIdx.x) * 4;
-    if (k >= K) return;
-    uint4 m = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int u = 0; u < kMaxRows; ++u) {
-      if (i0 + u >= i1) break;
-      const uint4 v = *reinterpret_cast<const uint4*>(x + static_cast<int64_t>(i0 + u) * ldx + k);
-      m.x = max(m.x, v.x & 0x7fffffffu);
-      m.y = max(m.y, v.y & 0x7fffffffu);
-      m.z = max(m.z, v.z & 0x7fffffffu);
-      m.w = max(m.w, v.w & 0x7fffffffu);
-    }
-    atomicMax(&cmax[k], m.x);
-    atomicMax(&cmax[k + 1], m.y);
-    atomicMax(&cmax[k + 2], m.z);
-    atomicMax(&cmax[k + 3], m.w);
-    return;
-  }
-  for (int h = 0; h < 4; ++h) {
-    const int k = blockIdx.x * 1024 + h * 256 + threadIdx.x;
-    if (k >= K) return;
-    uint32_t m = 0u;
-    for (int i = i0; i < i1; ++i)
-      m = max(m, __float_as_uint(x[static_cast<int64_t>(i) * ldx + k]) & 0x7fffffffu);
-    atomicMax(&cmax[k], m);
-  }
-}
-
 // The split of x^T (K rows of n entries) from x [n, ldx].
 __global__ void __launch_bounds__(256) transpose_split_kernel(const float* __restrict__ x, int n,
                                                               int K, int64_t ldx,
-                                                              const uint32_t* cmax,
                                                               const SplitOperand o) {
   __shared__ float s[kPassTile][kPassTile + 1];
-  __shared__ float sfac[kPassTile];
   griddep_launch_dependents();
-  griddep_wait();
   const int i0 = blockIdx.x * kPassTile, k0 = blockIdx.y * kPassTile;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float v[16];
@@ -629,18 +542,12 @@ __global__ void __launch_bounds__(256) transpose_split_kernel(const float* __res
     const int r = w + 8 * (u >> 1), cc = lane + 32 * (u & 1);
     v[u] = (i0 + r < n && k0 + cc < K) ? x[static_cast<int64_t>(i0 + r) * ldx + k0 + cc] : 0.0f;
   }
-  if (threadIdx.x < kPassTile) {
-    const int k = k0 + threadIdx.x;
-    const int e = row_exponent(k < K ? cmax[k] : 0u);
-    sfac[threadIdx.x] = pow2f(e);
-    if (i0 == 0 && k < K) o.exps[k] = e;
-  }
 #pragma unroll
   for (int u = 0; u < 16; ++u) s[w + 8 * (u >> 1)][lane + 32 * (u & 1)] = v[u];
   __syncthreads();
 #pragma unroll 4
   for (int r = w; r < kPassTile; r += 8)
-    put_row(o, k0 + r, i0, lane, s[2 * lane][r], s[2 * lane + 1][r], sfac[r]);
+    put_row(o, k0 + r, i0, lane, s[2 * lane][r], s[2 * lane + 1][r]);
 }
 
 int64_t square_tiles(int M, int N, int tn, bool symmetric) {
@@ -650,13 +557,13 @@ int64_t square_tiles(int M, int N, int tn, bool symmetric) {
 }
 
 // Tile width: the one whose rounds over the clusters cost least.  A 128-wide
-// tile is half the products of a 256-wide one but keeps shared memory busier
-// than the tensor pipe (158 bytes per cycle wanted of 128) and pays the same
-// fill and epilogue, so it counts 0.65.
+// tile is half the products of a 256-wide one but reads more of shared memory
+// per product and pays the same fill and epilogue, so it counts 0.7 (an update at
+// K = 2052, three rounds of 128 / two of 256: 449 / 442 us, at K = 2560 520 / 507).
 int square_tile_width(int M, int N, int n, int clusters, bool symmetric) {
   const int64_t r256 = (n * square_tiles(M, N, 256, symmetric) + clusters - 1) / clusters;
   const int64_t r128 = (n * square_tiles(M, N, 128, symmetric) + clusters - 1) / clusters;
-  return static_cast<double>(r128) * 0.65 < static_cast<double>(r256) ? 128 : 256;
+  return static_cast<double>(r128) * 0.7 < static_cast<double>(r256) ? 128 : 256;
 }
 
 template <int TN>
@@ -701,24 +608,15 @@ cudaError_t launch_square(const SquareArgs* a, int n, int sms, cudaStream_t s) {
   p.M = a->y.rows;
   p.N = a->x.rows;
   p.K = a->y.K;
+  p.chains = p.K <= kShortChainK ? 2 : 1;
   p.symmetric = a->symmetric ? 1 : 0;
-  for (int i = 0; i < n; ++i) {
-    p.pr[i].ey = a[i].y.exps;
-    p.pr[i].ex = a[i].x.exps;
-    p.pr[i].exp0_y = a[i].y.exp0;
-    p.pr[i].exp0_x = a[i].x.exp0;
-    p.pr[i].c = a[i].c;
-    p.pr[i].row_max = a[i].row_max;
-    p.pr[i].col_max = a[i].col_max;
-  }
+  for (int i = 0; i < n; ++i) p.c[i] = a[i].c;
   p.alpha = a->alpha;
   p.alpha_s = a->alpha_s;
   p.gamma = a->gamma;
   p.ldc = a->ldc;
   p.row = a->row_out;
   p.col = a->col_out;
-  p.zero_next = a->zero_next;
-  p.n_zero = a->n_zero;
   p.stop = a->stop;
   p.part = a->part;
   p.status = a->status;
@@ -737,8 +635,6 @@ cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int*
     pp.p[i].c = a[i].c;
     pp.p[i].ldc = K;
     pp.p[i].K = K;
-    pp.p[i].rmax = a[i].rmax;
-    pp.p[i].cmax = a[i].cmax;
     pp.p[i].row = a[i].row;
     pp.p[i].sym = a[i].sym;
   }
@@ -753,24 +649,11 @@ cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const flo
                           m, ldm);
 }
 
-cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx, uint32_t* cmax,
+cudaError_t launch_transpose_split(const float* x, int n, int K, int64_t ldx,
                                    const SplitOperand& o, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(cmax, 0, static_cast<size_t>(K) * sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
-  const int vec = ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 ? 1 : 0;
-  // n <= 2^24: at most 2^20 slabs, more than a grid's y dimension holds
-  const int slabs = (n + kMaxRows - 1) / kMaxRows;
-  for (int s0 = 0; s0 < slabs; s0 += 65535) {
-    const int cnt = std::min(65535, slabs - s0);
-    const int64_t row0 = static_cast<int64_t>(s0) * kMaxRows;
-    column_max_kernel<<<dim3((K + 1023) / 1024, cnt), 256, 0, s>>>(
-        x + row0 * ldx, static_cast<int>(n - row0), K, ldx, vec, cmax);
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   const dim3 grid((n + kPassTile - 1) / kPassTile, (K + kPassTile - 1) / kPassTile);
-  return launch_dependent(transpose_split_kernel, grid, dim3(256), 0, s, x, n, K, ldx,
-                          static_cast<const uint32_t*>(cmax), o);
+  transpose_split_kernel<<<grid, 256, 0, s>>>(x, n, K, ldx, o);
+  return cudaGetLastError();
 }
 
 }  // namespace bergson

@@ -1,8 +1,8 @@
 """Square fp32-accurate products (Fisher fit, Newton-Schulz) at tile edges.
 
-Sizes straddle the 128- and 256-row tiles, the 64-column stages and the
-256-column accumulation chains, with columns of very different scale, zero
-columns and an outlying example, against fp64.
+Sizes straddle the 128- and 256-row tiles of both kernels, the 64-column stages
+and the change from 32- to 64-column accumulation chains, with columns of very
+different scale, zero columns and an outlying example, against fp64.
 """
 import numpy as np
 import pytest
@@ -29,7 +29,8 @@ def _fit(x, pad=0):
 
 
 @pytest.mark.parametrize("n,K,pad", [(1, 4, 0), (7, 12, 4), (64, 128, 0), (65, 132, 8),
-                                     (300, 252, 0), (257, 260, 0), (130, 516, 4), (1025, 1028, 0)])
+                                     (300, 252, 0), (257, 260, 0), (130, 516, 4), (1025, 1028, 0),
+                                     (70, 3076, 0), (513, 3332, 4)])       # 256-wide tiles
 def test_fit_at_tile_edges(n, K, pad):
     g = wl.generator(n + K, "cpu")
     x = torch.randn((n, K), generator=g) * torch.logspace(-4, 4, K)
@@ -38,7 +39,8 @@ def test_fit_at_tile_edges(n, K, pad):
     R = np32(_fit(x, pad)).astype(np.float64)
     assert np.array_equal(R, R.T)
     want = orc.fisher_fit(x.numpy())
-    # per entry, against the Cauchy-Schwarz scale: both operands' 2^-23, a chain of at most 48
+    # per entry, against the Cauchy-Schwarz scale (above chains of 24 sums and n / 32 sums of
+    # chains, n / 64 from 513 on): both operands' 2^-23, a chain of at most 48
     # truncating sums of 2^-23, and n / 256 fp32 sums of chains
     d = np.sqrt(np.diag(want))
     err = np.abs(R - want) / np.maximum(np.outer(d, d), 1e-300)
@@ -57,7 +59,54 @@ def test_fit_keeps_infinities_and_nan_in_their_rows():
     assert not np.isfinite(R[bad]).any() and not np.isfinite(R[:, bad]).any()
 
 
-@pytest.mark.parametrize("K", [4, 60, 132, 260, 516])
+def test_fit_keeps_small_entries_of_a_column_with_an_outlier():
+    # example 5 is 2^36 above the rest, in the even columns only: beside it, R's entries of an even
+    # and an odd column are sums of entries 2^-36 of the column's largest
+    g = wl.generator(4, "cpu")
+    n, K = 300, 260
+    x = torch.randn((n, K), generator=g)
+    x[5] *= 2.0 ** 36
+    x[5, 1::2] = 0.0
+    R = np32(_fit(x)).astype(np.float64)[0::2, 1::2]
+    xd = x.numpy().astype(np.float64)
+    want = (xd[:, 0::2].T @ xd[:, 1::2]) / n
+    scale = np.abs(xd[:, 0::2]).T @ np.abs(xd[:, 1::2]) / n
+    # both operands' 2^-24, chains of at most 2 + 4 truncating sums, n / 32 fp32 sums of chains
+    assert (np.abs(R - want) / scale).max() <= (2 + 6 + n / 32) * 2.0 ** -23
+
+
+def _power(R, damping, iters=30):
+    K = R.shape[0]
+    M = torch.full((K, K), float("nan"), device=DEV)
+    ws = bg.workspace_tensor(bg.bergson_fisher_preconditioner_workspace(K), DEV)
+    bg.bergson_fisher_preconditioner(R.to(DEV), None, K, 1.0, damping, bg.BERGSON_FISHER_INV_SQRT,
+                                     iters, M, ws)
+    assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+    want = orc.fisher_power(orc.fisher_mix(R.numpy().astype(np.float64), None, 1.0, damping), -0.5)
+    return np32(M).astype(np.float64), want
+
+
+def test_power_keeps_entries_small_beside_the_diagonal():
+    # columns of R spread over e^+-8: half of M's entries lie below 1e-6 of sqrt(M_ii M_jj)
+    g = wl.generator(40, "cpu")
+    K = 256
+    x = torch.randn((3 * K, K), generator=g).double() * torch.exp(
+        4 * torch.randn((1, K), generator=g).double())
+    M, want = _power((x.T @ x / (3 * K)).float(), 0.1)
+    assert np.median(np.abs(M - want) / np.abs(want)) < 1e-3     # 7e-5 with tf32 parts
+
+
+@pytest.mark.parametrize("K", [128, 256, 512])
+def test_power_error_at_small_K(K):
+    g = wl.generator(41 + K, "cpu")
+    x = torch.randn((3 * K, K), generator=g)
+    M, want = _power((x.T @ x / (3 * K)).float(), 0.1)
+    # a product is off by at most 4 truncations of 2^-23 (a chain's two and the terms before them),
+    # an update by three products', and sqrt(cond R) = 3.7 is the iteration's amplification
+    assert np.linalg.norm(M - want) / np.linalg.norm(want) < 4 * 3 * 3.7 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("K", [4, 60, 132, 260, 516, 1028, 2052])    # from 1028: 256-wide tiles, ragged
 @pytest.mark.parametrize("power", [bg.BERGSON_FISHER_INV_SQRT, bg.BERGSON_FISHER_INV])
 def test_power_at_tile_edges(K, power):
     g = wl.generator(K, "cpu")
