@@ -731,6 +731,9 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
   score_bound_rule(N, kScoreBN, per_group, static_cast<int>(topk), &bound_j, &bound_r);
   const int64_t factor = bound_j == 0 ? kPrefixMinFactor : kPrefixBoundFactor;
   P.use_prefix = allow_prefix && N >= factor * prefix_rows && Q >= kPrefixMinQueries;
+  // A launch of more than kPlanCTAs CTAs has no room for its published scores, and
+  // leaves list keys there for the launches behind it.
+  bool pub_clear = room;
   for (int pass = 0; pass < n_qg_total; pass += sms) {
     const int n_qg = std::min(sms, n_qg_total - pass);
     // The prefix is cut to whole rounds of store tiles over the CTAs of a
@@ -749,7 +752,8 @@ ScoreLaunchPlan plan_score_launches(int64_t N, int64_t Q, int64_t topk, int ctas
       l.n_tiles = static_cast<int>((l.rows + l.bn - 1) / l.bn);
       l.cpg = std::max(1, std::min(sms / n_qg, l.n_tiles));
       l.grid = n_qg * l.cpg;
-      if (room && l.grid <= kPlanCTAs)         // more CTAs have no room for their words
+      pub_clear = pub_clear && l.grid <= kPlanCTAs;
+      if (pub_clear)
         score_bound_rule(l.rows, l.bn, l.cpg, static_cast<int>(topk), &l.bound_j, &l.bound_r);
       l.q_begin = pass * P.gsize;
       l.q_end = static_cast<int>(std::min<int64_t>(Q, static_cast<int64_t>(pass + n_qg) * P.gsize));

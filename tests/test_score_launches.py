@@ -28,6 +28,7 @@ def _launches(N, Q, topk, ctas):
 
 
 def check(N, Q, topk, ctas):
+    wide = False
     for p, l in _launches(N, Q, topk, ctas):
         assert (l["rows"], l["n_qg"]) == (p["rows"], p["n_qg"])
         # tiles cover the rows in steps one MMA takes (N of 16 at M = 128, of 32 at the pairs'
@@ -44,7 +45,9 @@ def check(N, Q, topk, ctas):
         assert (j > 0) == (r > 0)
         if j:
             assert j <= 32 and j * r >= topk and r <= l["cpg"]
-            assert l["grid"] <= 152                # the published words' room
+            # the published words' room, which a wider launch leaves full of list keys
+            assert l["grid"] <= 152 and not wide
+        wide = wide or l["grid"] > 152
 
 
 @pytest.mark.parametrize("N,Q,topk,ctas", SIZES)
@@ -55,6 +58,14 @@ def test_launches(N, Q, topk, ctas):
 def test_random_launches():
     for size in _random_sizes():
         check(*size)
+
+
+def test_a_wide_launch_leaves_no_bound_to_the_next():
+    # 160 CTAs: 160 query groups, then 18 (8 CTAs each) or 38 (4), whose words would fit
+    for groups in (17, 18, 38):
+        first, last = bg.bergson_debug_score_launches(9_000, K, 256 * (160 + groups), 10, 160)
+        assert first["grid"] == 160 and last["n_qg"] == groups + groups % 2
+        assert last["bound_j"] == 0
 
 
 def test_small_search_is_spread_over_the_sms():
