@@ -940,11 +940,11 @@ __global__ void __launch_bounds__(256, kBatch <= 8 ? 5 : 2) finish_kernel(const 
     if (first) {
       sy.start(ynorm + q, Q, planes);
       const float ny = sy.finish();
-      iy = ny > 0.0f ? 1.0f / sqrtf(ny) : 0.0f;
+      iy = ny > 0.0f ? 1.0f / sqrtf(ny) : -1.0f;       // -1: no norm; 0: an infinite one
       first = false;
     }
     const float nx = sx.finish(), s = sum.finish();
-    *dst = nx > 0.0f && iy > 0.0f ? s * (1.0f / sqrtf(nx)) * iy : 0.0f;
+    *dst = nx > 0.0f && iy >= 0.0f ? s * (1.0f / sqrtf(nx)) * iy : 0.0f;
   }
 }
 

@@ -88,3 +88,19 @@ def test_precondition_rows_random_matrix(B, K):
     assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
     want = x.numpy().astype(np.float64) @ M.numpy().astype(np.float64).T
     np.testing.assert_allclose(np32(out), want, atol=2e-6 * np.abs(want).max(), rtol=0)
+
+
+@pytest.mark.parametrize("B", [5, 40, 70])
+def test_infinite_norms_leave_nan_cosines(B):
+    # inf / ||inf|| is NaN, for a row and for a query, not a score of 0 (K = 32: each norm is one
+    # term a thread, so an infinity stays one)
+    g = wl.generator(B, "cpu")
+    x, y = torch.randn((B, 32), generator=g), torch.randn((300, 32), generator=g)
+    x[2, 17] = float("inf")
+    y[7, 30] = float("-inf")
+    got = _scores(x.to(DEV), y.to(DEV), True)
+    assert np.isnan(got[2]).all() and np.isnan(got[:, 7]).all()
+    x[2], y[7] = 0.0, 0.0
+    want = orc.onthefly_scores(x.numpy(), y.numpy(), True)
+    rest = np.ix_(np.arange(B) != 2, np.arange(300) != 7)
+    np.testing.assert_allclose(got[rest], want[rest], atol=2e-6, rtol=0)
