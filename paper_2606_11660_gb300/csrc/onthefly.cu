@@ -553,8 +553,10 @@ __host__ __device__ constexpr int chain_start(int L, int n_ch, int k) { return k
 // kTwo (batch tiles of up to 32 rows): one issuing thread still stalls about
 // 115 cycles per MMA, so two threads issue.  Warp 1: y_hi [x_hi; x_lo]^T
 // into the set's columns [0, 2 n_pad); warp 10: y_lo x_hi^T into [2 n_pad,
-// 3 n_pad), its B = x_hi split over the pair (each CTA loads its n_pad / 2
-// rows at the same offset).  Each issuer keeps a fixed order into its own
+// 3 n_pad), its B' = x_hi split over the pair (each CTA loads its n_pad / 2
+// rows at the same offset).  An M = 256 MMA takes N in steps of 32, so batch
+// tiles of 16 rows take all of B there too, into [2 n_pad, 4 n_pad), and load
+// no B' (kBoth; y_lo x_lo, in the last 16 columns, is not read).  Each issuer keeps a fixed order into its own
 // columns, so the sums stay deterministic.  Without kTwo, one thread issues
 // y_hi B^T and y_lo B^T into one 2 n_pad-column set (the fourth product
 // y_lo x_lo comes for free).  The epilogue adds the parts.
@@ -574,6 +576,15 @@ __host__ __device__ constexpr int chain_start(int L, int n_ch, int k) { return k
 // releases a set on the even CTA's `tempty`.  A stage's TMEM slot is written
 // again only after its `full` barrier completes anew, i.e. after the `empty`
 // commits of the MMAs that read it.
+// Bytes of a stage on pairs, and accumulator columns of a set.
+constexpr int kBoth = 16;
+__host__ __device__ constexpr int pair_stage_bytes(int n_pad, bool two) {
+  return kYBytes + n_pad * 128 + (two && n_pad != kBoth ? n_pad * 64 : 0);
+}
+__host__ __device__ constexpr int pair_set_cols(int n_pad, bool two) {
+  return (!two ? 2 : n_pad != kBoth ? 3 : 4) * n_pad;
+}
+
 template <bool kUnit, bool kTwo>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     xgemm_pair_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_xh,
@@ -588,7 +599,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   const int xbytes = p.n_pad * 128;
   // this CTA's y half, its half of B = [x_hi; x_lo], and with two issuers its
   // half of B' = x_hi for the y_lo products (N = n_pad: rows r n_pad / 2 ..)
-  const int stage_bytes = kYBytes + xbytes + (kTwo ? xbytes / 2 : 0);
+  const bool own_b = kTwo && p.n_pad != kBoth;     // B' is loaded
+  const int stage_bytes = pair_stage_bytes(p.n_pad, kTwo);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes);
   uint64_t* empty = full + p.stages;
   uint64_t* conv = empty + p.stages;
@@ -627,8 +639,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint64_t tmo = p.timeout_ns;
   // one accumulator set: y_hi [x_hi; x_lo]^T (2 n_pad columns), then with two
-  // issuers y_lo x_hi^T (n_pad columns)
-  const int set_cols = (kTwo ? 3 : 2) * p.n_pad;
+  // issuers y_lo x_hi^T (n_pad columns, and with all of B n_pad more)
+  const int set_cols = pair_set_cols(p.n_pad, kTwo);
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -638,7 +650,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       prefetch_tmap(&tm_y);
       const CUtensorMap* tm_x = rank == 0 ? &tm_xh : &tm_xl;
       prefetch_tmap(tm_x);
-      if constexpr (kTwo) prefetch_tmap(&tm_xh2);
+      if (own_b) prefetch_tmap(&tm_xh2);
       const uint64_t pol_y = policy_evict_first();    // streamed once
       const uint64_t pol_x = policy_evict_last();     // re-read by every tile
       int stage = 0;
@@ -650,7 +662,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       auto load_x = [&](int sg, int st, int nt) {
         tma_load_2d_hint(sbase + sg * stage_bytes + kYBytes, tm_x, smem_u32(&full[sg]), st * kXK,
                          nt * p.n_pad, pol_x);
-        if constexpr (kTwo)
+        if (own_b)
           tma_load_2d_hint(sbase + sg * stage_bytes + kYBytes + xbytes, &tm_xh2,
                            smem_u32(&full[sg]), st * kXK,
                            nt * p.n_pad + static_cast<int>(rank) * (p.n_pad / 2), pol_x);
@@ -694,13 +706,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   } else if (warp == 1 || warp == 10) {
     // ------------------------------------------------------------ MMA issuer(s) (even CTA)
     // kTwo: warp 1 issues the y_hi products into the set's first 2 n_pad
-    // columns and warp 10 the y_lo products into the next 2 n_pad, each in a
+    // columns and warp 10 the y_lo products into the columns after them, each in a
     // fixed order (two issuing threads keep the tensor pipe fed: one stalls
     // about 115 cycles per MMA instruction at these shapes).
     if (rank == 0 && lane == 0 && (warp == 1 || kTwo)) {
       const int who = warp == 10 ? 1 : 0;           // 1: the y_lo issuer
-      // y [x_hi; x_lo]^T, or for the y_lo issuer y_lo x_hi^T; M = 256
-      const uint32_t idesc = make_idesc_tf32(2 * kXM, (who ? 1 : 2) * p.n_pad);
+      // y [x_hi; x_lo]^T, or for the y_lo issuer y_lo x_hi^T (by B'); M = 256
+      const uint32_t idesc = make_idesc_tf32(2 * kXM, (who && own_b ? 1 : 2) * p.n_pad);
       int stage = 0;
       uint32_t ph = 0;
       int ab = 0;
@@ -720,7 +732,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
             tc_fence_after();
             const uint32_t ta = tmem + p.a_base + stage * 2 * kXK;    // y_hi, then y_lo
             const uint64_t dx =
-                sw128_desc(sbase + stage * stage_bytes + kYBytes + who * xbytes);   // B or B'
+                sw128_desc(sbase + stage * stage_bytes + kYBytes + (own_b ? who * xbytes : 0));
 #pragma unroll
             for (int kk = 0; kk < kXK / 8; ++kk) {   // 8 tf32 = 32 bytes: +2 in the address field
               const uint32_t acc = st != c0 || kk != 0;
@@ -994,13 +1006,12 @@ XGemmPlan xgemm_plan(int64_t B, int64_t Q, int64_t K) {
   const int ring_budget = kXSmemBudget - 1024 - kXBarBytes;
   int stage_bytes;
   if (pl.pair) {
-    // two accumulator sets of 2 n_pad columns (4 n_pad with two MMA issuers,
-    // batch tiles up to 32 rows), then the y_hi / y_lo ring (64 columns a
-    // stage)
+    // two accumulator sets (two MMA issuers for batch tiles up to 32 rows),
+    // then the y_hi / y_lo ring (64 columns a stage)
     pl.tmem_cols = 512;
     pl.two_issuers = pl.n_pad <= 32;
-    pl.a_base = pl.n_buf * (pl.two_issuers ? 3 : 2) * pl.n_pad;
-    stage_bytes = kYBytes + pl.n_pad * 128 + (pl.two_issuers ? pl.n_pad * 64 : 0);
+    pl.a_base = pl.n_buf * pair_set_cols(pl.n_pad, pl.two_issuers);
+    stage_bytes = pair_stage_bytes(pl.n_pad, pl.two_issuers);
     pl.stages = std::min({kXMaxStages, (512 - pl.a_base) / (2 * kXK), ring_budget / stage_bytes});
     pl.a_slots = pl.stages;
   } else {
@@ -1094,7 +1105,7 @@ cudaError_t xgemm_run(const XGemmArgs& a, int sms, cudaStream_t s) {
   p.status = a.status;
   p.timeout_ns = a.timeout_ns;
   const size_t stage_bytes =
-      pl.pair ? kYBytes + pl.n_pad * 128 + (pl.two_issuers ? pl.n_pad * 64 : 0)
+      pl.pair ? pair_stage_bytes(pl.n_pad, pl.two_issuers)
               : 2 * kYBytes + 2 * pl.n_pad * 128;
   const size_t smem = 1024 + pl.stages * stage_bytes + kXBarBytes;
   static PerDeviceOnce attr_pair[4], attr_m;

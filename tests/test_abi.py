@@ -447,12 +447,13 @@ def check_xgemm_plan(B, Q, K):
         assert 1 <= S <= min(steps, 64)
         bounds = [z * steps // S for z in range(S + 1)]
         assert bounds[0] == 0 and bounds[-1] == steps and all(a < b for a, b in zip(bounds, bounds[1:]))
-    # TMEM: two accumulator sets of 2 n_pad columns (4 n_pad on pairs with two
-    # MMA issuers, batch tiles up to 32 rows), and on pairs the y_hi / y_lo
-    # ring after them (64 columns a stage), within 512 columns
+    # TMEM: two accumulator sets of 2 n_pad columns (3 n_pad on pairs with two
+    # MMA issuers, batch tiles up to 32 rows; 4 n_pad for tiles of 16, whose y_lo
+    # MMAs take N = 32, the least at M = 256), and on pairs the y_hi / y_lo ring
+    # after them (64 columns a stage), within 512 columns
     assert p["n_buf"] == 2
     assert p["tmem_cols"] <= 512 and p["tmem_cols"] & (p["tmem_cols"] - 1) == 0
-    acc = 2 * (3 if pair and p["n_pad"] <= 32 else 2) * p["n_pad"]
+    acc = 2 * (4 if pair and p["n_pad"] == 16 else 3 if pair and p["n_pad"] <= 32 else 2) * p["n_pad"]
     if pair:
         # a TMEM slot (y_hi, y_lo: 64 columns) per stage
         assert p["a_base"] == acc and p["tmem_cols"] == 512
