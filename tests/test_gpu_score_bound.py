@@ -1,10 +1,11 @@
 """The scorer's in-flight bound, candidate lists and evened-out tiles.
 
 Each CTA publishes its j-th best first-tile score and lists only what reaches
-the r-th largest of them: sizes where j is 1, 2 .. 8 (kept up to date), 9 .. 32
-(first tile only) and where no bound is taken; stores sorted by score, which
-fill every list and turn it into a heap; exact ties; tiles of 64 .. 256 rows;
-scans long enough for the bound to be taken again (tiles 8 and 64).
+the r-th largest of them: sizes where j is 1, 2 .. 8, 9 .. 32 and where no bound
+is taken; stores sorted by score, which fill every list and turn it into a heap;
+exact ties; tiles of 64 .. 256 rows; scans long enough for the bound to be taken
+again from the lists (before tiles 2, 6, 20 of a CTA's more than 8, 24, 80), for
+each range of j on each kernel.
 """
 import pytest
 import torch
@@ -85,9 +86,18 @@ def test_equal_rows_come_in_index_order(Q, topk):
     assert (s == s[:, :1]).all()
 
 
-@pytest.mark.parametrize("Q,topk,tiles", [(2, 100, 10), (1, 30, 66), (260, 100, 10)])
-def test_bound_taken_again(Q, topk, tiles):
-    N = 256 * tiles * (152 if Q < 129 else 38)
+@pytest.mark.parametrize("Q,topk,tiles,j", [
+    (2, 100, 10, (1, 1)), (1, 30, 82, (1, 1)), (2, 300, 26, (2, 8)), (3, 1024, 10, (9, 32)),
+    (140, 60, 26, (1, 1)), (200, 200, 10, (2, 8)), (200, 800, 26, (9, 32)),     # pairs, one tile
+    (300, 40, 26, (1, 1)), (300, 100, 26, (2, 8)), (1024, 1000, 10, (9, 32)),   # pairs, two tiles
+])
+def test_bound_taken_again(Q, topk, tiles, j):
+    groups = 1 if Q < 129 else 2 * -(-Q // (256 if Q <= 256 else 512))
+    N = 256 * tiles * (152 // groups)
+    launch = bg.bergson_debug_score_launches(N, 64, Q, topk, 152)
+    assert len(launch) == 1 and launch[0]["n_qg"] == groups
+    assert j[0] <= launch[0]["bound_j"] <= j[1]
+    assert -(-launch[0]["n_tiles"] // launch[0]["cpg"]) == tiles > 8
     store, queries = _rows(N, 64, tiles), _queries(Q, 3)
     store[N // 2] = float("nan")                      # a row that is never found
     s, i = _search(store, queries, topk)
