@@ -124,7 +124,10 @@ typedef struct bergson_layer {
   int64_t bias_col_offset;        /* used with BERGSON_LAYER_BIAS */
 } bergson_layer;
 
-/* Bytes of workspace bergson_project_grads needs for these arguments. */
+/*
+ * Bytes of workspace for bergson_project_grads with these arguments.  The call
+ * takes somewhat less too (it then cuts the work more coarsely).
+ */
 BERGSON_API int bergson_project_grads_workspace(const bergson_layer* layers, int n_layers,
                                     int64_t B, int64_t T, size_t* ws_bytes);
 
@@ -613,8 +616,8 @@ BERGSON_API int bergson_store_load(const char* path, int64_t file_row_offset, in
  * Same arguments and result as bergson_project_grads, minus the workspace.
  * The scratch is a fixed static device array of BERGSON_NOALLOC_SCRATCH_BYTES
  * that every GPU loading the library keeps until the process exits; requests
- * needing more (see bergson_project_grads_workspace) fail with
- * BERGSON_EWORKSPACE and enqueue nothing.  The call itself allocates nothing
+ * that cannot do with it (bergson_project_grads_workspace may report more than
+ * the least they take) fail with BERGSON_EWORKSPACE and enqueue nothing.  The call itself allocates nothing
  * (no cudaMalloc, no workspace, no allocating library routine).
  * All calls share the one array: calls that overlap on the GPU (e.g. on two
  * streams) race and must be ordered by the caller.

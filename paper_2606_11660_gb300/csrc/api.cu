@@ -253,6 +253,13 @@ int validate_blocks(const bergson_layer* layers, int n_layers, int64_t ld_out,
 
 int chunks_of(int64_t d) { return static_cast<int>((d + kChunk - 1) / kChunk); }
 
+// How a launch is cut: finely (small launches into slots of one tile and smaller
+// pieces), coarsely (where the workspace has no room for that), or as the
+// workspace query reserves it.  A program sizes its workspace for its largest
+// batch; smaller ones are cut into more pieces and may need more, so the query
+// counts pieces from kSplitShare on whatever the share.
+enum class Cut { kFine, kCoarse, kReserve };
+
 // Builds a group's work table when its slots need more than "item i is slot i":
 // (1) cutting: when the launch is too coarse for the SMs to finish together
 // (largest slot above kSplitShare of one CTA's share), large slots are cut
@@ -261,7 +268,8 @@ int chunks_of(int64_t d) { return static_cast<int>((d + kChunk - 1) / kChunk); }
 // to each other (A-side pieces too), so the scheduler starts them together.
 // Cost unit: one 64-column chunk of one tile; the table runs largest first.
 void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, int64_t n_queries,
-               bool token_split, bool fine) {
+               bool token_split, Cut cut) {
+  const bool fine = cut == Cut::kFine, reserve = cut == Cut::kReserve;
   if (g.n_slots == 0) return;
   int64_t total = 0, max_slot = 0;
   for (int li : g.layers) {
@@ -272,15 +280,16 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, in
   const double share = static_cast<double>(total) / kPlanCTAs;
   const double excess = static_cast<double>(max_slot) - share;
   const bool split = n_queries == 0 ? static_cast<double>(max_slot) >
-                                          (share < kSmallShare ? kSplitSmallShare : kSplitShare) * share
+                                          (share < kSmallShare && !reserve ? kSplitSmallShare
+                                                                           : kSplitShare) * share
                                     : token_split && excess > kTokenSplitUnits +
                                                                   kTokenSplitPerQuery * n_queries;
   bool shared = false;
   for (const auto& u : g.units) shared = shared || u.second > 1;
   if (!split && !shared) return;
   // Tiles of a slot (the last slot of an example may have fewer).
-  const int slot_tiles = std::min(g.tpc, n_tiles);
-  double target = std::max(share / kPiecesPerShare, kMinPieceUnits);
+  const int slot_tiles = reserve ? g.tpc : std::min(g.tpc, n_tiles);
+  double target = std::max(share / kPiecesPerShare, reserve ? 0.0 : kMinPieceUnits);
   // A piece stores and its slot's finisher reloads 4k fp32 bytes per token,
   // against 128 bytes per token and chunk streamed: pieces of at least 2k
   // chunks keep that under 1/32 of the piece's traffic.  (Fewer, larger
@@ -429,10 +438,10 @@ void plan_work(const bergson_layer* layers, int64_t B, int n_tiles, Group& g, in
 }
 
 // n_queries > 0 lays out per-token score partials [n_layers, n_queries, B, T]
-// instead of per-item projection partials.  `fine` lets small launches be cut
-// more finely, which takes more workspace.
-ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
-                           int64_t n_queries, bool fine) {
+// instead of per-item projection partials.
+ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                        int64_t n_queries = 0, Cut cut = Cut::kFine) {
+  const bool fine = cut == Cut::kFine;
   ProjLayout L;
   L.n_tiles = static_cast<int>((T + kTileTokens - 1) / kTileTokens);
   L.mod_slot.assign(n_layers, 0);
@@ -532,7 +541,7 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
     g.n_chunks = (L.n_tiles + tpc - 1) / tpc;
     g.n_slots = static_cast<int>(mb * g.n_chunks);
     g.n_items = g.n_slots;
-    plan_work(layers, B, L.n_tiles, g, n_queries, token_tc, fine);
+    plan_work(layers, B, L.n_tiles, g, n_queries, token_tc, cut);
   }
   size_t off = 0;
   L.mods_off = off;
@@ -585,12 +594,19 @@ ProjLayout plan_project_at(const bergson_layer* layers, int n_layers, int64_t B,
 // A finely cut launch may need more workspace than a coarse one; one that would
 // then pass the allocation-free call's static scratch stays coarse, so that
 // the call takes what it always took.
-ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
-                        int64_t n_queries = 0) {
-  ProjLayout L = plan_project_at(layers, n_layers, B, T, n_queries, true);
+ProjLayout plan_within_scratch(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                               int64_t n_queries = 0) {
+  ProjLayout L = plan_project(layers, n_layers, B, T, n_queries);
   if (n_queries == 0 && L.total > BERGSON_NOALLOC_SCRATCH_BYTES)
-    L = plan_project_at(layers, n_layers, B, T, n_queries, false);
+    L = plan_project(layers, n_layers, B, T, n_queries, Cut::kCoarse);
   return L;
+}
+
+// What the workspace query reports.
+size_t project_workspace(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                         int64_t n_queries) {
+  return std::max(plan_within_scratch(layers, n_layers, B, T, n_queries).total,
+                  plan_project(layers, n_layers, B, T, n_queries, Cut::kReserve).total);
 }
 
 CUresult encode_act(CUtensorMap* tm, const void* ptr, int64_t d, int64_t T, int64_t B) {
@@ -794,6 +810,15 @@ int validate_score(const void* store, int64_t N, int64_t K, int64_t ld_store, co
 
 }  // namespace
 
+int project_least_workspace(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                            size_t* ws_bytes) {
+  const int st = validate_layers(layers, n_layers, B, T);
+  if (st != BERGSON_OK) return st;
+  *ws_bytes = std::min(plan_within_scratch(layers, n_layers, B, T).total,
+                       plan_project(layers, n_layers, B, T, 0, Cut::kCoarse).total);
+  return BERGSON_OK;
+}
+
 int record_error(int code, const char* fmt, ...) {
   char buf[512];
   va_list ap;
@@ -851,7 +876,7 @@ int bergson_debug_project_plan(const bergson_layer* layers, int n_layers, int64_
                                int64_t* n_shared) {
   const int st = validate_layers(layers, n_layers, B, T);
   if (st != BERGSON_OK) return st;
-  const ProjLayout L = plan_project(layers, n_layers, B, T);
+  const ProjLayout L = plan_within_scratch(layers, n_layers, B, T);
   int64_t slots = 0, items = 0, pieces = 0;
   for (const Group& g : L.groups) {
     slots += g.n_slots;
@@ -968,7 +993,7 @@ int bergson_project_grads_workspace(const bergson_layer* layers, int n_layers, i
   if (ws_bytes == nullptr) return fail(BERGSON_EINVAL, "ws_bytes is NULL");
   int st = validate_layers(layers, n_layers, B, T);
   if (st != BERGSON_OK) return st;
-  *ws_bytes = plan_project(layers, n_layers, B, T).total;
+  *ws_bytes = project_workspace(layers, n_layers, B, T, 0);
   return BERGSON_OK;
 }
 
@@ -998,10 +1023,10 @@ static int run_projection(const bergson_layer* layers, int n_layers, int64_t B, 
     if (B > 0 && out == nullptr) return fail(BERGSON_EINVAL, "out is NULL");
   }
   if (out != nullptr && !aligned(out, 4)) return fail(BERGSON_EALIGN, "out must be 4-byte aligned");
-  ProjLayout L = plan_project(layers, n_layers, B, T, token ? n_queries : 0);
+  ProjLayout L = plan_within_scratch(layers, n_layers, B, T, token ? n_queries : 0);
   // a workspace that only a coarse cut fits takes that
   if (ws_bytes < L.total)
-    L = plan_project_at(layers, n_layers, B, T, token ? n_queries : 0, false);
+    L = plan_project(layers, n_layers, B, T, token ? n_queries : 0, Cut::kCoarse);
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
   if (ws_bytes < L.total)
@@ -1149,7 +1174,7 @@ int bergson_token_scores_workspace(const bergson_layer* layers, int n_layers, in
     return fail(BERGSON_EUNSUPPORTED, "n_queries must be in [1, %d]", kMaxTokenQueries);
   int st = validate_layers(layers, n_layers, B, T);
   if (st != BERGSON_OK) return st;
-  *ws_bytes = plan_project(layers, n_layers, B, T, n_queries).total;
+  *ws_bytes = project_workspace(layers, n_layers, B, T, n_queries);
   return BERGSON_OK;
 }
 

@@ -11,6 +11,8 @@
 #include <atomic>
 #include <mutex>
 
+struct bergson_layer;           // bergson.h
+
 namespace bergson {
 
 // A per-device "done once" record for settings that CUDA keeps per function
@@ -185,6 +187,11 @@ struct ScoreParams {
 
 // Sets this thread's bergson_last_error() message (printf format) and returns `code`.
 int record_error(int code, const char* fmt, ...);
+
+// The least workspace bergson_project_grads takes for these arguments (its query
+// reports more).  Returns the validation status.
+int project_least_workspace(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
+                            size_t* ws_bytes);
 
 // ---- launchers (return the launch error, if any) ----
 

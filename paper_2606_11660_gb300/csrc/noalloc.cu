@@ -70,7 +70,7 @@ extern "C" BERGSON_API int bergson_project_grads_noalloc(const bergson_layer* la
                                                          const uint8_t* mask, float* out,
                                                          int64_t ld_out, void* stream) {
   size_t need = 0;
-  const int st = bergson_project_grads_workspace(layers, n_layers, B, T, &need);
+  const int st = bergson::project_least_workspace(layers, n_layers, B, T, &need);
   if (st != BERGSON_OK) return st;
   if (need > kScratchBytes)
     return bergson::record_error(
