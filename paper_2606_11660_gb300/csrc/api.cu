@@ -591,21 +591,10 @@ ProjLayout plan_project(const bergson_layer* layers, int n_layers, int64_t B, in
   return L;
 }
 
-// A finely cut launch may need more workspace than a coarse one; one that would
-// then pass the allocation-free call's static scratch stays coarse, so that
-// the call takes what it always took.
-ProjLayout plan_within_scratch(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
-                               int64_t n_queries = 0) {
-  ProjLayout L = plan_project(layers, n_layers, B, T, n_queries);
-  if (n_queries == 0 && L.total > BERGSON_NOALLOC_SCRATCH_BYTES)
-    L = plan_project(layers, n_layers, B, T, n_queries, Cut::kCoarse);
-  return L;
-}
-
 // What the workspace query reports.
 size_t project_workspace(const bergson_layer* layers, int n_layers, int64_t B, int64_t T,
                          int64_t n_queries) {
-  return std::max(plan_within_scratch(layers, n_layers, B, T, n_queries).total,
+  return std::max(plan_project(layers, n_layers, B, T, n_queries).total,
                   plan_project(layers, n_layers, B, T, n_queries, Cut::kReserve).total);
 }
 
@@ -814,7 +803,7 @@ int project_least_workspace(const bergson_layer* layers, int n_layers, int64_t B
                             size_t* ws_bytes) {
   const int st = validate_layers(layers, n_layers, B, T);
   if (st != BERGSON_OK) return st;
-  *ws_bytes = std::min(plan_within_scratch(layers, n_layers, B, T).total,
+  *ws_bytes = std::min(plan_project(layers, n_layers, B, T).total,
                        plan_project(layers, n_layers, B, T, 0, Cut::kCoarse).total);
   return BERGSON_OK;
 }
@@ -876,7 +865,7 @@ int bergson_debug_project_plan(const bergson_layer* layers, int n_layers, int64_
                                int64_t* n_shared) {
   const int st = validate_layers(layers, n_layers, B, T);
   if (st != BERGSON_OK) return st;
-  const ProjLayout L = plan_within_scratch(layers, n_layers, B, T);
+  const ProjLayout L = plan_project(layers, n_layers, B, T);
   int64_t slots = 0, items = 0, pieces = 0;
   for (const Group& g : L.groups) {
     slots += g.n_slots;
@@ -1023,7 +1012,7 @@ static int run_projection(const bergson_layer* layers, int n_layers, int64_t B, 
     if (B > 0 && out == nullptr) return fail(BERGSON_EINVAL, "out is NULL");
   }
   if (out != nullptr && !aligned(out, 4)) return fail(BERGSON_EALIGN, "out must be 4-byte aligned");
-  ProjLayout L = plan_within_scratch(layers, n_layers, B, T, token ? n_queries : 0);
+  ProjLayout L = plan_project(layers, n_layers, B, T, token ? n_queries : 0);
   // a workspace that only a coarse cut fits takes that
   if (ws_bytes < L.total)
     L = plan_project(layers, n_layers, B, T, token ? n_queries : 0, Cut::kCoarse);

@@ -15,8 +15,8 @@
 // Properties a caller must know:
 //   * The scratch is a file-scope __device__ array of BERGSON_NOALLOC_SCRATCH_BYTES
 //     (32 MiB).  Every GPU that loads this part of the library keeps it until
-//     the process exits.  Requests whose workspace would exceed it are
-//     rejected with BERGSON_EWORKSPACE before anything is enqueued.
+//     the process exits.  Requests that cannot do with it, however coarsely
+//     cut, are rejected with BERGSON_EWORKSPACE before anything is enqueued.
 //   * All calls share that one array.  It keeps whatever the last call left
 //     there; every call rewrites everything it reads (descriptors, counters,
 //     projection slices, partial sums) before reading it.  Calls whose work

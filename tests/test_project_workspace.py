@@ -69,3 +69,27 @@ def test_queried_size_is_taken_and_projections_alone_are_not():
         assert _status(arr, len(arr), B, T, size, k) == bg.BERGSON_EDEVICE_TIMEOUT
         p = sum(4 * (k[0] * l.d_in + k[1] * l.d_out) for l in arr)     # P'
         assert _status(arr, len(arr), B, T, p, k) == bg.BERGSON_EWORKSPACE
+
+
+@pytest.mark.parametrize("family,blocks,k,B,T", [("llama8b", 7, (16, 16), 1, 129),
+                                                 ("llama8b", 7, (16, 16), 4, 129),
+                                                 ("pythia1b4", 12, (32, 32), 2, 512)])
+def test_large_projections_leave_the_slots_of_a_small_launch(family, blocks, k, B, T):
+    # more than the allocation-free call's 32 MB, for P' mostly: slots of one tile all the same
+    arr = _layers(DIMS[family] * blocks, k)
+    assert _query(arr, len(arr), B, T) > 32 << 20
+    n = [ctypes.c_int64() for _ in range(4)]
+    assert bg.lib().bergson_debug_project_plan(arr, len(arr), B, T, *map(ctypes.byref, n)) == 0
+    assert n[0].value == len(arr) * B * -(-T // 128)
+
+
+@pytest.mark.parametrize("family,blocks,k,B,T", [("llama8b", 5, (16, 16), 2, 512),
+                                                 ("llama8b", 2, (32, 32), 8, 300),
+                                                 ("pythia1b4", 6, (64, 16), 1, 129)])
+def test_allocation_free_call_takes_what_its_scratch_can_do(family, blocks, k, B, T):
+    arr = _layers(DIMS[family] * blocks, k)
+    assert _query(arr, len(arr), B, T) > 32 << 20     # with the finest cut
+    st = bg.lib().bergson_project_grads_noalloc(arr, len(arr), B, T, None, FAKE,
+                                                len(arr) * k[0] * k[1], None)
+    assert st == bg.BERGSON_EINVAL                    # FAKE is no device memory; not EWORKSPACE
+    assert "not device memory" in bg.bergson_last_error()
