@@ -524,11 +524,13 @@ def bench_fisher(args, world, dev, state, peaks):
     true_res = float(torch.linalg.norm(MRM.double())) / K ** 0.5
     del MRM
     torch.cuda.empty_cache()
-    gemm_flops = 2.0 * K ** 3 * (3 * iters_done + len(ns_res) - iters_done)
+    # T, Z T and Y T of each update, and the T whose residual ends the iteration; the first
+    # T and Z are not products
+    n_products = max(0, 3 * iters_done - 1)
+    gemm_flops = 2.0 * K ** 3 * n_products
     apply_gbs = 4.0 * K * (K + 2 * cfg.B) / (apply_ms * 1e-3) / 1e9   # M once, rows in and out
-    # fp32-accurate products run three tf32 MMAs each; the tf32 rate is the
-    # measured bf16 peak times the nominal tf32 : bf16 ratio (1.1 : 2.25).
-    tf32_eff = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) * (1.1 / 2.25) / 3.0
+    # fp32-accurate products are six bf16 ones of the operands' parts
+    fp32_eff = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) / 6.0
     ns_tflops = gemm_flops / (pow_ms * 1e-3) / 1e12
     return {"value": round(cfg.B * world / (step_ms * 1e-3), 2), "unit": "examples/s",
             "ms_per_step": round(step_ms, 4), "apply_ms": round(apply_ms, 4),
@@ -547,12 +549,12 @@ def bench_fisher(args, world, dev, state, peaks):
                                "peak": peaks["hbm_gbs"], "unit": "GB/s",
                                "frac": round(apply_gbs / peaks["hbm_gbs"], 4)},
             "roofline_newton_schulz": {"bound": "tensor", "achieved": round(ns_tflops, 1),
-                                       "peak": round(tf32_eff, 1), "unit": "TFLOP/s",
-                                       "frac": round(ns_tflops / tf32_eff, 4),
-                                       "peak_source": "measured sustained bf16 x 1.1/2.25 "
-                                                      "(nominal tf32:bf16) / 3 tf32 products"},
+                                       "peak": round(fp32_eff, 1), "unit": "TFLOP/s",
+                                       "frac": round(ns_tflops / fp32_eff, 4),
+                                       "peak_source": "measured sustained bf16 / 6 products of "
+                                                      "bf16 parts"},
             "what": "step = project_grads + precondition_rows (R^-1/2, K=12288) + build_store; "
-                    "fit and R^-1/2 are one-time costs (3xTF32 tcgen05 GEMMs)"}
+                    "fit and R^-1/2 are one-time costs (tcgen05 products of three bf16 parts)"}
 
 
 def bench_streamed(args, world, dev, name, peaks):
