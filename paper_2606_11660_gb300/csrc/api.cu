@@ -37,7 +37,8 @@ constexpr double kSmallShare = 200.0;
 constexpr double kSplitSmallShare = 1.5;
 constexpr double kMinPieceUnits = 4.0;               // ... of at least 4 chunks of a tile
 constexpr double kFinePieceShare = 0.8;              // largest piece, in shares, before the minimum
-                                                     // piece size is lowered
+                                                     // piece size is lowered,
+constexpr int kFineMaxK = 96;                        // and k_in + k_out up to which it is
 // Token scores: pieces cost their slot's last one some 17 us (sums, query
 // blocks behind them) and 0.16 us a query, and save 0.35 us per unit by which
 // the largest slot exceeds a share.  With and without, us a call: a
@@ -48,7 +49,6 @@ constexpr double kFinePieceShare = 0.8;              // largest piece, in shares
 constexpr double kTokenSplitUnits = 64.0;
 constexpr double kTokenSplitPerQuery = 0.75;
 constexpr int kTokenSlotsPerCTA = 16;
-constexpr int kFineMaxK = 96;                        // k_in + k_out up to which it is
 // Few slots (below two a CTA) of shares below this: slots of one tile.
 constexpr double kFineSlotUnits = 400.0;
 constexpr int kMaxScoreCTAs = 160;                   // upper bound on persistent score CTAs
