@@ -397,7 +397,8 @@ BERGSON_API int bergson_aggregate_rows(const float* rows, int64_t n, int64_t K, 
  * (or bergson_score_grads) as usual.  All matrices are fp32 row-major with
  * 16-byte aligned rows (leading dimensions multiples of 4); K % 4 == 0,
  * K <= 65536.  Workspaces: bergson_fisher_fit_workspace(n, K),
- * bergson_fisher_preconditioner_workspace(K) (about 7 K^2 floats) and, for
+ * bergson_fisher_preconditioner_workspace(K) (about 8 K^2 floats up to
+ * K = 12288 and 5.5 K^2 above; the calls take down to 2/3 of the fit's and 5.5 K^2) and, for
  * precondition_rows, bergson_score_grads_workspace(B, K, K).
  * Errors: EINVAL, EALIGN, EWORKSPACE, ECUDA.
  */

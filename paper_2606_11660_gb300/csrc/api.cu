@@ -1678,7 +1678,7 @@ int bergson_fisher_fit(const float* rows, int64_t n, int64_t K, int64_t ld, floa
   if (ld < K) return fail(BERGSON_EINVAL, "ld must be >= K");
   int st = check_square(R, K, ldr, "R");
   if (st != BERGSON_OK) return st;
-  const size_t need = round_up(fisher_fit_workspace(n, K), 256);
+  const size_t need = fisher_fit_least(n, K);
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
   if (ws_bytes < need)
@@ -1689,7 +1689,7 @@ int bergson_fisher_fit(const float* rows, int64_t n, int64_t K, int64_t ld, floa
   int* status = status_word(dg.dev);
   if (status == nullptr) return fail(BERGSON_ECUDA, "device status word unavailable");
   cudaError_t e = launch_fisher_fit(rows, static_cast<int>(n), static_cast<int>(K), ld, R, ldr,
-                                    static_cast<float*>(workspace), status, sm_count(dg.dev),
+                                    workspace, ws_bytes, status, sm_count(dg.dev),
                                     static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return fail_cuda(e, "Fisher fit launch");
   return BERGSON_OK;
@@ -1720,7 +1720,7 @@ static int run_fisher_preconditioner(const float* R1, const float* R2, int64_t K
     return fail(BERGSON_EINVAL, "unknown power %d", power);
   if (iterations < 1 || iterations > 100) return fail(BERGSON_EINVAL, "iterations in [1, 100]");
   if (!(tol >= 0.0f)) return fail(BERGSON_EINVAL, "tol must be >= 0");
-  const size_t need = round_up(fisher_power_workspace(K), 256);
+  const size_t need = fisher_power_least(K);
   if (workspace == nullptr) return fail(BERGSON_EINVAL, "workspace is NULL");
   if (!aligned(workspace, 256)) return fail(BERGSON_EALIGN, "workspace must be 256-byte aligned");
   if (ws_bytes < need)
@@ -1733,7 +1733,7 @@ static int run_fisher_preconditioner(const float* R1, const float* R2, int64_t K
   cudaError_t e = launch_fisher_power(R1, R2, static_cast<int>(K), ldr, lam, damping,
                                       power == BERGSON_FISHER_INV ? 1 : 0, iterations, tol,
                                       residuals, iterations_done, M, ldm,
-                                      static_cast<float*>(workspace), status, sm_count(dg.dev),
+                                      workspace, ws_bytes, status, sm_count(dg.dev),
                                       static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return fail_cuda(e, "Fisher preconditioner launch");
   return BERGSON_OK;

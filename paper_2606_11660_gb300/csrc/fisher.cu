@@ -223,12 +223,11 @@ SplitOperand take_split(uint8_t* ws, size_t* off, int rows, int K) {
   return o;
 }
 
-// The Z and Y products of an update go in one launch, which takes a matrix more
-// of workspace, while one of them leaves half the SMs idle (25 of 256 x 256 tiles
-// for 76 clusters at K = 1280).  From there on they follow each other, and the Y
-// product's result takes the room of T, which only the Z product reads.
-constexpr int kTogetherK = 1280;
-bool zy_together(int64_t K) { return K <= kTogetherK; }
+// Above this K the workspace query reports the lean layout (see
+// launch_fisher_power).  An update with the full one / the lean one: K = 256 35 / 48
+// us, 1024 67 / 96, 2304 389 / 466, 4096 1.50 / 1.62 ms, 8192 11.2 / 11.4, 12,288 38.0 /
+// 38.4.
+constexpr int kFullK = 12288;
 
 // Iterates enqueued between two read-backs of their residuals.  Everything after
 // the first one within the tolerance finds the stop flag set and does nothing,
@@ -246,54 +245,77 @@ size_t part_floats(int64_t K) {
 
 }  // namespace
 
-size_t fisher_fit_workspace(int64_t n, int64_t K) {
-  return split_bytes(K, n);
+size_t fisher_fit_workspace(int64_t n, int64_t K) { return split_bytes(K, n); }
+
+// Two thirds of it (8 rows' planes at least).
+size_t fisher_fit_least(int64_t n, int64_t K) {
+  return std::max(split_bytes(K, std::min<int64_t>(n, 8)), split_bytes(K, n) * 2 / 3);
 }
 
 cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* r, int64_t ldr,
-                              float* ws, int* status, int sms, cudaStream_t s) {
-  uint8_t* base = reinterpret_cast<uint8_t*>(ws);
-  size_t off = 0;
-  const SplitOperand xt = take_split(base, &off, K, n);
-  const cudaError_t e = launch_transpose_split(x, n, K, ldx, xt, s);
-  if (e != cudaSuccess) return e;
-  SquareArgs a;
-  a.x = xt;
-  a.y = xt;
-  a.symmetric = true;
-  a.alpha = 1.0f / static_cast<float>(n);
-  a.c = r;
-  a.ldc = ldr;
-  a.status = status;
-  return launch_square(&a, 1, sms, s);
+                              void* ws, size_t ws_bytes, int* status, int sms, cudaStream_t s) {
+  // as many rows at a time as the workspace holds: all of them in the queried size
+  int part = n;
+  if (split_bytes(K, n) > ws_bytes)
+    part = static_cast<int>(ws_bytes / split_bytes(K, 8)) * 8;
+  for (int i0 = 0; i0 < n; i0 += part) {
+    const int rows = std::min(part, n - i0);
+    size_t off = 0;
+    const SplitOperand xt = take_split(static_cast<uint8_t*>(ws), &off, K, rows);
+    cudaError_t e = launch_transpose_split(x + i0 * ldx, rows, K, ldx, xt, s);
+    if (e != cudaSuccess) return e;
+    SquareArgs a;
+    a.x = xt;
+    a.y = xt;
+    a.symmetric = true;
+    a.accumulate = i0 > 0;
+    a.alpha = 1.0f / static_cast<float>(n);
+    a.c = r;
+    a.ldc = ldr;
+    a.status = status;
+    if ((e = launch_square(&a, 1, sms, s)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-size_t fisher_power_workspace(int64_t K) {
-  const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
-  return (zy_together(K) ? 2 : 1) * kk + 4 * split_bytes(K, K) +
+namespace {
+
+size_t power_bytes(int64_t K, int splits, int matrices) {
+  return splits * split_bytes(K, K) +
+         matrices * round_up256(static_cast<size_t>(K) * K * sizeof(float)) +
          round_up256(part_floats(K) * sizeof(float)) + kScalBytes;
 }
+size_t full_bytes(int64_t K) { return power_bytes(K, 4, 2); }
 
+}  // namespace
+
+size_t fisher_power_least(int64_t K) { return power_bytes(K, 3, 1); }
+
+size_t fisher_power_workspace(int64_t K) {
+  return K <= kFullK ? full_bytes(K) : fisher_power_least(K);
+}
+
+// Full layout (32 K^2 bytes): the splits of Z, Y, T and T^T and the fp32 Z and Y
+// products, which go in one launch, as do the passes over them.
+// Lean (22 K^2): T^T is transposed from T's split into Z's room once the Z product
+// has read that, and the Y product takes T's room.  Same results, a launch and a
+// transposition more an update, and two products' last rounds instead of one.
 cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t ldr, float lam,
                                 float damping, int inverse, int iterations, float tol,
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
-                                float* ws, int* status, int sms, cudaStream_t s) {
-  // The splits of Z, Y, T and T^T and the fp32 Z and Y products.
-  uint8_t* base = reinterpret_cast<uint8_t*>(ws);
+                                void* ws, size_t ws_bytes, int* status, int sms, cudaStream_t s) {
+  const bool full = ws_bytes >= full_bytes(K);
+  uint8_t* base = static_cast<uint8_t*>(ws);
   const size_t kk = round_up256(static_cast<size_t>(K) * K * sizeof(float));
   size_t off = 0;
   const SplitOperand zs = take_split(base, &off, K, K);
   const SplitOperand ys = take_split(base, &off, K, K);
   const SplitOperand ts = take_split(base, &off, K, K);
-  const SplitOperand tts = take_split(base, &off, K, K);
+  const SplitOperand tts = full ? take_split(base, &off, K, K) : zs;
   float* zf = reinterpret_cast<float*>(base + off);
   off += kk;
-  const bool together = zy_together(K);
-  float* yf = reinterpret_cast<float*>(ts.planes);
-  if (together) {
-    yf = reinterpret_cast<float*>(base + off);
-    off += kk;
-  }
+  float* yf = reinterpret_cast<float*>(full ? base + off : reinterpret_cast<uint8_t*>(ts.planes));
+  if (full) off += kk;
   float* part = reinterpret_cast<float*>(base + off);
   off += round_up256(part_floats(K) * sizeof(float));
   float* scal = reinterpret_cast<float*>(base + off);  // trace, c, 1/c, 1/sqrt(c), 1/c, -, stop
@@ -348,7 +370,7 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
       t.alpha = -0.5f;
       t.gamma = 1.5f;
       t.row_out = ts;
-      t.col_out = tts;
+      if (full) t.col_out = tts;
       t.part = track ? part : nullptr;
       t.stop = stop;
       t.status = status;
@@ -389,17 +411,34 @@ cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t
       a[0].row = tts;
       a[1].c = yf;
       a[1].row = ys;
-      const SquareArgs y1 = product(ys, tts, yf);
-      const SquarePassArgs yp = sym_pass(yf, ys);
-      if ((e = launch_square_pass(a, 2, K, stop, s)) != cudaSuccess ||
-          (e = launch_square(&y1, 1, sms, s)) != cudaSuccess ||
-          (e = launch_square_pass(&yp, 1, K, stop, s)) != cudaSuccess)
-        return e;
+      if (full) {
+        const SquareArgs y1 = product(ys, tts, yf);
+        const SquarePassArgs yp = sym_pass(yf, ys);
+        if ((e = launch_square_pass(a, 2, K, stop, s)) != cudaSuccess ||
+            (e = launch_square(&y1, 1, sms, s)) != cudaSuccess ||
+            (e = launch_square_pass(&yp, 1, K, stop, s)) != cudaSuccess)
+          return e;
+      } else {
+        // Y0 leaves T's room for T0^T, and Y1 goes to Z's until that is split
+        float* y1f = reinterpret_cast<float*>(zs.planes);
+        SquarePassArgs t0;
+        t0.c = zf;
+        t0.row = ts;
+        const SquareArgs y1 = product(ys, ts, y1f);
+        const SquarePassArgs yp = sym_pass(y1f, ys), zp = sym_pass(zf, zs);
+        if ((e = launch_square_pass(a + 1, 1, K, stop, s)) != cudaSuccess ||
+            (e = launch_square_pass(&t0, 1, K, stop, s)) != cudaSuccess ||
+            (e = launch_square(&y1, 1, sms, s)) != cudaSuccess ||
+            (e = launch_square_pass(&yp, 1, K, stop, s)) != cudaSuccess ||
+            (e = launch_square_pass(&zp, 1, K, stop, s)) != cudaSuccess)
+          return e;
+      }
     } else {
       const SquareArgs zy[2] = {product(ts, zs, zf), product(ys, tts, yf)};
       const SquarePassArgs ps[2] = {sym_pass(zf, zs), sym_pass(yf, ys)};
-      if ((e = launch_square(zy, together ? 2 : 1, sms, s)) != cudaSuccess ||
-          (!together && (e = launch_square(zy + 1, 1, sms, s)) != cudaSuccess) ||
+      if ((e = launch_square(zy, full ? 2 : 1, sms, s)) != cudaSuccess ||
+          (!full && ((e = launch_split_transpose(ts, tts, stop, s)) != cudaSuccess ||
+                     (e = launch_square(zy + 1, 1, sms, s)) != cudaSuccess)) ||
           (e = launch_square_pass(ps, 2, K, stop, s)) != cudaSuccess)
         return e;
     }

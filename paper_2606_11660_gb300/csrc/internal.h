@@ -270,10 +270,14 @@ cudaError_t launch_row_scales(const float* x, int n, int K, int64_t ld, int unit
 cudaError_t launch_aggregate(const float* rows, int64_t n, int K, int64_t ld,
                              const int64_t* offsets, int G, int mode, const float* scale,
                              float* out, int64_t ld_out, cudaStream_t s);
+// Workspaces: what the queries report, and the least the calls take (the fit then
+// goes over the rows in parts, the power's products one at a time).
 size_t fisher_fit_workspace(int64_t n, int64_t K);
+size_t fisher_fit_least(int64_t n, int64_t K);
 cudaError_t launch_fisher_fit(const float* x, int n, int K, int64_t ldx, float* r, int64_t ldr,
-                              float* ws, int* status, int sms, cudaStream_t s);
+                              void* ws, size_t ws_bytes, int* status, int sms, cudaStream_t s);
 size_t fisher_power_workspace(int64_t K);
+size_t fisher_power_least(int64_t K);
 // At most `iterations` Newton-Schulz updates.  With residuals != nullptr or
 // tol > 0 the residual ||I - Z Y||_F / sqrt(K) of every iterate is read back
 // (the stream is synchronised every few iterates) into residuals[0 ..] and the
@@ -282,7 +286,7 @@ size_t fisher_power_workspace(int64_t K);
 cudaError_t launch_fisher_power(const float* r1, const float* r2, int K, int64_t ldr, float lam,
                                 float damping, int inverse, int iterations, float tol,
                                 float* residuals, int* iterations_done, float* m, int64_t ldm,
-                                float* ws, int* status, int sms, cudaStream_t s);
+                                void* ws, size_t ws_bytes, int* status, int sms, cudaStream_t s);
 
 // Square fp32-accurate products (square.cu).  An operand of `rows` rows of K
 // entries, split into three bf16 planes (`rows` rows each, leading dimension ld, a
@@ -300,9 +304,10 @@ struct SquareArgs {
   float alpha = 1.0f;
   const float* alpha_s = nullptr;  // alpha' = alpha * (*alpha_s) when given
   float gamma = 0.0f;
+  bool accumulate = false;         // C += the product (with c)
   float* c = nullptr;              // [x.rows, ldc], or nullptr: C goes to the splits of its rows
-  int64_t ldc = 0;                 //   and columns (x.rows and y.rows multiples of 4)
-  SplitOperand row_out, col_out;
+  int64_t ldc = 0;                 //   and, where col_out has planes, columns (x.rows and y.rows
+  SplitOperand row_out, col_out;   //   multiples of 4)
   const int* stop = nullptr;       // device flag: nonzero = compute and write nothing
   float* part = nullptr;           // square_part_floats() sums of (C - I)^2, or nullptr
   int* status = nullptr;
@@ -320,6 +325,9 @@ struct SquarePassArgs {
 };
 cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int* stop,
                                cudaStream_t s);
+// The split of a K x K matrix's columns from that of its rows.
+cudaError_t launch_split_transpose(const SplitOperand& from, const SplitOperand& to,
+                                   const int* stop, cudaStream_t s);
 // m = (c + c^T) / 2 * (*scale)
 cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,
                                    int64_t ldm, cudaStream_t s);

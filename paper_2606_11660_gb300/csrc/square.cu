@@ -69,6 +69,7 @@ struct SqParams {
   int n_mt, n_nt;            // tiles
   int n_tiles;               // of one product
   int symmetric;             // x == y: tiles with some b <= q, mirrored into C[q, b]
+  int accumulate;            // the product is added to C
   float alpha;
   const float* alpha_s;      // or nullptr
   float gamma;               // added on the diagonal
@@ -153,7 +154,7 @@ __device__ __forceinline__ void put_splits(const SqParams& p, const float* tile,
       const float* v = tile + j * 33 + l4;
       put_four(p.row, bc + j, q0 + l4, make_float4(v[0], v[1], v[2], v[3]));
     }
-    if (j < nq && l4 < nb) {                       // column q0 + j of C, rows bc + l4, ..
+    if (p.col.planes != nullptr && j < nq && l4 < nb) {   // column q0 + j of C, rows bc + l4, ..
       const float* v = tile + l4 * 33 + j;
       put_four(p.col, q0 + j, bc + l4, make_float4(v[0], v[33], v[66], v[99]));
     }
@@ -384,6 +385,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSqThreads, 1)
           float v = al * tile[j * 33 + lane];
           if (b == q) v += p.gamma;
           const bool in = qin && j < nb;
+          if (p.accumulate && in && (!p.symmetric || b <= q)) v += *dst;
           if (in && out != nullptr && (!p.symmetric || b <= q)) *dst = v;
           tile[j * 33 + lane] = in ? v : 0.0f;
           const float r = in ? v - (b == q ? 1.0f : 0.0f) : 0.0f;
@@ -505,6 +507,37 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// to = the split of from's columns: its planes transposed (both K x K).  64 x 64
+// tiles through shared memory, 16 bytes an access; columns past K lie within ld.
+__global__ void __launch_bounds__(256) split_transpose_kernel(const SplitOperand from,
+                                                              const SplitOperand to,
+                                                              const int* stop) {
+  __shared__ __align__(16) __nv_bfloat16 tile[kPassTile][kPassTile + 8];
+  griddep_launch_dependents();
+  griddep_wait();
+  if (stop != nullptr && *stop != 0) return;
+  const int64_t plane = static_cast<int64_t>(blockIdx.z) * from.rows * from.ld;
+  const int i0 = blockIdx.y * kPassTile, j0 = blockIdx.x * kPassTile;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = (threadIdx.x >> 3) + 32 * u, c = 8 * (threadIdx.x & 7);
+    if (i0 + r < from.rows && j0 + c < from.K)
+      *reinterpret_cast<uint4*>(&tile[r][c]) = *reinterpret_cast<const uint4*>(
+          from.planes + plane + static_cast<int64_t>(i0 + r) * from.ld + j0 + c);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = (threadIdx.x >> 3) + 32 * u, c = 8 * (threadIdx.x & 7);
+    if (j0 + r >= to.rows || i0 + c >= to.K) continue;
+    __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) v[x] = tile[c + x][r];
+    *reinterpret_cast<uint4*>(to.planes + plane + static_cast<int64_t>(j0 + r) * to.ld + i0 + c) =
+        *reinterpret_cast<const uint4*>(v);
+  }
+}
+
 // m = (c + c^T) / 2 * (*scale)
 __global__ void __launch_bounds__(256) symmetric_scale_kernel(const float* c, int K, int64_t ldc,
                                                               const float* scale, float* m,
@@ -610,6 +643,7 @@ cudaError_t launch_square(const SquareArgs* a, int n, int sms, cudaStream_t s) {
   p.K = a->y.K;
   p.chains = p.K <= kShortChainK ? 2 : 1;
   p.symmetric = a->symmetric ? 1 : 0;
+  p.accumulate = a->accumulate ? 1 : 0;
   for (int i = 0; i < n; ++i) p.c[i] = a[i].c;
   p.alpha = a->alpha;
   p.alpha_s = a->alpha_s;
@@ -640,6 +674,13 @@ cudaError_t launch_square_pass(const SquarePassArgs* a, int n, int K, const int*
   }
   const int t = (K + kPassTile - 1) / kPassTile;
   return launch_dependent(square_pass_kernel, dim3(t * (t + 1) / 2, n), dim3(256), 0, s, pp);
+}
+
+cudaError_t launch_split_transpose(const SplitOperand& from, const SplitOperand& to,
+                                   const int* stop, cudaStream_t s) {
+  const int t = (from.K + kPassTile - 1) / kPassTile;
+  return launch_dependent(split_transpose_kernel, dim3(t, t, kPlanes), dim3(256), 0, s, from, to,
+                          stop);
 }
 
 cudaError_t launch_symmetric_scale(const float* c, int K, int64_t ldc, const float* scale, float* m,

@@ -136,3 +136,44 @@ def test_power_that_starts_converged(power):
     assert done == 0 and len(res) == 1 and abs(res[0] - 0.5) < 1e-6
     want = 2.0 ** (-0.5 if power == bg.BERGSON_FISHER_INV_SQRT else -1.0)
     np.testing.assert_allclose(np32(M), np.eye(4) * want, rtol=1e-6)
+
+
+def _r256(n):
+    return -(-n // 256) * 256
+
+
+def _fp16_sizes(n, K):
+    """The workspaces of fit and power with operands in two fp16 planes and a scale per row."""
+    split = lambda rows, cols: _r256(4 * rows * (-(-cols // 8) * 8)) + _r256(4 * rows)
+    part = max(K, (-(-K // 64)) ** 2, 16 * -(-K // 256) * -(-K // 128))
+    return (split(K, n) + _r256(4 * K),
+            2 * _r256(4 * K * K) + 4 * split(K, K) + _r256(36 * K) + _r256(4 * part) + 512)
+
+
+@pytest.mark.parametrize("n,K", [(9, 128), (70, 132), (300, 260), (1025, 516), (513, 1028)])
+def test_smaller_workspaces(n, K):
+    # room for two thirds of the rows: R in two parts; for three splits: the products one by one
+    g = wl.generator(n, "cpu")
+    x = torch.randn((n, K), generator=g) * torch.logspace(-1, 1, K)
+    fit_bytes, power_bytes = _fp16_sizes(n, K)
+    assert fit_bytes < bg.bergson_fisher_fit_workspace(n, K)
+    assert power_bytes < bg.bergson_fisher_preconditioner_workspace(K)
+    R = torch.full((K, K), float("nan"), device=DEV)
+    bg.bergson_fisher_fit(x.to(DEV), n, K, R, bg.workspace_tensor(fit_bytes, DEV)[:fit_bytes])
+    assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+    want = orc.fisher_fit(x.numpy())
+    d = np.sqrt(np.diag(want))
+    err = np.abs(np32(R).astype(np.float64) - want) / np.outer(d, d)
+    assert err.max() <= (2 + 24 + n / 32 + 2) * 2.0 ** -23 and torch.equal(R, R.T)
+    for power in (bg.BERGSON_FISHER_INV_SQRT, bg.BERGSON_FISHER_INV):
+        for tol in (0.0, 1e-3):
+            out = []
+            for size in (bg.bergson_fisher_preconditioner_workspace(K), power_bytes):
+                M = torch.full((K, K), float("nan"), device=DEV)
+                ws = bg.workspace_tensor(size, DEV)[:size]
+                ws.fill_(0x7F)
+                out.append((M, bg.bergson_fisher_preconditioner_tol(R, None, K, 1.0, 0.1, power, 12,
+                                                                    tol, M, ws)))
+                assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+            assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+            assert not torch.isnan(out[0][0]).any()
