@@ -20,7 +20,7 @@
 //
 // Measured (one GB300, n = 1024, 12 updates at K = 3072): 17.4 ms per fit and
 // power with tf32 parts on single CTAs, K slices through partial sums in
-// memory and separate transpose / symmetrise / norm passes; 8.2 ms as here.
+// memory and separate transpose / symmetrise / norm passes; 8.7 ms as here.
 // Per update: 63 / 116 / 1220 us at K = 256 / 1024 / 3072 before, 34 / 66 / 653
 // here.
 
