@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(1024) frob_final_kernel(const float* __restric
   const float t = ordered_sum(part, n_part);
   if (threadIdx.x != 0) return;
   *stop = 0;
-  const float c = sqrtf(t);
+  // a norm that overflows leaves NaN: 1 / c = 0 would make M = 0 of it
+  const float c = isfinite(t) ? sqrtf(t) : __int_as_float(0x7fffffff);
   scal[1] = c;
   scal[2] = 1.0f / c;
   scal[3] = 1.0f / sqrtf(c);

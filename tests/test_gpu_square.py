@@ -177,3 +177,16 @@ def test_smaller_workspaces(n, K):
                 assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
             assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
             assert not torch.isnan(out[0][0]).any()
+
+
+@pytest.mark.parametrize("K", [8, 604, 1284])
+@pytest.mark.parametrize("tol", [0.0, 1e-4])
+def test_a_norm_that_overflows_gives_nan(K, tol):
+    # ||R||_F^2 > 2^128: no scale to iterate from, and not M = 0
+    R = torch.eye(K, device=DEV) * 1e25
+    for power in (bg.BERGSON_FISHER_INV_SQRT, bg.BERGSON_FISHER_INV):
+        M = torch.zeros((K, K), device=DEV)
+        ws = bg.workspace_tensor(bg.bergson_fisher_preconditioner_workspace(K), DEV)
+        done, res = bg.bergson_fisher_preconditioner_tol(R, None, K, 1.0, 0.1, power, 5, tol, M, ws)
+        assert bg.bergson_sync_status() == bg.BERGSON_OK, bg.bergson_last_error()
+        assert torch.isnan(M).all() and done == 5 and np.isnan(res).all()
